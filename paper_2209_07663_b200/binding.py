@@ -3,7 +3,9 @@
 Marshals arguments only: tensors become raw pointers, options become the C
 structs, return codes become exceptions.  Every step of the table's work runs in
 the CUDA library.  There is no fallback: if libmono.so is missing, loading
-raises.
+raises.  The calls that a training or serving loop makes each step go through a
+small CPython extension (csrc/binding_native.cpp) instead of ctypes: on a small
+batch the host is what bounds them.
 """
 from __future__ import annotations
 
@@ -81,11 +83,12 @@ def _struct_dict(s: ctypes.Structure) -> dict:
 
 
 _lib = None
+_native = None          # csrc/binding_native.cpp, bound to the functions of the loaded library
 
 
 def load_library(path: Optional[str] = None):
     """Load libmono.so and declare its prototypes.  Raises if it is not there."""
-    global _lib
+    global _lib, _native
     if _lib is not None and path is None:
         return _lib
     path = path or LIB_PATH
@@ -131,8 +134,29 @@ def load_library(path: Optional[str] = None):
     for name, (res, args) in proto.items():
         fn = getattr(L, name)
         fn.restype, fn.argtypes = res, args
-    _lib = L
+    native = _load_native()
+    native.bind({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in proto}, _ptr)
+    _lib, _native = L, native
     return L
+
+
+def _load_native():
+    import importlib.util
+    path = os.path.join(_PKG, "_binding_native.so")
+    if not os.path.exists(path):
+        raise RuntimeError(f"{path} is missing: build it with `python -m paper_2209_07663_b200.build`")
+    import torch  # noqa: F401  (the extension links against its libraries)
+    spec = importlib.util.spec_from_file_location("_binding_native", path)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    return module
+
+
+def _hot():
+    """The native module, loading the library first if nothing has."""
+    if _native is None:
+        load_library()
+    return _native
 
 
 def error_string(code: int) -> str:
@@ -193,76 +217,74 @@ def mono_reserve(t: int, max_ids: int, max_bags: int) -> None:
 
 
 def mono_lookup_pool(t: int, ids, n_ids: int, slot_offsets, n_bags: int, out) -> None:
-    _check("mono_lookup_pool", load_library().mono_lookup_pool(t, _ptr(ids), n_ids, _ptr(slot_offsets), n_bags,
-                                                               _ptr(out)), t)
+    rc = (_native or _hot()).lookup_pool(t, ids, n_ids, slot_offsets, n_bags, out)
+    if rc:
+        _check("mono_lookup_pool", rc, t)
 
 
 def mono_lookup_pool_noalloc(t: int, ids, n_ids: int, slot_offsets, n_bags: int, out) -> None:
     """mono_lookup_pool for callers that may not allocate device memory: the per-ID scratch
     lives in a fixed array inside the library, so at most MONO_NOALLOC_MAX_IDS IDs per call,
     and calls must not overlap on the GPU."""
-    _check("mono_lookup_pool_noalloc", load_library().mono_lookup_pool_noalloc(t, _ptr(ids), n_ids, _ptr(slot_offsets),
-                                                                               n_bags, _ptr(out)), t)
+    rc = (_native or _hot()).lookup_pool_noalloc(t, ids, n_ids, slot_offsets, n_bags, out)
+    if rc:
+        _check("mono_lookup_pool_noalloc", rc, t)
 
 
 def mono_apply_grads(t: int, ids, n_ids: int, slot_offsets, n_bags: int, grad_pooled, now: int) -> None:
-    _check("mono_apply_grads", load_library().mono_apply_grads(t, _ptr(ids), n_ids, _ptr(slot_offsets), n_bags,
-                                                               _ptr(grad_pooled), now), t)
+    rc = (_native or _hot()).apply_grads(t, ids, n_ids, slot_offsets, n_bags, grad_pooled, now)
+    if rc:
+        _check("mono_apply_grads", rc, t)
 
 
 def mono_expire(t: int, now: int) -> None:
-    _check("mono_expire", load_library().mono_expire(t, now), t)
+    rc = (_native or _hot()).expire(t, now)
+    if rc:
+        _check("mono_expire", rc, t)
 
 
 def mono_group_ahead(t: int, ids, n_ids: int, slot_offsets, n_bags: int) -> None:
-    _check("mono_group_ahead", load_library().mono_group_ahead(t, _ptr(ids), n_ids, _ptr(slot_offsets), n_bags), t)
+    rc = (_native or _hot()).group_ahead(t, ids, n_ids, slot_offsets, n_bags)
+    if rc:
+        _check("mono_group_ahead", rc, t)
 
 
 def mono_prepare_push(t: int, ids, n_ids: int, slot_offsets, n_bags: int) -> None:
-    _check("mono_prepare_push", load_library().mono_prepare_push(t, _ptr(ids), n_ids, _ptr(slot_offsets), n_bags), t)
-
-
-def _group_args(handles, ids, slot_offsets, vectors):
-    """Host arrays of the grouped calls: one entry per table."""
-    n = len(handles)
-    if not (len(ids) == len(slot_offsets) == len(vectors) == n):
-        raise ValueError("grouped calls take one batch per table")
-    ptrs = ctypes.c_void_p * n
-    i64s = ctypes.c_int64 * n
-    return (n, ptrs(*handles), ptrs(*[_ptr(x) for x in ids]), i64s(*[x.numel() for x in ids]),
-            ptrs(*[_ptr(x) for x in slot_offsets]), i64s(*[x.numel() - 1 for x in slot_offsets]),
-            ptrs(*[_ptr(x) for x in vectors]))
+    rc = (_native or _hot()).prepare_push(t, ids, n_ids, slot_offsets, n_bags)
+    if rc:
+        _check("mono_prepare_push", rc, t)
 
 
 def mono_group_prepare_push(handles, ids, slot_offsets, group_stream: int = 0) -> None:
     """Announce every table's next batch (lists of device tensors, one per table)."""
-    n, tp, ip, nip, op, nbp, _ = _group_args(handles, ids, slot_offsets, ids)
-    code = load_library().mono_group_prepare_push(n, tp, ip, nip, op, nbp, group_stream or None)
-    if code != 0:
-        raise MonoError("mono_group_prepare_push", code)
+    rc = (_native or _hot()).group_prepare_push(handles, ids, slot_offsets, group_stream)
+    if rc:
+        raise MonoError("mono_group_prepare_push", rc)
 
 
 def mono_group_lookup_pool(handles, ids, slot_offsets, outs, group_stream: int = 0) -> None:
     """ids / slot_offsets / outs: lists of device tensors, one per table."""
-    n, tp, ip, nip, op, nbp, vp_ = _group_args(handles, ids, slot_offsets, outs)
-    code = load_library().mono_group_lookup_pool(n, tp, ip, nip, op, nbp, vp_, group_stream or None)
-    if code != 0:
-        raise MonoError("mono_group_lookup_pool", code)
+    rc = (_native or _hot()).group_lookup_pool(handles, ids, slot_offsets, outs, group_stream)
+    if rc:
+        raise MonoError("mono_group_lookup_pool", rc)
 
 
 def mono_group_apply_grads(handles, ids, slot_offsets, grads, now: int, group_stream: int = 0) -> None:
-    n, tp, ip, nip, op, nbp, vp_ = _group_args(handles, ids, slot_offsets, grads)
-    code = load_library().mono_group_apply_grads(n, tp, ip, nip, op, nbp, vp_, now, group_stream or None)
-    if code != 0:
-        raise MonoError("mono_group_apply_grads", code)
+    rc = (_native or _hot()).group_apply_grads(handles, ids, slot_offsets, grads, now, group_stream)
+    if rc:
+        raise MonoError("mono_group_apply_grads", rc)
 
 
 def mono_expire_slice(t: int, now: int, slice_index: int, n_slices: int) -> None:
-    _check("mono_expire_slice", load_library().mono_expire_slice(t, now, slice_index, n_slices), t)
+    rc = (_native or _hot()).expire_slice(t, now, slice_index, n_slices)
+    if rc:
+        _check("mono_expire_slice", rc, t)
 
 
 def mono_fence(t: int) -> None:
-    _check("mono_fence", load_library().mono_fence(t), t)
+    rc = (_native or _hot()).fence(t)
+    if rc:
+        _check("mono_fence", rc, t)
 
 
 def mono_snapshot_save(t: int) -> None:
@@ -278,13 +300,15 @@ def mono_snapshot_drop(t: int) -> None:
 
 
 def mono_lookup_pool_host(t: int, ids, n_ids: int, slot_offsets, n_bags: int, out) -> None:
-    _check("mono_lookup_pool_host", load_library().mono_lookup_pool_host(t, _ptr(ids), n_ids, _ptr(slot_offsets),
-                                                                         n_bags, _ptr(out)), t)
+    rc = (_native or _hot()).lookup_pool_host(t, ids, n_ids, slot_offsets, n_bags, out)
+    if rc:
+        _check("mono_lookup_pool_host", rc, t)
 
 
 def mono_apply_grads_host(t: int, ids, n_ids: int, slot_offsets, n_bags: int, grad_pooled, now: int) -> None:
-    _check("mono_apply_grads_host", load_library().mono_apply_grads_host(t, _ptr(ids), n_ids, _ptr(slot_offsets),
-                                                                         n_bags, _ptr(grad_pooled), now), t)
+    rc = (_native or _hot()).apply_grads_host(t, ids, n_ids, slot_offsets, n_bags, grad_pooled, now)
+    if rc:
+        _check("mono_apply_grads_host", rc, t)
 
 
 def mono_status(t: int) -> dict:
@@ -369,6 +393,7 @@ class MonoTable:
         self.dim, self.capacity = int(dim), int(capacity)
         self.threshold = max(int(filter_threshold), 1)
         opt.setdefault("stream", torch.cuda.current_stream().cuda_stream)
+        self._device = torch.cuda.current_device()
         self.handle = mono_table_create(capacity, dim, filter_threshold, ttl, **opt)
 
     def close(self):
@@ -394,9 +419,18 @@ class MonoTable:
             x = torch.from_numpy(a)
         if x.dtype == torch.uint64:
             x = x.view(torch.int64)
+        if x.dtype == dtype and x.is_cuda and x.get_device() == self._device and x.is_contiguous():
+            return x
         return x.to(device="cuda", dtype=dtype).contiguous()
 
     def lookup_pool(self, ids, offsets, out=None):
+        if out is not None:
+            # tensors that are where and what the call needs go straight to it (None: they are not)
+            rc = _native.table_pull(self.handle, self._device, ids, offsets, out)
+            if rc is not None:
+                if rc:
+                    _check("mono_lookup_pool", rc, self.handle)
+                return out
         torch = self._torch
         ids, offsets = self._dev(ids, torch.int64), self._dev(offsets, torch.int64)
         n_bags = offsets.numel() - 1

@@ -1,10 +1,12 @@
-"""Build the CUDA shared library (libmono.so) in-tree for sm_100a with nvcc."""
+"""Build the CUDA shared library (libmono.so) in-tree for sm_100a with nvcc, and the small CPython
+extension that hands tensors to it."""
 from __future__ import annotations
 
 import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
@@ -12,6 +14,9 @@ LIB = os.path.join(PKG, "libmono.so")
 # the same sources with -DMONO_DEBUG: every index the library computes for itself is range-checked
 # on the device and a bad one reported through the status bits (binding: MONO_LIBRARY=checked)
 LIB_CHECKED = os.path.join(PKG, "libmono_checked.so")
+# the hot calls' Python side (csrc/binding_native.cpp); touches no table and needs no nvcc
+NATIVE = os.path.join(PKG, "_binding_native.so")
+NATIVE_SOURCE = os.path.join(CSRC, "binding_native.cpp")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "--cudart", "static", "-ldl"]
@@ -22,7 +27,7 @@ def _sources():
 
 
 def _newest_input() -> float:
-    files = glob.glob(os.path.join(CSRC, "*")) + [os.path.join(PKG, "..", "include", "mono.h")]
+    files = glob.glob(os.path.join(CSRC, "*.cu*")) + [os.path.join(PKG, "..", "include", "mono.h")]
     return max(os.path.getmtime(f) for f in files)
 
 
@@ -33,9 +38,27 @@ def find_nvcc() -> str:
     return nvcc
 
 
+def build_native(force: bool = False) -> str:
+    """Compile csrc/binding_native.cpp against the torch that is installed, unless it is up to date."""
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= os.path.getmtime(NATIVE_SOURCE):
+        return NATIVE
+    import torch
+    from torch.utils import cpp_extension
+    tmp = f"{NATIVE}.{os.getpid()}.tmp"
+    lib_dir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-shared", "-fPIC",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           *[f"-isystem{d}" for d in cpp_extension.include_paths()], f"-I{sysconfig.get_paths()['include']}",
+           NATIVE_SOURCE, "-o", tmp, f"-L{lib_dir}", "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
     """Compile csrc/*.cu into libmono.so (or, with `checked`, into libmono_checked.so) unless it is
-    already up to date."""
+    already up to date.  The Python side of the hot calls comes with it."""
+    build_native(force=force and not checked)
     lib = LIB_CHECKED if checked else LIB
     if not force and os.path.exists(lib) and os.path.getmtime(lib) >= _newest_input():
         return lib
