@@ -6,8 +6,8 @@
 //
 // Three cases, by how often the ID occurs in the batch:
 // Every repeated ID has a segment of bag_of_sorted[] that lists the bags of its
-// occurrences (filed by file_segments_kernel: inside the lookup when the batch was
-// announced, else inside the push).
+// occurrences (filed by the pull, gather_pool_kernel, when the batch was announced, else by
+// file_segments_kernel inside the push).
 //  - once (most distinct IDs of a long-tailed batch): its gradient is the
 //    pooled gradient of its one bag, so update_singletons_kernel updates the
 //    row straight from that bag's gradient row;
@@ -20,6 +20,7 @@
 #pragma once
 
 #include "kernels_dedup.cuh"
+#include "kernels_forward.cuh"
 
 namespace mono {
 
@@ -126,31 +127,16 @@ __device__ inline void reduce_segment(const Work& wk, const float* __restrict__ 
   }
 }
 
-// One pass over the occurrences once the distinct IDs have been looked up: every
-// occurrence of a repeated ID reads its ID's slot of the per-call set and is filed under
-// its ID -- its bag goes into the ID's segment of bag_of_sorted[], at the occurrence's rank -- and, when
-// occ_row is given (the lookup of a batch that was announced), leaves there the row its ID
-// owns, or the table's all-zero row, for the pooling kernel.
-__device__ inline void file_segments_body(const Work& wk, long long n_ids, long long n_bags, uint32_t* __restrict__ occ_row,
-                                          uint32_t zero_row, uint32_t vblock, uint32_t vgrid) {
+// The filing pass of a push whose batch was not announced, or not pulled since (otherwise the pull
+// has filed the bags, FiledRows): one pass over the occurrences.
+__device__ inline void file_segments_body(const Work& wk, long long n_ids, long long n_bags, uint32_t vblock, uint32_t vgrid) {
   const long long stride = (long long)vgrid * blockDim.x;
-  for (long long j = (long long)vblock * blockDim.x + threadIdx.x; j < n_ids; j += stride) {
-    const uint2 o = wk.occ[j];
-    uint32_t row = zero_row;
-    if (o.x != kNoSlot && MONO_INDEX_OK(wk.error_bits, o.x, wk.n_slots)) {
-      const uint4 bs = __ldg(reinterpret_cast<const uint4*>(wk.bset + o.x));     // key (x, y), segment start, row
-      if (bs.w != kNoRow) row = bs.w;
-      if (bs.z != kNoSegment) {                                                   // (an ID that occurs once has no segment)
-        const uint32_t bag = wk.occ_bag[j];
-        if (bag < n_bags && MONO_INDEX_OK(wk.error_bits, (unsigned long long)bs.z + o.y, wk.max_ids)) wk.bag_of_sorted[bs.z + o.y] = bag;
-      }
-    }
-    if (occ_row) occ_row[j] = row;
-  }
+  const FiledRows rows{wk, n_bags, 0u};
+  for (long long j = (long long)vblock * blockDim.x + threadIdx.x; j < n_ids; j += stride) (void)rows.file(j);
 }
 __global__ void __launch_bounds__(256)
-file_segments_kernel(Work wk, long long n_ids, long long n_bags, uint32_t* __restrict__ occ_row, uint32_t zero_row) { after_previous_kernel();
-  file_segments_body(wk, n_ids, n_bags, occ_row, zero_row, blockIdx.x, gridDim.x);
+file_segments_kernel(Work wk, long long n_ids, long long n_bags) { after_previous_kernel();
+  file_segments_body(wk, n_ids, n_bags, blockIdx.x, gridDim.x);
 }
 
 // The IDs that occur once in the batch (most distinct IDs of a long-tailed batch): the

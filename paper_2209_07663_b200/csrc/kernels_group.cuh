@@ -21,13 +21,15 @@ struct GroupItem {
   const long long* off;
   long long n_ids, n_bags;
   float* out;                    // lookup
-  uint32_t* occ_row;             // lookup: row of every occurrence
+  uint32_t* occ_row;             // lookup: where a tile's rows go that do not fit its block's shared memory
   const float* grad;             // push
   unsigned long long dedup_seed;
   uint32_t now;
   uint32_t prepared;             // lookup: 1 = rows from the per-call set (the batch was announced), 0 = from the key store
   uint32_t lane_class;           // 0..3: lane groups of 4 / 8 / 16 / 32 with one column vector per lane;
                                  // 4..6: 32 lanes with 2 / 4 / 8 vectors per lane
+  uint32_t pool_wide;            // lookup: 32-byte accesses (classes 4..6 only)
+  uint32_t tile_bags;            // lookup: bags per block
   uint32_t active;               // 0: the table takes no part in this call (empty batch)
 };
 
@@ -82,18 +84,11 @@ group_table_insert_kernel(const GroupItem* __restrict__ items, const uint32_t* _
   table_insert_body(it.tv, it.wk, it.now, vblock, vgrid);
 }
 
-// the filing pass inside a push ...
+// (of a push whose batch was not pulled since it was announced, or not announced)
 __global__ void __launch_bounds__(256)
 group_file_segments_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
-  file_segments_body(it.wk, it.n_ids, it.n_bags, nullptr, 0u, vblock, vgrid);
-}
-
-// ... and inside the lookup of announced batches, where it also leaves every occurrence's row
-__global__ void __launch_bounds__(256)
-group_file_rows_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  if (it.prepared) file_segments_body(it.wk, it.n_ids, it.n_bags, it.occ_row, (uint32_t)it.tv.capacity, vblock, vgrid);
+  file_segments_body(it.wk, it.n_ids, it.n_bags, vblock, vgrid);
 }
 
 __global__ void __launch_bounds__(256)
@@ -157,20 +152,35 @@ __device__ inline void by_lane_class(uint32_t lane_class, F&& f) {
   }
 }
 
-// (lookup of the tables whose batches were not announced: their occurrences probe the key store)
-__global__ void __launch_bounds__(256)
-group_probe_rows_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  if (!it.prepared) probe_rows_body(it.tv, it.ids, it.n_ids, it.occ_row, vblock, vgrid);
-}
+// The rows of a table of the group, whose batch may have been announced or not.
+struct AnyRows {
+  const GroupItem& it;
+  __device__ __forceinline__ void resolve(long long first, uint32_t n, uint32_t* dst) const {
+    if (it.prepared) FiledRows{it.wk, it.n_bags, (uint32_t)it.tv.capacity}.resolve(first, n, dst);
+    else ProbedRows<1>{it.tv, it.ids, it.tv.st->stash_hw}.resolve(first, n, dst);
+  }
+};
 
 template <int WIDE>
-__global__ void __launch_bounds__(256)
-group_gather_pool_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
+__global__ void __launch_bounds__(kPoolThreads, WIDE ? 4 : 6)
+group_pool_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
-  by_lane_class<WIDE>(it.lane_class, [&](auto g, auto nv) {
-    gather_pool_body<decltype(g)::value, decltype(nv)::value>(it.tv, it.occ_row, it.n_ids, it.off, it.n_bags, it.out, vblock, vgrid);
-  });
+  const auto pool = [&](auto g, auto nv, auto vw) {
+    pool_tile_body<decltype(g)::value, decltype(nv)::value, decltype(vw)::value>(it.tv, AnyRows{it}, it.occ_row, it.n_ids, it.off, it.n_bags, it.out,
+                                                                                 it.tile_bags, vblock);
+  };
+  if (WIDE && it.pool_wide) {
+    using W = std::integral_constant<int, 32>;
+    using V8 = std::integral_constant<int, 8>;
+    switch (it.lane_class) {
+      case 4: pool(W{}, std::integral_constant<int, 1>{}, V8{}); break;
+      case 5: pool(W{}, std::integral_constant<int, 2>{}, V8{}); break;
+      case 6: pool(W{}, std::integral_constant<int, 4>{}, V8{}); break;
+      default: break;
+    }
+    return;
+  }
+  by_lane_class<WIDE>(it.lane_class, [&](auto g, auto nv) { pool(g, nv, std::integral_constant<int, 4>{}); });
 }
 
 template <int WIDE>

@@ -31,13 +31,13 @@ using namespace mono;
 static __device__ __align__(256) uint32_t g_noalloc_occ_row[MONO_NOALLOC_MAX_IDS];
 
 enum KernelId {
-  K_PROBE, K_GATHER, K_FILL_BAG, K_DEDUP, K_LOOKUP, K_UPDATE, K_SKETCH, K_INSERT, K_EXPAND, K_ORDER, K_FILE, K_SINGLES, K_REDUCE, K_FOLD, K_COMBINE, K_FINISH, K_EXPIRE,
+  K_POOL, K_FILL_BAG, K_DEDUP, K_LOOKUP, K_UPDATE, K_SKETCH, K_INSERT, K_EXPAND, K_ORDER, K_FILE, K_SINGLES, K_REDUCE, K_FOLD, K_COMBINE, K_FINISH, K_EXPIRE,
   K_STASH_TRIM, K_CLEAR, K_REDUCE_PARTS, K_ADOPT, K_COUNT
 };
-// (table_lookup and table_update are the two halves of table_update_kernel; a push that was not
+// (gather_pool: either of the two pooling kernels; table_lookup and table_update are the two halves of table_update_kernel; a push that was not
 // announced runs both in one launch, counted as table_update)
 static const char* const kKernelNames[K_COUNT] = {
-  "probe_rows", "gather_pool", "fill_occ_bag", "dedup_tile", "table_lookup", "table_update", "sketch_add", "table_insert", "expand_parts", "order_parts",
+  "gather_pool", "fill_occ_bag", "dedup_tile", "table_lookup", "table_update", "sketch_add", "table_insert", "expand_parts", "order_parts",
   "file_segments", "update_singletons", "reduce_adagrad", "fold_partials", "combine_adagrad",
   "finish_apply", "expire", "stash_trim", "clear_set", "reduce_parts", "adopt_group"
 };
@@ -316,46 +316,59 @@ int dispatch_dim(uint32_t dim, F&& f) {
   return f(std::integral_constant<int, 32>{}, std::integral_constant<int, 8>{});
 }
 
-// The pooling kernel over the row indices in `occ_row`.
-int launch_gather(mono_table* t, const uint32_t* occ_row, int64_t n_ids, const long long* off, int64_t n_bags, float* out) {
-  return dispatch_dim(t->tv.dim, [&](auto g, auto nv) -> int {
-    constexpr int G = decltype(g)::value, NV = decltype(nv)::value;
-    const int64_t groups_per_block = 256 / G;
-    int64_t blocks = (n_bags + groups_per_block - 1) / groups_per_block;
-    // (two waves of blocks: measured 0.8 % of a step faster on the largest configuration than eight, and 3.5 %
-    // faster than one block per 16 bags, although the kernel alone takes the same time)
-    const int64_t cap = (int64_t)grid_for(t, 8) * 2;
-    if (blocks > cap) blocks = cap;
-    LAUNCH(t, K_GATHER, launch_after(gather_pool_kernel<G, NV>, (int)blocks, 256, t->stream, t->tv, occ_row, n_ids, off, n_bags, out));
+// ... and for the pooling kernels: rows of more than 128 columns that are multiples of 32 bytes, going to
+// an output that is aligned likewise, move 32 bytes per lane, so that half as many accesses fill more of a
+// warp's lanes (narrower rows measured no faster that way, and long bags slower).
+bool pools_wide(uint32_t dim, const float* out) { return dim > 128 && dim % 8 == 0 && aligned(out, 32); }
+
+template <typename F>
+int dispatch_pool(uint32_t dim, const float* out, F&& f) {
+  using V4 = std::integral_constant<int, 4>;
+  using V8 = std::integral_constant<int, 8>;
+  if (!pools_wide(dim, out)) return dispatch_dim(dim, [&](auto g, auto nv) -> int { return f(g, nv, V4{}); });
+  if (dim <= 256) return f(std::integral_constant<int, 32>{}, std::integral_constant<int, 1>{}, V8{});
+  if (dim <= 512) return f(std::integral_constant<int, 32>{}, std::integral_constant<int, 2>{}, V8{});
+  return f(std::integral_constant<int, 32>{}, std::integral_constant<int, 4>{}, V8{});
+}
+
+// Bags per block of the pooling kernels for a batch that may fill `slots` resident blocks.  As many as leave the
+// tile's IDs within the shared memory (850 of 1024 on average: larger tiles repay a block's fixed latencies, and one
+// that overflows takes its rows through memory), at least one per lane group of the block, and then no more than
+// spreads the batch over whole waves of blocks; at least eight, below which a block is all latency.
+uint32_t pool_tile(int64_t n_ids, int64_t n_bags, int64_t slots, int groups) {
+  if (n_bags <= 0) return 8;
+  const double per_bag = n_ids > n_bags ? (double)n_ids / (double)n_bags : 1.0;
+  int64_t most = (int64_t)(850.0 / per_bag);
+  if (most < groups) most = groups;
+  if (most > kPoolBags) most = kPoolBags;
+  if (slots < 1) slots = 1;
+  const int64_t waves = (n_bags + slots * most - 1) / (slots * most);
+  const int64_t tile = (n_bags + slots * waves - 1) / (slots * waves);
+  return (uint32_t)(tile < 8 ? 8 : tile);
+}
+
+// The pull: one kernel, which takes the rows from the key store, or, for a batch that was announced
+// (`filed`), from the per-call set, filing the bags for the push on the way.
+int launch_pool(mono_table* t, const unsigned long long* ids, uint32_t* spill, int64_t n_ids, const long long* off, int64_t n_bags,
+                float* out, bool filed) {
+  return dispatch_pool(t->tv.dim, out, [&](auto g, auto nv, auto vw) -> int {
+    constexpr int G = decltype(g)::value, NV = decltype(nv)::value, VW = decltype(vw)::value;
+    const uint32_t tile = pool_tile(n_ids, n_bags, grid_for(t, pool_blocks_per_sm<G, NV, VW>()), kPoolThreads / G);
+    const unsigned blocks = (unsigned)((n_bags + tile - 1) / tile);
+    if (filed) LAUNCH(t, K_POOL, launch_after(gather_pool_kernel<G, NV, VW>, blocks, kPoolThreads, t->stream, t->tv, t->wk, spill, n_ids, off, n_bags, out, tile));
+    else LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
     CUDA_TRY(t, cudaGetLastError());
     return (int)MONO_OK;
   });
 }
 
-int launch_probe(mono_table* t, const unsigned long long* ids, int64_t n_ids, uint32_t* occ_row) {
-  if (n_ids <= 0) return MONO_OK;
-  int64_t blocks = (n_ids + 255) / 256;
-  const int64_t cap = (int64_t)grid_for(t, 8) * 8;
-  if (blocks > cap) blocks = cap;
-  LAUNCH(t, K_PROBE, launch_after(probe_rows_kernel, (int)blocks, 256, t->stream, t->tv, ids, n_ids, occ_row));
-  CUDA_TRY(t, cudaGetLastError());
-  return MONO_OK;
-}
-
 int launch_lookup(mono_table* t, const unsigned long long* ids, int64_t n_ids, const long long* off,
                   int64_t n_bags, float* out, bool prepared) {
   if (n_bags == 0) return MONO_OK;
-  if (prepared && n_ids > 0) {
-    // every distinct ID of this batch was looked up when it was announced: one pass over the
-    // occurrences takes the rows from the per-call set and files the bags for the push
-    LAUNCH(t, K_FILE, launch_after(file_segments_kernel, grid_for(t, 8), 256, t->stream, t->wk, n_ids, n_bags, t->occ_row,
-                                                                                  (uint32_t)t->tv.capacity));
-    t->prep.filed = true;
-  } else {
-    const int rc = launch_probe(t, ids, n_ids, t->occ_row);
-    if (rc != MONO_OK) return rc;
-  }
-  return launch_gather(t, t->occ_row, n_ids, off, n_bags, out);
+  const bool filed = prepared && n_ids > 0;
+  const int rc = launch_pool(t, ids, t->occ_row, n_ids, off, n_bags, out, filed);
+  if (rc == MONO_OK && filed) t->prep.filed = true;
+  return rc;
 }
 
 // The part of a push that depends on the IDs alone: bag of every occurrence, and the
@@ -412,14 +425,14 @@ int launch_apply(mono_table* t, const unsigned long long* ids, int64_t n_ids, co
   if (is_prepared_batch(t, ids, n_ids, off, n_bags)) {
     // grouped and looked up already; filed too, if its lookup has run
     t->prep.valid = false;
-    if (!t->prep.filed) LAUNCH(t, K_FILE, launch_after(file_segments_kernel, g8, 256, s, wk, n_ids, n_bags, nullptr, 0u));
+    if (!t->prep.filed) LAUNCH(t, K_FILE, launch_after(file_segments_kernel, g8, 256, s, wk, n_ids, n_bags));
     LAUNCH(t, K_UPDATE, launch_after(table_update_kernel<kCommit>, g8 * 4, 256, s, tv, wk, now));
   } else {
     if ((rc0 = discard_prepared(t)) != MONO_OK) return rc0;
     if (n_ids == 0 || n_bags == 0) return MONO_OK;
     if ((rc0 = launch_group(t, s, ids, n_ids, off, n_bags)) != MONO_OK) return rc0;
     LAUNCH(t, K_UPDATE, launch_after(table_update_kernel<kLookUp | kCommit>, g8 * 4, 256, s, tv, wk, now));
-    LAUNCH(t, K_FILE, launch_after(file_segments_kernel, g8, 256, s, wk, n_ids, n_bags, nullptr, 0u));
+    LAUNCH(t, K_FILE, launch_after(file_segments_kernel, g8, 256, s, wk, n_ids, n_bags));
   }
   // The long segments (the few hottest IDs) are reduced on a stream of their own -- expand,
   // order, the parts, fold, combine, one after the other with no event in between -- beside
@@ -486,7 +499,7 @@ int check_now(mono_table* t, int64_t now) {
 // ---- grouped calls: one launch over several tables -------------------------------------------
 
 enum GroupKernel {
-  GK_FILL, GK_DEDUP, GK_UPDATE, GK_INSERT, GK_FILE, GK_EXPAND, GK_ORDER, GK_GATHER, GK_GATHER_WIDE, GK_REDUCE, GK_REDUCE_WIDE,
+  GK_FILL, GK_DEDUP, GK_UPDATE, GK_INSERT, GK_FILE, GK_EXPAND, GK_ORDER, GK_POOL, GK_POOL_WIDE, GK_REDUCE, GK_REDUCE_WIDE,
   GK_SINGLES, GK_SINGLES_WIDE, GK_FOLD, GK_COMBINE, GK_CLEAR, GK_COUNT
 };
 
@@ -512,7 +525,8 @@ int64_t clamp_blocks(int64_t work, int64_t per_block, int64_t cap) {
 
 // Blocks that table `t` contributes to grouped kernel `k` (the grid it would launch alone, but no
 // larger than its batch needs: a group may hold hundreds of small tables).
-uint32_t group_blocks(const mono_table* t, int k, int64_t n_ids, int64_t n_bags) {
+uint32_t group_blocks(const mono_table* t, int k, const GroupItem& it) {
+  const int64_t n_ids = it.n_ids, n_bags = it.n_bags;
   const int64_t g8 = grid_for(t, 8), g4 = grid_for(t, 4);
   const uint32_t lc = lane_class_of(t->tv.dim);
   const int G = lanes_of_class(lc);
@@ -524,8 +538,8 @@ uint32_t group_blocks(const mono_table* t, int k, int64_t n_ids, int64_t n_bags)
     case GK_INSERT: case GK_FILE: return (uint32_t)clamp_blocks(n_ids, 256, g8);
     case GK_EXPAND: return (uint32_t)clamp_blocks(n_ids / kSegChunk + 1, 1, g8 * 4);
     case GK_ORDER: return (uint32_t)clamp_blocks(n_ids / kSegChunk + 1, kWindows, 64);
-    case GK_GATHER: return wide ? 0u : (uint32_t)clamp_blocks(n_bags, 256 / G, g8 * 8);
-    case GK_GATHER_WIDE: return wide ? (uint32_t)clamp_blocks(n_bags, 256 / G, g8 * 8) : 0u;
+    case GK_POOL: return wide ? 0u : (uint32_t)((n_bags + it.tile_bags - 1) / it.tile_bags);
+    case GK_POOL_WIDE: return wide ? (uint32_t)((n_bags + it.tile_bags - 1) / it.tile_bags) : 0u;
     case GK_REDUCE: return wide ? 0u : (uint32_t)clamp_blocks(n_ids / 2 + 1, 128 / G, g8 * 8);
     case GK_REDUCE_WIDE: return wide ? (uint32_t)clamp_blocks(n_ids / 2 + 1, 128 / G, g8 * 8) : 0u;
     case GK_SINGLES: return wide ? 0u : (uint32_t)clamp_blocks(n_ids, 128, g8 * 8);
@@ -605,6 +619,8 @@ void group_describe(GroupPlan& p, int32_t i, mono_table* t, const uint64_t* ids,
   it.dedup_seed = t->tv.seed0 ^ 0xA5A5A5A55A5A5A5Aull;
   it.prepared = prepared ? 1u : 0u;
   it.lane_class = lane_class_of(t->tv.dim);
+  it.pool_wide = pools_wide(t->tv.dim, out) ? 1u : 0u;
+  it.tile_bags = 8u;
   it.active = (n_ids > 0 && n_bags > 0) ? 1u : 0u;
   if (it.lane_class >= 4) p.any_wide = true; else p.any_narrow = true;
   if (t->tv.sketch_depth) p.any_sketch = true;
@@ -617,7 +633,7 @@ int group_upload(GroupPlan& p, mono_table* const* tables) {
     uint64_t total = 0;
     for (int32_t i = 0; i < p.n; ++i) {
       st[i] = (uint32_t)total;
-      if (p.items[i].active) total += group_blocks(tables[i], k, p.items[i].n_ids, p.items[i].n_bags);
+      if (p.items[i].active) total += group_blocks(tables[i], k, p.items[i]);
       if (total >= (1ull << 31)) return MONO_ERR_ARG;
     }
     st[p.n] = (uint32_t)total;
@@ -916,22 +932,21 @@ int mono_group_lookup_pool(int32_t n_tables, mono_table* const* tables, const ui
     if ((rc = reserve(t, n_ids[i], n_bags[i])) != MONO_OK) return rc;
   }
   GroupPlan p;
+  int64_t all_ids = 0;
   if ((rc = group_begin(p, n_tables, tables, group_stream)) != MONO_OK) return rc;
   for (int32_t i = 0; i < n_tables; ++i) {
     group_describe(p, i, tables[i], ids[i], n_ids[i], slot_offsets[i], n_bags[i], out[i], nullptr, 0u,
                    is_prepared_batch(tables[i], ids[i], n_ids[i], slot_offsets[i], n_bags[i]));
     p.items[i].active = n_bags[i] > 0 ? 1u : 0u;           // a bag without IDs still pools to zeros
+    all_ids += n_ids[i] + n_bags[i];
   }
+  // every table's tiles are sized for its share of the GPU
+  for (int32_t i = 0; i < n_tables; ++i)
+    p.items[i].tile_bags = pool_tile(n_ids[i], n_bags[i], (int64_t)(grid_for(p.owner, 6) * ((double)(n_ids[i] + n_bags[i]) / (double)(all_ids ? all_ids : 1))),
+                                     kPoolThreads / lanes_of_class(p.items[i].lane_class));
   if ((rc = group_upload(p, tables)) != MONO_OK) return rc;
-  bool any_prepared = false;
-  for (int32_t i = 0; i < n_tables; ++i) any_prepared |= p.items[i].prepared && p.items[i].n_ids > 0;
-  bool any_unprepared = false;
-  for (int32_t i = 0; i < n_tables; ++i) any_unprepared |= !p.items[i].prepared && p.items[i].n_ids > 0;
-  // (each of the two passes skips the other kind of table)
-  if (any_prepared) GROUP_LAUNCH(p, K_FILE, GK_FILE, 256, group_file_rows_kernel);
-  if (any_unprepared) GROUP_LAUNCH(p, K_PROBE, GK_FILE, 256, group_probe_rows_kernel);
-  GROUP_LAUNCH(p, K_GATHER, GK_GATHER, 256, group_gather_pool_kernel<0>);
-  GROUP_LAUNCH(p, K_GATHER, GK_GATHER_WIDE, 256, group_gather_pool_kernel<1>);
+  GROUP_LAUNCH(p, K_POOL, GK_POOL, kPoolThreads, group_pool_kernel<0>);
+  GROUP_LAUNCH(p, K_POOL, GK_POOL_WIDE, kPoolThreads, group_pool_kernel<1>);
   CUDA_TRY(p.owner, cudaGetLastError());
   for (int32_t i = 0; i < n_tables; ++i)
     if (p.items[i].prepared && p.items[i].n_ids > 0) tables[i]->prep.filed = true;
@@ -1087,8 +1102,7 @@ int mono_lookup_pool_noalloc(mono_table* t, const uint64_t* ids, int64_t n_ids, 
   if ((rc = noalloc_scratch(t, &occ_row)) != MONO_OK) return rc;
   const unsigned long long* d_ids = reinterpret_cast<const unsigned long long*>(ids);
   const long long* d_off = reinterpret_cast<const long long*>(slot_offsets);
-  if ((rc = launch_probe(t, d_ids, n_ids, occ_row)) != MONO_OK) return rc;
-  return launch_gather(t, occ_row, n_ids, d_off, n_bags, out);
+  return launch_pool(t, d_ids, occ_row, n_ids, d_off, n_bags, out, false);
 }
 
 // Streams, events and staging of the host-buffer calls, made by the first of them.
