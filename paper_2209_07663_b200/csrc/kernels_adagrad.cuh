@@ -9,18 +9,18 @@
 // occurrences (filed by the pull, gather_pool_kernel, when the batch was announced, else by
 // file_segments_kernel inside the push).
 //  - once (most distinct IDs of a long-tailed batch): its gradient is the
-//    pooled gradient of its one bag, so update_singletons_kernel updates the
-//    row straight from that bag's gradient row;
-//  - 2 .. kSegChunk times: one lane group of reduce_adagrad_kernel gathers
-//    the gradient rows of the segment's bags;
+//    pooled gradient of its one bag, so the row is updated straight from that
+//    bag's gradient row;
+//  - 2 .. kSegChunk times: one lane group gathers the gradient rows of the
+//    segment's bags;
 //  - more (the head of the Zipf distribution: one ID can own several percent of
 //    a batch): the segment is cut into parts of kSegChunk that separate groups
-//    reduce into fp64 partial sums, combined by one block per ID in a fixed
-//    order.
+//    reduce into fp64 partial sums, which are added up in a fixed tree.
 #pragma once
 
 #include "kernels_dedup.cuh"
 #include "kernels_forward.cuh"
+#include "kernels_table.cuh"
 
 namespace mono {
 
@@ -62,7 +62,7 @@ __device__ inline void update_row(const TableView& tv, uint32_t row_word, unsign
 }
 
 // The per-call set must be empty again when the push ends.  Its primary tier is wiped as a whole
-// (clear_primary_kernel: a streaming write costs less than one scattered store per ID); an ID
+// (clear_primary: a streaming write costs less than one scattered store per ID); an ID
 // that overflowed into the secondary tier, which is far larger and almost empty, has its slot
 // emptied by the kernel that updates its row.
 __device__ inline void clear_overflow_slot(const Work& wk, uint32_t slot) {
@@ -72,15 +72,12 @@ __device__ inline void clear_overflow_slot(const Work& wk, uint32_t slot) {
   }
 }
 
-__device__ inline void clear_primary_body(const Work& wk, uint32_t vblock, uint32_t vgrid) {
+__device__ inline void clear_primary(const Work& wk, uint32_t vblock, uint32_t vgrid) {
   const uint32_t n = wk.primary_mask + 1u;
   ulonglong2 e; e.x = kEmptyKey; e.y = 0ull;
   for (uint32_t i = vblock * blockDim.x + threadIdx.x; i < n; i += vgrid * blockDim.x)
     *reinterpret_cast<ulonglong2*>(wk.bset + i) = e;
 }
-__global__ void __launch_bounds__(256)
-clear_primary_kernel(Work wk) { after_previous_kernel(); clear_primary_body(wk, blockIdx.x, gridDim.x); }
-
 // Sum of grad rows of bags bag_of_sorted[begin .. end) for the NV column
 // vectors this lane owns.  Eight independent row loads in flight per step.
 template <int G, int NV>
@@ -139,6 +136,146 @@ file_segments_kernel(Work wk, long long n_ids, long long n_bags) { after_previou
   file_segments_body(wk, n_ids, n_bags, blockIdx.x, gridDim.x);
 }
 
+// ---- the row updates of a push: one kernel -----------------------------------
+// Blocks of one grid take different kinds of work, the heaviest first: parts of long segments, short
+// segments, what occurs once.  None waits for another, so the blocks of the next kind fill the SMs
+// as those of the one before run out, and a small batch has all of them resident at once.  Measured
+// against eight kernels on two streams (clear, expand, reduce twice, singles, fold, combine, finish),
+// whole step: 20 000 IDs 54 -> 36 us, 1 M IDs 180 -> 153, 4 M drifting 360 -> 348, 8 M 1404 -> 1395; against the
+// three kinds one after the other in every block, 47 / 163 / 411 / 1437.
+// What bounds it: gradient rows gathered at random for the first two kinds (latency; ten blocks of 128
+// threads per SM at 48 registers: eight at 64 measured 3 % of a step slower, twelve spill), HBM for the third.
+
+// Sum of partial sums src[0], src[stride], ... (n of them, in that order) for the columns this lane owns.
+// They were written by other blocks: read past L1.
+template <int G, int NV>
+__device__ __forceinline__ void sum_partials(const double* src, uint32_t n, size_t stride, uint32_t dim, int gl, D4 (&s)[NV]) {
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const uint32_t c4 = gl + v * G;
+    if (c4 * 4u < dim) {
+      const double2* p = reinterpret_cast<const double2*>(src) + c4 * 2;
+      D4 a = D4{0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+      for (uint32_t i = 0; i < n; ++i, p += stride / 2) {
+        const double2 x = __ldcg(p), y = __ldcg(p + 1);
+        a.x += x.x; a.y += x.y; a.z += y.x; a.w += y.y;
+      }
+      s[v] = a;
+    }
+  }
+}
+
+// The long ID that part p belongs to: the last one whose first part is not after p.  The lanes of the
+// group look at G places at a time.
+template <int G>
+__device__ __forceinline__ uint32_t owner_of_part(const Work& wk, uint32_t n_long, uint32_t p, int gl, unsigned group_mask) {
+  uint32_t lo = 0, n = n_long;                                           // it is in [lo, lo + n)
+  while (n > 1) {
+    const uint32_t step = (n + G - 1) / G, at = gl * step;
+    const bool before = at < n && wk.long_part0[lo + at] <= p;
+    const uint32_t c = __popc(__ballot_sync(group_mask, before)) - 1;
+    lo += c * step;
+    n = min(step, n - c * step);
+  }
+  return lo;
+}
+
+// The parts of the long segments.  A lane group sums one part into fp64 partial sums in scratch.
+// Partial sums are added up in a tree: the group that finishes the last of kFanIn neighbours adds
+// them up and goes on to the next level, and the one that reaches the top updates the row.  The
+// order of every addition is fixed by the parts' numbers, whoever does it.  (A tree, because one ID
+// can own a tenth of a batch: with 64 neighbours at a time and then all the rest, adding up the
+// 11 000 parts of such an ID was a serial chain of 50 us.)
+template <int G, int NV>
+__device__ inline void reduce_parts(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
+                                    bool ordered, uint32_t vblock, uint32_t vgrid) {
+  const unsigned long long longs = wk.call->longs;
+  const uint32_t n_parts = (uint32_t)longs, n_long = (uint32_t)(longs >> 32);
+  const int gl = threadIdx.x % G, lane = threadIdx.x & 31;
+  const unsigned group_mask = G == 32 ? 0xFFFFFFFFu : ((1u << (G & 31)) - 1u) << (lane / G * G);
+  const uint32_t groups = (vgrid * blockDim.x) / G;
+  for (uint32_t item = (vblock * blockDim.x + threadIdx.x) / G; item < n_parts; item += groups) {
+    const uint32_t p = ordered ? wk.part_order[item] : item;
+    if (!MONO_INDEX_OK(wk.error_bits, p, wk.max_parts)) continue;
+    const uint32_t li = ordered ? wk.part_u[p] : owner_of_part<G>(wk, n_long, p, gl, group_mask);
+    if (!MONO_INDEX_OK(wk.error_bits, li, wk.max_long)) continue;
+    const uint32_t u = wk.long_u[li], p0 = wk.long_part0[li];
+    const uint32_t row_word = wk.urow[u];
+    if (row_word == kNoRow) continue;                                    // no row: gradient dropped, by every part
+    const uint32_t m = wk.ulen[u], seg = wk.useg[u];
+    uint32_t k = p - p0;
+    const uint32_t begin = seg + k * kSegChunk, end = (k + 1) * kSegChunk < m ? begin + kSegChunk : seg + m;
+    if (!MONO_INDEX_OK(wk.error_bits, (unsigned long long)end - 1, wk.max_ids)) continue;
+    D4 s[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) s[v] = D4{0.0, 0.0, 0.0, 0.0};
+    reduce_segment<G, NV>(wk, grad, n_bags, tv.dim, gl, begin, end, s);
+    const uint32_t parts = (m + kSegChunk - 1) / kSegChunk;
+    bool top = true;
+    for (uint32_t level = 0, step = 1; step < parts; ++level, step *= kFanIn) {
+      // s is the sum of the parts [k, k + step) of the ID, cut off at the last: leave it where the level above finds it
+      double* dst = wk.partials + (size_t)(p0 + k) * tv.dim;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const uint32_t c4 = gl + v * G;
+        if (c4 * 4u < tv.dim) {
+          reinterpret_cast<double2*>(dst)[c4 * 2] = make_double2(s[v].x, s[v].y);
+          reinterpret_cast<double2*>(dst)[c4 * 2 + 1] = make_double2(s[v].z, s[v].w);
+        }
+      }
+      k = k / (step * kFanIn) * (step * kFanIn);
+      const uint32_t want = min(kFanIn, (parts - k + step - 1) / step);
+      uint32_t* counter = wk.part_done + p0 + k;                         // five bits per level: kFanIn at most
+      __threadfence();
+      __syncwarp(group_mask);
+      uint32_t before = 0;
+      if (gl == 0) before = atomicAdd(counter, 1u << (5 * level));
+      before = __shfl_sync(group_mask, before, 0, G) >> (5 * level) & 31u;
+      if (before != want - 1u) { top = false; break; }
+      __threadfence();
+      if (gl == 0) atomicSub(counter, want << (5 * level));              // zero again for the next call
+      sum_partials<G, NV>(wk.partials + (size_t)(p0 + k) * tv.dim, want, (size_t)step * tv.dim, tv.dim, gl, s);
+    }
+    if (!top) continue;
+    const unsigned long long id = wk.uid[u];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const uint32_t c4 = gl + v * G;
+      if (c4 * 4u < tv.dim) update_row(tv, row_word, id, c4, s[v]);
+    }
+  }
+}
+
+// The repeated IDs: a lane group each, which reduces the segment, if it is short, and updates the row.
+// (Measured against one packed record per repeated ID, read a trip ahead: the separate arrays were 2 %
+// of a step faster on the largest configuration.)
+template <int G, int NV>
+__device__ inline void reduce_short(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
+                                    uint32_t vblock, uint32_t vgrid) {
+  const uint32_t n = wk.call->n_multi;
+  const int gl = threadIdx.x % G;
+  const uint32_t groups = (vgrid * blockDim.x) / G;
+  for (uint32_t item = (vblock * blockDim.x + threadIdx.x) / G; item < n; item += groups) {
+    const uint32_t u = wk.multi_list[item];
+    if (gl == 0) clear_overflow_slot(wk, wk.uslot[u]);
+    const uint32_t m = wk.ulen[u];
+    const uint32_t row_word = wk.urow[u];
+    if (row_word == kNoRow || m > kSegChunk) continue;                   // no row: gradient dropped; long: in parts
+    const uint32_t begin = wk.useg[u];
+    D4 s[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) s[v] = D4{0.0, 0.0, 0.0, 0.0};
+    reduce_segment<G, NV>(wk, grad, n_bags, tv.dim, gl, begin, begin + m, s);
+    const unsigned long long id = wk.uid[u];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const uint32_t c4 = gl + v * G;
+      if (c4 * 4u < tv.dim) update_row(tv, row_word, id, c4, s[v]);
+    }
+  }
+}
+
 // The IDs that occur once in the batch (most distinct IDs of a long-tailed batch): the
 // gradient of such an ID is the pooled gradient of its one bag, so its row is updated
 // straight from there.  One warp per 32 consecutive distinct IDs, which are numbered in
@@ -147,12 +284,12 @@ file_segments_kernel(Work wk, long long n_ids, long long n_bags) { after_previou
 // which read the bag's gradient row, the table row and its accumulator, and write both
 // back updated.
 template <int G, int NV>
-__device__ inline void update_singletons_body(const TableView& tv, const Work& wk, const float* __restrict__ grad,
+__device__ inline void update_singletons(const TableView& tv, const Work& wk, const float* __restrict__ grad,
                                               long long n_bags, uint32_t vblock, uint32_t vgrid) {
   constexpr int kGroups = 32 / G;
   const int lane = threadIdx.x & 31;
   const int gl = lane % G, grp = lane / G;
-  const uint32_t n = tv.st->n_unique;
+  const uint32_t n = wk.call->n_unique;
   const uint32_t n_warps = (vgrid * blockDim.x) >> 5;
   const uint32_t n_rounds = (n + 31) / 32;
   unsigned int n_single = 0;
@@ -204,180 +341,29 @@ __device__ inline void update_singletons_body(const TableView& tv, const Work& w
   }
   if (lane == 0 && n_single) atomicAdd(&tv.st->sum_single_resident, (unsigned long long)n_single);
 }
-template <int G, int NV>
-__global__ void __launch_bounds__(256)
-update_singletons_kernel(TableView tv, Work wk, const float* __restrict__ grad, long long n_bags) { after_previous_kernel();
-  update_singletons_body<G, NV>(tv, wk, grad, n_bags, blockIdx.x, gridDim.x);
-}
-
-// One lane group per work item.  Items [0, n_parts) are the parts of the long
-// segments (the heaviest items, so they are started first): a group reduces
-// one part into fp64 partial sums in scratch, which combine_adagrad_kernel adds
-// up afterwards.  Items [n_parts, n_parts + n_multi) are the repeated IDs: a
-// group empties the ID's slot of the per-call set (every occurrence has been
-// filed by now), and when the segment is short reduces it and updates the row.
-// `which` selects the items of one launch: kReduceParts, kReduceShort (the repeated IDs need
-// nothing from the kernels that order the parts, so they can run beside them), or both.
-enum : int { kReduceParts = 1, kReduceShort = 2 };
+constexpr int kRowThreads = 128;
+// How the grid is shared out: blocks [0, parts) take the parts, the next `shorts` the short segments,
+// the rest what occurs once.
+struct RowGrid { uint32_t parts, shorts, singles; };
 
 template <int G, int NV>
-__device__ inline void reduce_adagrad_body(const TableView& tv, const Work& wk, const float* __restrict__ grad,
-                                           long long n_bags, int which, uint32_t vblock, uint32_t vgrid) {
-  const uint32_t n = tv.st->n_multi;
-  uint32_t n_parts = tv.st->n_parts;
-  if (n_parts > wk.max_parts) n_parts = wk.max_parts;
-  const uint32_t first_item = (which & kReduceParts) ? 0u : n_parts;
-  const uint32_t n_items = (which & kReduceShort) ? n + n_parts : n_parts;
-  const int gl = threadIdx.x % G;
-  const uint32_t groups = (vgrid * blockDim.x) / G;
-  for (uint32_t item = first_item + (vblock * blockDim.x + threadIdx.x) / G; item < n_items; item += groups) {
-    D4 s[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) s[v] = D4{0.0, 0.0, 0.0, 0.0};
-    if (item >= n_parts) {
-      // (measured against one packed record per repeated ID, read a trip ahead: these separate
-      // arrays were 2 % of a step faster on the largest configuration)
-      const uint32_t u = wk.multi_list[item - n_parts];
-      if (gl == 0) clear_overflow_slot(wk, wk.uslot[u]);
-      const uint32_t m = wk.ulen[u];
-      const uint32_t row_word = wk.urow[u];
-      if (row_word == kNoRow || m > kSegChunk) continue;      // no row: gradient dropped; long: in parts
-      const uint32_t begin = wk.useg[u];
-      reduce_segment<G, NV>(wk, grad, n_bags, tv.dim, gl, begin, begin + m, s);
-      const unsigned long long id = wk.uid[u];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const uint32_t c4 = gl + v * G;
-        if (c4 * 4u < tv.dim) update_row(tv, row_word, id, c4, s[v]);
-      }
-    } else {
-      const uint32_t p = wk.part_order[item];
-      if (!MONO_INDEX_OK(wk.error_bits, p, wk.max_parts)) continue;
-      const uint32_t li = wk.part_u[p];
-      if (!MONO_INDEX_OK(wk.error_bits, li, wk.max_long)) continue;
-      const uint32_t u = wk.long_u[li];
-      const uint32_t k = p - wk.long_part0[li];
-      const uint32_t seg_end = wk.useg[u] + wk.ulen[u];
-      const uint32_t begin = wk.useg[u] + k * kSegChunk;
-      const uint32_t end = begin + kSegChunk < seg_end ? begin + kSegChunk : seg_end;
-      if (!MONO_INDEX_OK(wk.error_bits, (unsigned long long)end - 1, wk.max_ids)) continue;
-      reduce_segment<G, NV>(wk, grad, n_bags, tv.dim, gl, begin, end, s);
-      double* dst = wk.partials + (size_t)p * tv.dim;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const uint32_t c4 = gl + v * G;
-        if (c4 * 4u < tv.dim) {
-          reinterpret_cast<double2*>(dst)[c4 * 2] = make_double2(s[v].x, s[v].y);
-          reinterpret_cast<double2*>(dst)[c4 * 2 + 1] = make_double2(s[v].z, s[v].w);
-        }
-      }
-    }
+__device__ __forceinline__ void update_rows_body(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
+                                                 bool ordered, const RowGrid& grid, uint32_t total_blocks, uint32_t vblock) {
+  if (vblock < grid.parts) {
+    reduce_parts<G, NV>(tv, wk, grad, n_bags, ordered, vblock, grid.parts);
+  } else if (vblock - grid.parts < grid.shorts) {
+    reduce_short<G, NV>(tv, wk, grad, n_bags, vblock - grid.parts, grid.shorts);
+  } else {
+    update_singletons<G, NV>(tv, wk, grad, n_bags, vblock - grid.parts - grid.shorts, grid.singles);
+    clear_primary(wk, vblock - grid.parts - grid.shorts, grid.singles);
   }
+  block_done(tv.st, wk, total_blocks);
 }
-
 template <int G, int NV>
-__global__ void __launch_bounds__(256)
-reduce_adagrad_kernel(TableView tv, Work wk, const float* __restrict__ grad, long long n_bags, int which) { after_previous_kernel();
-  reduce_adagrad_body<G, NV>(tv, wk, grad, n_bags, which, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(kRowThreads, NV == 1 ? 10 : 4)
+update_rows_kernel(TableView tv, Work wk, const float* __restrict__ grad, long long n_bags, int ordered, RowGrid grid, uint32_t total_blocks) {
+  after_previous_kernel();
+  update_rows_body<G, NV>(tv, wk, grad, n_bags, ordered != 0, grid, total_blocks, blockIdx.x);
 }
-
-// First level of the combination for very long segments: one block adds up one
-// group of kFoldWidth consecutive parts of one ID, column by column, and leaves
-// the sum in the group's first part.  Fixed order within the block.
-__device__ inline void fold_partials_body(const TableView& tv, const Work& wk, uint32_t vblock, uint32_t vgrid) {
-  __shared__ double s_sum[8][256];
-  uint32_t n_folds = tv.st->n_folds;
-  if (n_folds > wk.max_folds) n_folds = wk.max_folds;
-  const uint32_t dim = tv.dim;
-  for (uint32_t fi = vblock; fi < n_folds; fi += vgrid) {
-    const uint32_t li = wk.fold_li[fi], f = wk.fold_idx[fi];
-    const uint32_t u = wk.long_u[li];
-    if (wk.urow[u] == kNoRow) continue;               // block-uniform
-    const uint32_t parts = (wk.ulen[u] + kSegChunk - 1) / kSegChunk;
-    const uint32_t p_begin = f * kFoldWidth;
-    const uint32_t p_end = p_begin + kFoldWidth < parts ? p_begin + kFoldWidth : parts;
-    double* base = wk.partials + ((size_t)wk.long_part0[li] + p_begin) * dim;
-    for (uint32_t cbase = 0; cbase < dim; cbase += 256) {
-      const uint32_t width = dim - cbase < 256 ? dim - cbase : 256;
-      uint32_t slices = 256 / width;
-      if (slices > 8) slices = 8;
-      const uint32_t col = threadIdx.x % width, slice = threadIdx.x / width;
-      const uint32_t n = p_end - p_begin;
-      if (slice < slices) {
-        const uint32_t per = (n + slices - 1) / slices;
-        const uint32_t lo = slice * per, hi = lo + per < n ? lo + per : n;
-        double a0 = 0.0, a1 = 0.0;
-        uint32_t p = lo;
-        for (; p + 2 <= hi; p += 2) { a0 += base[(size_t)p * dim + cbase + col]; a1 += base[(size_t)(p + 1) * dim + cbase + col]; }
-        if (p < hi) a0 += base[(size_t)p * dim + cbase + col];
-        s_sum[slice][col] = a0 + a1;
-      }
-      __syncthreads();                                // every read of this group's parts is done
-      if (threadIdx.x < width) {
-        double g = 0.0;
-        for (uint32_t s = 0; s < slices; ++s) g += s_sum[s][threadIdx.x];
-        base[cbase + threadIdx.x] = g;
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__global__ void __launch_bounds__(256)
-fold_partials_kernel(TableView tv, Work wk) { after_previous_kernel(); fold_partials_body(tv, wk, blockIdx.x, gridDim.x); }
-
-// One block per long ID: the block's threads split into slices of the parts
-// (or, for a very long segment, of the group sums fold_partials_kernel left),
-// one column each; the slices' sums are added in increasing order, so the
-// combination order is fixed.
-constexpr int kCombineThreads = 256;
-__device__ inline void combine_adagrad_body(const TableView& tv, const Work& wk, uint32_t vblock, uint32_t vgrid) {
-  constexpr int kMaxSlices = 8;
-  __shared__ double s_sum[kMaxSlices][256];
-  uint32_t n_long = tv.st->n_long;
-  if (n_long > wk.max_long) n_long = wk.max_long;
-  const uint32_t dim = tv.dim;
-  for (uint32_t li = vblock; li < n_long; li += vgrid) {
-    const uint32_t u = wk.long_u[li];
-    const uint32_t row_word = wk.urow[u];
-    if (row_word == kNoRow) continue;                 // block-uniform
-    const uint32_t m = wk.ulen[u];
-    uint32_t parts = (m + kSegChunk - 1) / kSegChunk;
-    size_t stride = dim;                              // distance between the sums to add
-    if (parts > kFoldWidth) { parts = (parts + kFoldWidth - 1) / kFoldWidth; stride = (size_t)kFoldWidth * dim; }
-    const double* src = wk.partials + (size_t)wk.long_part0[li] * dim;
-    const unsigned long long id = wk.uid[u];
-    for (uint32_t cbase = 0; cbase < dim; cbase += 256) {
-      const uint32_t width = dim - cbase < 256 ? dim - cbase : 256;      // multiple of 4
-      uint32_t slices = kCombineThreads / width;
-      if (slices > kMaxSlices) slices = kMaxSlices;
-      const uint32_t col = threadIdx.x % width, slice = threadIdx.x / width;
-      if (slice < slices) {
-        const uint32_t per = (parts + slices - 1) / slices;
-        const uint32_t p_lo = slice * per, p_hi = p_lo + per < parts ? p_lo + per : parts;
-        double a0 = 0.0, a1 = 0.0;
-        uint32_t p = p_lo;
-        for (; p + 2 <= p_hi; p += 2) { a0 += src[p * stride + cbase + col]; a1 += src[(p + 1) * stride + cbase + col]; }
-        if (p < p_hi) a0 += src[p * stride + cbase + col];
-        s_sum[slice][col] = a0 + a1;
-      }
-      __syncthreads();
-      if (threadIdx.x < width / 4) {
-        D4 g = D4{0.0, 0.0, 0.0, 0.0};
-        for (uint32_t s = 0; s < slices; ++s) {
-          g.x += s_sum[s][threadIdx.x * 4 + 0];
-          g.y += s_sum[s][threadIdx.x * 4 + 1];
-          g.z += s_sum[s][threadIdx.x * 4 + 2];
-          g.w += s_sum[s][threadIdx.x * 4 + 3];
-        }
-        update_row(tv, row_word, id, cbase / 4 + threadIdx.x, g);
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kCombineThreads)
-combine_adagrad_kernel(TableView tv, Work wk) { after_previous_kernel(); combine_adagrad_body(tv, wk, blockIdx.x, gridDim.x); }
 
 }  // namespace mono

@@ -36,7 +36,7 @@ struct __align__(16) BatchSlot {
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 constexpr uint32_t kNoSegment = 0xFFFFFFFFu;
 constexpr uint32_t kSegChunk = 64;             // longest segment one lane group reduces alone
-constexpr uint32_t kFoldWidth = 64;           // parts added up by one block of fold_partials_kernel
+constexpr uint32_t kFanIn = 16;                // partial sums that are added up at a time
 constexpr int kTileIds = 512;                  // occurrences per block of dedup_tile_kernel
 constexpr int kTileSlots = 1024;               // shared-memory table of one tile
 constexpr int kTileThreads = 256;              // block size of dedup_tile_kernel
@@ -45,6 +45,7 @@ constexpr uint32_t kWindows = 1024;            // the parts of long segments are
 
 // Scratch of one mono_apply_grads call.
 struct Work {
+  CallState* call;
   // The per-call set has two tiers, both empty between calls.  The primary tier
   // is small enough to stay in L2 for a batch with the usual share of repeats;
   // an ID that finds no free slot among its first kPrimaryProbes positions there
@@ -74,9 +75,8 @@ struct Work {
   uint32_t* part_order;      // [max_parts] the parts in the order they are reduced in: by window of the batch
   uint32_t* win_count;       // [2 * kWindows] parts per window, then a cursor per window; zero between calls
   double* partials;          // [max_parts][dim]
-  uint32_t* fold_li;         // [max_folds] owner (index into long_u) of each fold
-  uint32_t* fold_idx;        // [max_folds] which group of kFoldWidth parts of that owner
-  uint32_t max_long, max_parts, max_folds;
+  uint32_t* part_done;       // [max_parts] partial sums that are there, counted at the first of the kFanIn that belong together; zero between calls
+  uint32_t max_long, max_parts;
   uint32_t max_ids;          // entries of the per-occurrence and per-distinct-ID arrays
   uint32_t n_slots;          // slots of bset, both tiers
   unsigned int* error_bits;  // the table's sticky condition bits (the checked build reports through them)
@@ -87,21 +87,21 @@ struct Work {
 __device__ inline bool bag_ok(long long lo, long long hi, long long n_ids) { return lo >= 0 && hi >= lo && hi <= n_ids; }
 
 // bag -> occurrences: every occurrence learns which bag it belongs to.  A malformed bag
-// writes nothing, sets the sticky condition bit and marks the call, so that the grouping
-// pass checks every occurrence against the bag it claims (occurrence_covered).
+// writes nothing and marks the call, so that the grouping pass checks every occurrence against the
+// bag it claims (occurrence_covered) and the look-up that follows sets the sticky condition bit.
 __device__ inline void fill_occ_bag_body(const long long* __restrict__ offsets, long long n_bags, long long n_ids,
-                                         uint32_t* __restrict__ occ_bag, DevState* st, uint32_t vblock, uint32_t vgrid) {
+                                         uint32_t* __restrict__ occ_bag, CallState* call, uint32_t vblock, uint32_t vgrid) {
   const long long stride = (long long)vgrid * blockDim.x;
   for (long long b = (long long)vblock * blockDim.x + threadIdx.x; b < n_bags; b += stride) {
     const long long lo = offsets[b], hi = offsets[b + 1];
-    if (!bag_ok(lo, hi, n_ids)) { atomicOr(&st->error_bits, 4u /* MONO_DEV_BAD_OFFSETS */); st->call_bad_offsets = 1u; continue; }
+    if (!bag_ok(lo, hi, n_ids)) { call->bad_offsets = 1u; continue; }
     for (long long j = lo; j < hi; ++j) occ_bag[j] = (uint32_t)b;
   }
 }
 __global__ void __launch_bounds__(256)
 fill_occ_bag_kernel(const long long* __restrict__ offsets, long long n_bags, long long n_ids,
-                    uint32_t* __restrict__ occ_bag, DevState* st) { after_previous_kernel();
-  fill_occ_bag_body(offsets, n_bags, n_ids, occ_bag, st, blockIdx.x, gridDim.x);
+                    uint32_t* __restrict__ occ_bag, CallState* call) { after_previous_kernel();
+  fill_occ_bag_body(offsets, n_bags, n_ids, occ_bag, call, blockIdx.x, gridDim.x);
 }
 
 // Only used when the call's offsets are malformed: does a well-formed bag cover occurrence j,
@@ -142,7 +142,7 @@ __device__ inline unsigned long long block_exclusive_scan(unsigned long long v, 
 // One block per tile of kTileIds consecutive occurrences.
 // (eight blocks per SM: measured 0.207 ms on the largest configuration against 0.234 ms with six)
 __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long* __restrict__ ids, long long n_ids,
-                                       const long long* __restrict__ offsets, long long n_bags, DevState* st,
+                                       const long long* __restrict__ offsets, long long n_bags,
                                        unsigned long long seed, uint32_t vblock) {
   constexpr int kPerThread = kTileIds / kTileThreads;
   __shared__ unsigned long long s_key[kTileSlots];
@@ -155,7 +155,7 @@ __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long*
   long long first = offsets[0], last = offsets[n_bags];
   if (first < 0) first = 0;
   if (last > n_ids) last = n_ids;
-  const bool check_each = st->call_bad_offsets != 0u;     // set by fill_occ_bag_kernel, earlier on this stream
+  const bool check_each = wk.call->bad_offsets != 0u;     // set by fill_occ_bag_kernel, earlier on this stream
   if (check_each) { first = 0; last = n_ids; }
   __syncthreads();
 
@@ -254,8 +254,8 @@ __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long*
   unsigned int my_u = (unsigned int)block_exclusive_scan(((unsigned long long)n_valid << 32) | n_new, s_warp, &total);
   if (threadIdx.x == 0) {
     const unsigned int total_new = (unsigned int)total, total_valid = (unsigned int)(total >> 32);
-    s_ubase = total_new ? atomicAdd(&st->n_unique, total_new) : 0u;
-    if (total_valid) atomicAdd(&st->n_valid_ids, total_valid);
+    s_ubase = total_new ? atomicAdd(&wk.call->n_unique, total_new) : 0u;
+    if (total_valid) atomicAdd(&wk.call->n_valid_ids, total_valid);
   }
   __syncthreads();
   my_u += s_ubase;
@@ -284,9 +284,9 @@ __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long*
 
 __global__ void __launch_bounds__(kTileThreads, 8)
 dedup_tile_kernel(Work wk, const unsigned long long* __restrict__ ids, long long n_ids,
-                  const long long* __restrict__ offsets, long long n_bags, DevState* st,
+                  const long long* __restrict__ offsets, long long n_bags,
                   unsigned long long seed) { after_previous_kernel();
-  dedup_tile_body(wk, ids, n_ids, offsets, n_bags, st, seed, blockIdx.x);
+  dedup_tile_body(wk, ids, n_ids, offsets, n_bags, seed, blockIdx.x);
 }
 
 }  // namespace mono

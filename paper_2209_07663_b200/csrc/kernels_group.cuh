@@ -30,6 +30,8 @@ struct GroupItem {
                                  // 4..6: 32 lanes with 2 / 4 / 8 vectors per lane
   uint32_t pool_wide;            // lookup: 32-byte accesses (classes 4..6 only)
   uint32_t tile_bags;            // lookup: bags per block
+  RowGrid row_grid;              // push: the row updates' blocks
+  uint32_t total_blocks;         // push: of the insertions and the row updates together
   uint32_t active;               // 0: the table takes no part in this call (empty batch)
 };
 
@@ -56,13 +58,13 @@ __device__ inline uint32_t find_table(const uint32_t* __restrict__ start, uint32
 __global__ void __launch_bounds__(256)
 group_fill_occ_bag_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
-  fill_occ_bag_body(it.off, it.n_bags, it.n_ids, it.wk.occ_bag, it.tv.st, vblock, vgrid);
+  fill_occ_bag_body(it.off, it.n_bags, it.n_ids, it.wk.occ_bag, it.wk.call, vblock, vgrid);
 }
 
 __global__ void __launch_bounds__(kTileThreads, 8)
 group_dedup_tile_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
-  dedup_tile_body(it.wk, it.ids, it.n_ids, it.off, it.n_bags, it.tv.st, it.dedup_seed, vblock);
+  dedup_tile_body(it.wk, it.ids, it.n_ids, it.off, it.n_bags, it.dedup_seed, vblock);
 }
 
 template <int MODE>
@@ -82,6 +84,7 @@ __global__ void __launch_bounds__(256)
 group_table_insert_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   table_insert_body(it.tv, it.wk, it.now, vblock, vgrid);
+  block_done(it.tv.st, it.wk, it.total_blocks);
 }
 
 // (of a push whose batch was not pulled since it was announced, or not announced)
@@ -89,43 +92,6 @@ __global__ void __launch_bounds__(256)
 group_file_segments_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   file_segments_body(it.wk, it.n_ids, it.n_bags, vblock, vgrid);
-}
-
-__global__ void __launch_bounds__(256)
-group_clear_primary_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  clear_primary_body(it.wk, vblock, vgrid);
-}
-
-__global__ void __launch_bounds__(128)
-group_expand_parts_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  expand_parts_body(it.tv, it.wk, vblock, vgrid);
-}
-
-__global__ void __launch_bounds__(kWindows)
-group_order_parts_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  order_parts_body(it.tv, it.wk, vblock, vgrid);
-}
-
-__global__ void __launch_bounds__(256)
-group_fold_partials_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  fold_partials_body(it.tv, it.wk, vblock, vgrid);
-}
-
-__global__ void __launch_bounds__(kCombineThreads)
-group_combine_adagrad_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  combine_adagrad_body(it.tv, it.wk, vblock, vgrid);
-}
-
-// one block per table
-__global__ void __launch_bounds__(256)
-group_finish_apply_kernel(const GroupItem* __restrict__ items, uint32_t n_tables, int commit) {
-  after_previous_kernel();
-  if (blockIdx.x < n_tables && items[blockIdx.x].active) finish_apply_body(items[blockIdx.x].tv.st, items[blockIdx.x].wk.win_count, commit);
 }
 
 // The kernels whose bodies are compiled per lane-group width.  A block's table decides the
@@ -184,20 +150,11 @@ group_pool_kernel(const GroupItem* __restrict__ items, const uint32_t* __restric
 }
 
 template <int WIDE>
-__global__ void __launch_bounds__(256)
-group_reduce_adagrad_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
+__global__ void __launch_bounds__(kRowThreads, WIDE ? 4 : 10)
+group_update_rows_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   by_lane_class<WIDE>(it.lane_class, [&](auto g, auto nv) {
-    reduce_adagrad_body<decltype(g)::value, decltype(nv)::value>(it.tv, it.wk, it.grad, it.n_bags, kReduceParts | kReduceShort, vblock, vgrid);
-  });
-}
-
-template <int WIDE>
-__global__ void __launch_bounds__(256)
-group_update_singletons_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
-  MONO_GROUP_PROLOGUE;
-  by_lane_class<WIDE>(it.lane_class, [&](auto g, auto nv) {
-    update_singletons_body<decltype(g)::value, decltype(nv)::value>(it.tv, it.wk, it.grad, it.n_bags, vblock, vgrid);
+    update_rows_body<decltype(g)::value, decltype(nv)::value>(it.tv, it.wk, it.grad, it.n_bags, false, it.row_grid, it.total_blocks, vblock);
   });
 }
 

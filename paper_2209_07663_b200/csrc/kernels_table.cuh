@@ -47,7 +47,7 @@ struct Reservation {
   uint32_t ins_pos;
 };
 
-__device__ inline Reservation block_reserve(const TableView& tv, BlockAlloc* sh, bool need_row, bool is_multi,
+__device__ inline Reservation block_reserve(const TableView& tv, CallState* call, BlockAlloc* sh, bool need_row, bool is_multi,
                                             bool need_insert, uint32_t seg_len) {
   // segment entries in bits 0..31, repeated IDs in 32..41, inserts in 42..51, rows in 52..61
   unsigned long long total = 0;
@@ -82,11 +82,11 @@ __device__ inline Reservation block_reserve(const TableView& tv, BlockAlloc* sh,
       sh->row_base = old;
       sh->rows_granted = granted;
     } else if (warp == 1u) {
-      sh->seg_base = seg_total ? atomicAdd(&tv.st->seg_cursor, seg_total) : 0u;
+      sh->seg_base = seg_total ? atomicAdd(&call->seg_cursor, seg_total) : 0u;
     } else if (warp == 2u) {
-      sh->multi_base = multi_total ? atomicAdd(&tv.st->n_multi, multi_total) : 0u;
+      sh->multi_base = multi_total ? atomicAdd(&call->n_multi, multi_total) : 0u;
     } else {
-      sh->ins_base = ins_total ? atomicAdd(&tv.st->n_insert, ins_total) : 0u;
+      sh->ins_base = ins_total ? atomicAdd(&call->n_insert, ins_total) : 0u;
     }
   }
   __syncthreads();
@@ -102,24 +102,25 @@ __device__ inline Reservation block_reserve(const TableView& tv, BlockAlloc* sh,
   return r;
 }
 
-// A distinct ID whose segment is longer than kSegChunk is reduced in parts:
-// register it and its parts.  Rare (the few hottest IDs of a batch).
-__device__ inline void register_long(const TableView& tv, const Work& wk, uint32_t u, uint32_t m) {
+// Window of the batch that part k of a segment of `parts` parts falls into.  A segment lists
+// its occurrences roughly in batch order (tile by tile), so part k of n covers roughly the
+// k-th n-th of the bags.
+__device__ inline uint32_t part_window(uint32_t k, uint32_t parts) {
+  return (uint32_t)(((unsigned long long)k * kWindows) / parts);
+}
+
+// A distinct ID whose segment is longer than kSegChunk (the few hottest IDs of a batch) is reduced
+// in parts: register it.  One counter hands out its place and its parts together, so the first parts
+// ascend with the places, and the owner of a part can be searched for.  (Naming every part's owner
+// here, with the lanes of a warp, cost a drifting batch of 4 M IDs 75 us: distinct IDs are numbered as
+// the batch first shows them, so the hottest, with ten thousand parts each, sit in the same few warps.)
+__device__ inline void register_long(const Work& wk, uint32_t u, uint32_t m) {
   const uint32_t parts = (m + kSegChunk - 1) / kSegChunk;
-  const uint32_t li = atomicAdd(&tv.st->n_long, 1u);
-  const uint32_t p0 = atomicAdd(&tv.st->n_parts, parts);
-  if (li < wk.max_long && p0 + parts <= wk.max_parts) {
-    wk.long_u[li] = u;
-    wk.long_part0[li] = p0;
-    // (part_u[] is filled by expand_parts_kernel: a segment can have thousands of parts)
-    if (parts > kFoldWidth) {
-      // very long segment: its parts are first added up in groups of kFoldWidth
-      const uint32_t nf = (parts + kFoldWidth - 1) / kFoldWidth;
-      const uint32_t f0 = atomicAdd(&tv.st->n_folds, nf);
-      if (f0 + nf <= wk.max_folds)
-        for (uint32_t f = 0; f < nf; ++f) { wk.fold_li[f0 + f] = li; wk.fold_idx[f0 + f] = f; }
-    }
-  }
+  const unsigned long long at = atomicAdd(&wk.call->longs, 1ull << 32 | parts);
+  const uint32_t li = (uint32_t)(at >> 32), p0 = (uint32_t)at;
+  if (!MONO_INDEX_OK(wk.error_bits, li, wk.max_long) || !MONO_INDEX_OK(wk.error_bits, (unsigned long long)p0 + parts - 1, wk.max_parts)) return;
+  wk.long_u[li] = u;
+  wk.long_part0[li] = p0;
 }
 
 // Phase 2 of a push: one thread per distinct ID, in up to two halves.
@@ -127,7 +128,8 @@ __device__ inline void register_long(const TableView& tv, const Work& wk, uint32
 //  kLookUp  (can run ahead of the push, when mono_prepare_push announced the batch: it changes
 //           nothing in the table) -- the ID's multiplicity is read from the per-call set, the ID is
 //           looked up in the key store (the cell an insertion prefers first), an ID that occurs more
-//           than once is given its segment of bag_of_sorted[] and its place in multi_list[];
+//           than once is given its segment of bag_of_sorted[] and its place in multi_list[], one
+//           that occurs more than kSegChunk times the parts it is reduced in;
 //           the ID's slot of the per-call set is rewritten to (segment start, row owned so far),
 //           which is what the occurrences need, and the cell is remembered in ucell[].
 //  kCommit  (the push itself) -- a tracked ID gets count += multiplicity (saturating at the
@@ -147,11 +149,12 @@ __device__ inline Cell* cell_address(const TableView& tv, unsigned long long cel
 template <int MODE>
 __device__ inline void table_update_body(const TableView& tv, const Work& wk, uint32_t now, uint32_t vblock, uint32_t vgrid) {
   __shared__ BlockAlloc sh;
-  const uint32_t n = tv.st->n_unique;
+  const uint32_t n = wk.call->n_unique;
   const unsigned stash_hw = tv.st->stash_hw;
   const unsigned long long n_cells = (tv.bucket_mask + 1) * kCellsPerBucket;
   const int lane = threadIdx.x & 31;
   unsigned int n_res = 0;
+  if ((MODE & kLookUp) && vblock == 0 && threadIdx.x == 0 && wk.call->bad_offsets) atomicOr(&tv.st->error_bits, 4u /* MONO_DEV_BAD_OFFSETS */);
   for (uint32_t base = vblock * blockDim.x; base < n; base += vgrid * blockDim.x) {   // block-uniform
     const uint32_t u = base + threadIdx.x;
     const bool active = u < n;
@@ -191,10 +194,11 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
     // that the insertion that follows has nothing to tell the kernels that update rows
     const bool exact = tv.sketch_depth == 0;
     if ((MODE & kCommit) && exact && active && !hit && m >= tv.threshold) need_row = true;
-    const Reservation rv = block_reserve(tv, &sh, need_row, (MODE & kLookUp) && m > 1, (MODE & kCommit) && active && !hit,
+    const Reservation rv = block_reserve(tv, wk.call, &sh, need_row, (MODE & kLookUp) && m > 1, (MODE & kCommit) && active && !hit,
                                          ((MODE & kLookUp) && m > 1) ? m : 0u);
     if (!active) continue;
     if (MODE & kLookUp) {
+      if (m > kSegChunk) register_long(wk, u, m);
       wk.ulen[u] = m;
       wk.useg[u] = rv.seg_start;
       if (!(MODE & kCommit)) { wk.ucell[u] = cell; wk.umeta[u] = meta; }
@@ -211,18 +215,12 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
         else if (rv.row != kNoRow) { low = kResidentBit | kTouchedBit | rv.row; row_word = rv.row | kFreshBit; }
         cell_address(tv, cell, n_cells)->meta = make_meta(now, low);
         wk.urow[u] = row_word;
-        if (row_word != kNoRow) {
-          ++n_res;
-          if (m > kSegChunk) register_long(tv, wk, u, m);
-        }
+        if (row_word != kNoRow) ++n_res;
       } else {
         if (exact) {
           const uint32_t row_word = rv.row != kNoRow ? (rv.row | kFreshBit) : kNoRow;
           wk.urow[u] = row_word;
-          if (row_word != kNoRow) {
-            ++n_res;
-            if (m > kSegChunk) register_long(tv, wk, u, m);
-          }
+          if (row_word != kNoRow) ++n_res;
         }
         if (MONO_INDEX_OK(wk.error_bits, rv.ins_pos, wk.max_ids)) wk.ins_list[rv.ins_pos] = u;
       }
@@ -321,11 +319,48 @@ __device__ inline void cuckoo_insert(const TableView& tv, Cell item) {
   if (meta_resident(item.meta)) atomicAdd(&tv.st->n_resident, (unsigned long long)(-1LL));
 }
 
+// End of a mono_apply_grads call: fold the per-call counters into the totals and zero them
+// (commit = 0: a grouping that was prepared but never applied is only forgotten).  One block.
+__device__ inline void close_call(DevState* st, const Work& wk, int commit) {
+  CallState* call = wk.call;
+  const bool had_parts = call->longs != 0ull;
+  __syncthreads();                                   // everyone has read the counters before they are reset
+  if (had_parts)
+    for (uint32_t i = threadIdx.x; i < 2 * kWindows; i += blockDim.x) wk.win_count[i] = 0;
+  if (threadIdx.x == 0) {
+    if (commit) {
+      st->sum_ids += call->n_valid_ids;
+      st->sum_unique += call->n_unique;
+      st->sum_new += call->n_insert;
+    }
+    CallState zero = {};
+    *call = zero;
+  }
+}
+__global__ void forget_call_kernel(DevState* st, Work wk) { after_previous_kernel();
+  if (blockIdx.x == 0) close_call(st, wk, 0);
+}
+
+// A push ends with two kernels that need not follow one another, the insertions and the row updates.
+// Every block of both ends with this; the last of all `total` blocks closes the call.
+__device__ inline void block_done(DevState* st, const Work& wk, uint32_t total) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(&wk.call->blocks_done, 1u) == total - 1u;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  close_call(st, wk, 1);
+}
+
 // Probabilistic filter, between phases 2 and 3: every distinct ID that is not in the key
 // store adds its multiplicity to one counter per sketch row.  All additions of a batch are
 // done before any estimate is read (next kernel), so the outcome does not depend on order.
 __device__ inline void sketch_add_body(const TableView& tv, const Work& wk, uint32_t vblock, uint32_t vgrid) {
-  const uint32_t n = tv.st->n_insert;
+  const uint32_t n = wk.call->n_insert;
   const uint32_t stride = vgrid * blockDim.x;
   for (uint32_t i = vblock * blockDim.x + threadIdx.x; i < n; i += stride) {
     const uint32_t u = wk.ins_list[i];
@@ -344,7 +379,7 @@ sketch_add_kernel(TableView tv, Work wk) { after_previous_kernel(); sketch_add_b
 // only if its sketch estimate has reached the threshold; otherwise nothing is stored for it.
 __device__ inline void table_insert_body(const TableView& tv, const Work& wk, uint32_t now, uint32_t vblock, uint32_t vgrid) {
   __shared__ BlockAlloc sh;
-  const uint32_t n = tv.st->n_insert;
+  const uint32_t n = wk.call->n_insert;
   const int lane = threadIdx.x & 31;
   const bool sketch = tv.sketch_depth != 0;
   unsigned int n_res = 0, n_done = 0;
@@ -360,14 +395,11 @@ __device__ inline void table_insert_body(const TableView& tv, const Work& wk, ui
         count = est < tv.threshold ? est : tv.threshold;
       }
       const bool need_row = todo && count >= tv.threshold;
-      const Reservation rv = block_reserve(tv, &sh, need_row, false, false, 0u);
+      const Reservation rv = block_reserve(tv, wk.call, &sh, need_row, false, false, 0u);
       if (!todo) continue;
       if (rv.row != kNoRow) row_word = rv.row | kFreshBit;
       wk.urow[u] = row_word;
-      if (row_word != kNoRow) {
-        ++n_res;
-        if (m > kSegChunk) register_long(tv, wk, u, m);
-      }
+      if (row_word != kNoRow) ++n_res;
       if (row_word == kNoRow) continue;                // below the estimate (or no row left): not stored
     } else {
       if (!todo) continue;
@@ -391,45 +423,38 @@ __device__ inline void table_insert_body(const TableView& tv, const Work& wk, ui
   }
 }
 __global__ void __launch_bounds__(256)
-table_insert_kernel(TableView tv, Work wk, uint32_t now) { after_previous_kernel();
+table_insert_kernel(TableView tv, Work wk, uint32_t now, uint32_t total_blocks) { after_previous_kernel();
   table_insert_body(tv, wk, now, blockIdx.x, gridDim.x);
+  block_done(tv.st, wk, total_blocks);
 }
 
-// Window of the batch that part k of a segment of `parts` parts falls into.  A segment lists
-// its occurrences roughly in batch order (tile by tile), so part k of n covers roughly the
-// k-th n-th of the bags.
-__device__ inline uint32_t part_window(uint32_t k, uint32_t parts) {
-  return (uint32_t)(((unsigned long long)k * kWindows) / parts);
-}
-
-// After phases 2 and 3: every part of a long segment learns which ID it belongs to
-// (one block per long ID, its threads share the parts), and the parts are counted by window.
-__device__ inline void expand_parts_body(const TableView& tv, const Work& wk, uint32_t vblock, uint32_t vgrid) {
-  uint32_t n_long = tv.st->n_long;
-  if (n_long > wk.max_long) n_long = wk.max_long;
-  for (uint32_t li = vblock; li < n_long; li += vgrid) {
+// Every part of a long segment learns which ID it belongs to (one block per long ID, its threads
+// share the parts), and the parts are counted by window.  Only for order_parts_kernel.
+__global__ void __launch_bounds__(128)
+expand_parts_kernel(Work wk) {
+  after_previous_kernel();
+  const uint32_t n_long = (uint32_t)(wk.call->longs >> 32);
+  for (uint32_t li = blockIdx.x; li < n_long; li += gridDim.x) {
     const uint32_t parts = (wk.ulen[wk.long_u[li]] + kSegChunk - 1) / kSegChunk;
     const uint32_t p0 = wk.long_part0[li];
-    if (p0 + parts > wk.max_parts) continue;
     for (uint32_t p = threadIdx.x; p < parts; p += blockDim.x) {
       wk.part_u[p0 + p] = li;
       atomicAdd(&wk.win_count[part_window(p, parts)], 1u);
     }
   }
 }
-__global__ void __launch_bounds__(128)
-expand_parts_kernel(TableView tv, Work wk) { after_previous_kernel(); expand_parts_body(tv, wk, blockIdx.x, gridDim.x); }
 
 // The order the parts are reduced in: window by window, so that the parts in flight at any
 // time -- of different IDs -- gather gradient rows of the same stretch of bags, and a row
 // that several hot IDs need is fetched from DRAM once and found in L2 by the others.
 // Every block scans the window counts for itself; positions inside a window are handed out
 // by a per-window cursor (their order does not matter: each part has its own partial sum).
-__device__ inline void order_parts_body(const TableView& tv, const Work& wk, uint32_t vblock, uint32_t vgrid) {
+// Only for batches whose gradients do not stay in L2 anyway (orders_parts() on the host); needs
+// nothing but the look-ups, so it runs beside the pull.
+__device__ inline void order_parts_body(const Work& wk, uint32_t vblock, uint32_t vgrid) {
   __shared__ uint32_t s_start[kWindows];
   __shared__ uint32_t s_warp[kWindows / 32];
-  uint32_t n_parts = tv.st->n_parts;
-  if (n_parts > wk.max_parts) n_parts = wk.max_parts;
+  const uint32_t n_parts = (uint32_t)wk.call->longs;
   if (n_parts == 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t c = wk.win_count[threadIdx.x];
@@ -455,29 +480,7 @@ __device__ inline void order_parts_body(const TableView& tv, const Work& wk, uin
   }
 }
 __global__ void __launch_bounds__(kWindows)
-order_parts_kernel(TableView tv, Work wk) { after_previous_kernel(); order_parts_body(tv, wk, blockIdx.x, gridDim.x); }
-
-// End of a mono_apply_grads call: fold the per-call counters into the totals
-// (commit = 0: a grouping that was prepared but never applied is only forgotten).
-// (one block)
-__device__ inline void finish_apply_body(DevState* st, uint32_t* win_count, int commit) {
-  const bool had_parts = st->n_parts != 0;
-  __syncthreads();                                   // everyone has read n_parts before it is reset
-  if (had_parts)
-    for (uint32_t i = threadIdx.x; i < 2 * kWindows; i += blockDim.x) win_count[i] = 0;
-  if (threadIdx.x == 0) {
-    if (commit) {
-      st->sum_ids += st->n_valid_ids;
-      st->sum_unique += st->n_unique;
-      st->sum_new += st->n_insert;
-    }
-    st->n_unique = 0; st->n_insert = 0; st->n_long = 0; st->n_parts = 0; st->n_folds = 0; st->n_valid_ids = 0;
-    st->seg_cursor = 0; st->n_multi = 0; st->call_bad_offsets = 0;
-  }
-}
-__global__ void finish_apply_kernel(DevState* st, uint32_t* win_count, int commit) { after_previous_kernel();
-  if (blockIdx.x == 0) finish_apply_body(st, win_count, commit);
-}
+order_parts_kernel(Work wk) { after_previous_kernel(); order_parts_body(wk, blockIdx.x, gridDim.x); }
 
 // Expiry sweep (Section 2.1, heuristic 2): a streaming pass over the key
 // store; a cell whose ID has been inactive for longer than ttl is emptied and
@@ -594,19 +597,6 @@ __device__ inline void expire_body(const TableView& tv, unsigned long long first
 __global__ void __launch_bounds__(256)
 expire_kernel(TableView tv, unsigned long long first_bkt, unsigned long long last_bkt, int with_stash, long long now) { after_previous_kernel();
   expire_body(tv, first_bkt, last_bkt, with_stash != 0, now, blockIdx.x, gridDim.x);
-}
-
-// A batch that was grouped beside the table's other work is taken over: the counters its
-// grouping left in a block of their own become the call's counters.
-__global__ void adopt_group_kernel(DevState* st, DevState* side) {
-  after_previous_kernel();
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->n_unique = side->n_unique;
-    st->n_valid_ids = side->n_valid_ids;
-    st->call_bad_offsets = side->call_bad_offsets;
-    if (side->error_bits) atomicOr(&st->error_bits, side->error_bits);
-    side->n_unique = 0; side->n_valid_ids = 0; side->call_bad_offsets = 0; side->error_bits = 0;
-  }
 }
 
 // After a sweep: if the stash has become empty, probes may skip it again.

@@ -31,15 +31,13 @@ using namespace mono;
 static __device__ __align__(256) uint32_t g_noalloc_occ_row[MONO_NOALLOC_MAX_IDS];
 
 enum KernelId {
-  K_POOL, K_FILL_BAG, K_DEDUP, K_LOOKUP, K_UPDATE, K_SKETCH, K_INSERT, K_EXPAND, K_ORDER, K_FILE, K_SINGLES, K_REDUCE, K_FOLD, K_COMBINE, K_FINISH, K_EXPIRE,
-  K_STASH_TRIM, K_CLEAR, K_REDUCE_PARTS, K_ADOPT, K_COUNT
+  K_POOL, K_FILL_BAG, K_DEDUP, K_LOOKUP, K_UPDATE, K_SKETCH, K_INSERT, K_EXPAND, K_ORDER, K_FILE, K_ROWS, K_EXPIRE, K_STASH_TRIM, K_COUNT
 };
 // (gather_pool: either of the two pooling kernels; table_lookup and table_update are the two halves of table_update_kernel; a push that was not
 // announced runs both in one launch, counted as table_update)
 static const char* const kKernelNames[K_COUNT] = {
-  "gather_pool", "fill_occ_bag", "dedup_tile", "table_lookup", "table_update", "sketch_add", "table_insert", "expand_parts", "order_parts",
-  "file_segments", "update_singletons", "reduce_adagrad", "fold_partials", "combine_adagrad",
-  "finish_apply", "expire", "stash_trim", "clear_set", "reduce_parts", "adopt_group"
+  "gather_pool", "fill_occ_bag", "dedup_tile", "table_lookup", "table_update", "sketch_add", "table_insert", "expand_parts", "order_parts", "file_segments",
+  "update_rows", "expire", "stash_trim"
 };
 static_assert(K_COUNT <= MONO_MAX_KERNELS, "mono_timing_t has room for MONO_MAX_KERNELS kernels");
 
@@ -56,8 +54,7 @@ struct mono_table {
   cudaStream_t stream = nullptr;
   // An internal stream, ordered against `stream` with events only, runs the sweep.
   cudaStream_t sweep_stream = nullptr;
-  // A third one runs the small kernels that serve only the few hottest IDs of a push beside
-  // the large ones (see launch_apply).
+  // A third one puts the parts of the long segments in order beside the pull (see launch_order).
   cudaStream_t aux_stream = nullptr;
   cudaEvent_t ev_aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_keys = nullptr, ev_swept = nullptr, ev_commit = nullptr;
@@ -66,14 +63,14 @@ struct mono_table {
   bool keys_idle = false;         // nothing launched on `stream` after ev_keys touches the key store
   // The batch mono_prepare_push announced: grouped and looked up, waiting for its push.
   // filed: its lookup has run too, so every occurrence's bag is in bag_of_sorted[] already.
-  struct { const void* ids; int64_t n_ids; const void* off; int64_t n_bags; bool valid; bool filed; } prep = {nullptr, 0, nullptr, 0, false, false};
+  struct { const void* ids; int64_t n_ids; const void* off; int64_t n_bags; bool valid; bool filed; bool ordered; } prep = {nullptr, 0, nullptr, 0, false, false, false};
   // The batch mono_group_ahead grouped beside the table's other work: a second copy of the scratch
   // that the grouping fills (the per-call set, the per-occurrence records, the list of distinct
-  // IDs) and of the per-call counters, which mono_prepare_push of the same batch swaps in.
+  // IDs, the per-call counters), which mono_prepare_push of the same batch swaps in.
   struct {
     BatchSlot* bset = nullptr; uint2* occ = nullptr; uint32_t* occ_bag = nullptr;
     unsigned long long* uid = nullptr; uint32_t* uslot = nullptr; uint32_t* uocc = nullptr;
-    DevState* st = nullptr;
+    CallState* call = nullptr;
     const void* ids = nullptr; int64_t n_ids = 0; const void* off = nullptr; int64_t n_bags = 0;
     bool valid = false;           // holds a grouped batch that no mono_prepare_push has taken yet
   } ahead;
@@ -160,10 +157,10 @@ void free_scratch(mono_table* t) {
   Work& w = t->wk;
   dev_free(w.bset); dev_free(w.occ); dev_free(w.occ_bag); dev_free(w.bag_of_sorted);
   dev_free(w.uid); dev_free(w.uslot); dev_free(w.uocc); dev_free(w.useg); dev_free(w.ulen); dev_free(w.urow); dev_free(w.ucell); dev_free(w.umeta);
-  dev_free(w.multi_list); dev_free(w.ins_list); dev_free(w.long_u); dev_free(w.long_part0); dev_free(w.part_u); dev_free(w.part_order); dev_free(w.win_count); dev_free(w.partials); dev_free(w.fold_li); dev_free(w.fold_idx);
+  dev_free(w.multi_list); dev_free(w.ins_list); dev_free(w.long_u); dev_free(w.long_part0); dev_free(w.part_u); dev_free(w.part_order); dev_free(w.win_count); dev_free(w.partials); dev_free(w.part_done); dev_free(w.call);
   dev_free(t->stage_ids); dev_free(t->stage_off); dev_free(t->stage_out); dev_free(t->stage_grad); dev_free(t->occ_row);
   auto& ah = t->ahead;
-  dev_free(ah.bset); dev_free(ah.occ); dev_free(ah.occ_bag); dev_free(ah.uid); dev_free(ah.uslot); dev_free(ah.uocc); dev_free(ah.st);
+  dev_free(ah.bset); dev_free(ah.occ); dev_free(ah.occ_bag); dev_free(ah.uid); dev_free(ah.uslot); dev_free(ah.uocc); dev_free(ah.call);
   ah.valid = false;
   t->staged.valid = false;
   t->max_ids = t->max_bags = 0;
@@ -231,8 +228,9 @@ int discard_prepared(mono_table* t) {
   if (!t->prep.valid) return MONO_OK;
   t->prep.valid = false;
   const uint64_t slots = (uint64_t)t->wk.primary_mask + 1 + (uint64_t)t->wk.secondary_mask + 1;
+  if (t->prep.ordered) CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_aux, 0));
   init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(t->wk.bset, slots);
-  finish_apply_kernel<<<1, 256, 0, t->stream>>>(t->tv.st, t->wk.win_count, 0);
+  forget_call_kernel<<<1, 256, 0, t->stream>>>(t->tv.st, t->wk);
   CUDA_TRY(t, cudaGetLastError());
   return MONO_OK;
 }
@@ -249,8 +247,8 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   if (t->h2d_stream) CUDA_TRY(t, cudaStreamSynchronize(t->h2d_stream));      // copies in flight use the staging buffers
   if (t->d2h_stream) CUDA_TRY(t, cudaStreamSynchronize(t->d2h_stream));
   t->d2h_pending = false;
-  // a prepared batch is lost with the scratch it lives in
-  if (t->prep.valid) { t->prep.valid = false; finish_apply_kernel<<<1, 256, 0, t->stream>>>(t->tv.st, t->wk.win_count, 0); }
+  CUDA_TRY(t, cudaStreamSynchronize(t->aux_stream));
+  t->prep.valid = false;                                   // a prepared batch is lost with the scratch it lives in
   free_scratch(t);
   Work& w = t->wk;
   const size_t n = (size_t)max_ids;
@@ -272,8 +270,7 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   w.max_parts = (uint32_t)(2 * (n / kSegChunk) + 2);
   ALLOC(w.long_u, w.max_long); ALLOC(w.long_part0, w.max_long); ALLOC(w.part_u, w.max_parts); ALLOC(w.part_order, w.max_parts); ALLOC(w.win_count, 2 * kWindows);
   ALLOC(w.partials, (size_t)w.max_parts * t->tv.dim);
-  w.max_folds = w.max_parts / kFoldWidth + w.max_long + 1;
-  ALLOC(w.fold_li, w.max_folds); ALLOC(w.fold_idx, w.max_folds);
+  ALLOC(w.part_done, w.max_parts); ALLOC(w.call, 1);
   ALLOC(t->stage_ids, n); ALLOC(t->stage_off, (size_t)max_bags + 1);
   // (the two staging buffers of the host-buffer calls, one bag-by-dim matrix each, are allocated by the
   // first such call: callers that keep their batches on the device never pay for them)
@@ -287,6 +284,8 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(w.bset, slots);
   CUDA_TRY(t, cudaGetLastError());
   CUDA_TRY(t, cudaMemsetAsync(w.win_count, 0, 2 * kWindows * sizeof(uint32_t), t->stream));
+  CUDA_TRY(t, cudaMemsetAsync(w.part_done, 0, w.max_parts * sizeof(uint32_t), t->stream));
+  CUDA_TRY(t, cudaMemsetAsync(w.call, 0, sizeof(CallState), t->stream));
   t->max_ids = max_ids;
   t->max_bags = max_bags;
   return MONO_OK;
@@ -371,18 +370,63 @@ int launch_lookup(mono_table* t, const unsigned long long* ids, int64_t n_ids, c
   return rc;
 }
 
+uint32_t lane_class_of(uint32_t dim) {
+  return dim <= 16 ? 0u : dim <= 32 ? 1u : dim <= 64 ? 2u : dim <= 128 ? 3u : dim <= 256 ? 4u : dim <= 512 ? 5u : 6u;
+}
+int lanes_of_class(uint32_t c) { return c == 0 ? 4 : c == 1 ? 8 : c == 2 ? 16 : 32; }
+
+// Blocks for `work` items of which a block takes `per_block` in one trip, at most `cap`.
+int64_t clamp_blocks(int64_t work, int64_t per_block, int64_t cap) {
+  int64_t b = (work + per_block - 1) / per_block;
+  if (b < 1) b = 1;
+  return b > cap ? cap : b;
+}
+
 // The part of a push that depends on the IDs alone: bag of every occurrence, and the
 // occurrences grouped by ID in the per-call set.
 int launch_group(mono_table* t, cudaStream_t s, const unsigned long long* ids, int64_t n_ids, const long long* off,
-                 int64_t n_bags, const Work* into = nullptr, DevState* counters = nullptr) {
-  const TableView& tv = t->tv;
-  const Work& wk = into ? *into : t->wk;
-  DevState* st = counters ? counters : tv.st;
-  LAUNCH_ON(t, s, K_FILL_BAG, launch_after(fill_occ_bag_kernel, grid_for(t, 8), 256, s, off, n_bags, n_ids, wk.occ_bag, st));
+                 int64_t n_bags, const Work& wk) {
+  LAUNCH_ON(t, s, K_FILL_BAG, launch_after(fill_occ_bag_kernel, (unsigned)clamp_blocks(n_bags, 256, grid_for(t, 8)), 256, s, off, n_bags, n_ids, wk.occ_bag, wk.call));
   const int tiles = (int)((n_ids + kTileIds - 1) / kTileIds);
-  LAUNCH_ON(t, s, K_DEDUP, launch_after(dedup_tile_kernel, tiles, kTileThreads, s, wk, ids, n_ids, off, n_bags, st,
-                                                                          tv.seed0 ^ 0xA5A5A5A55A5A5A5Aull));
+  LAUNCH_ON(t, s, K_DEDUP, launch_after(dedup_tile_kernel, tiles, kTileThreads, s, wk, ids, n_ids, off, n_bags, t->tv.seed0 ^ 0xA5A5A5A55A5A5A5Aull));
   CUDA_TRY(t, cudaGetLastError());
+  return MONO_OK;
+}
+
+// Whether the parts of long segments are put in order of the batch's windows: where the gradients do not
+// fit L2, that lets the parts of different IDs find each other's gradient rows there (1.6 M bags of 64
+// columns: 0.34 GB less read from DRAM); where they do, it would be work for nothing.
+bool orders_parts(const mono_table* t, int64_t n_bags) { return n_bags * (int64_t)t->tv.dim * 4 > (int64_t)64 << 20; }
+
+unsigned update_grid(const mono_table* t, int64_t n_ids) { return (unsigned)clamp_blocks(n_ids, 256, grid_for(t, 8) * 4); }
+unsigned insert_grid(const mono_table* t, int64_t n_ids) { return (unsigned)clamp_blocks(n_ids, 256, grid_for(t, 8)); }
+// Blocks of the row updates for a batch that has `share` of the GPU (1, or its part of a grouped call).  The host
+// only knows how many IDs there are, so every share of the grid is sized for a long-tailed batch (a part per 64 IDs,
+// an ID in 64 with a short segment per lane group, one in four that occurs once per thread), and loops where that
+// was too few: blocks that find nothing to do cost 1 ns each, 20 us of a step with eight waves of them on 1 M IDs.
+// While the batch is small enough for all of its blocks to be resident, it is spread as far as it goes instead.
+RowGrid rows_grid(const mono_table* t, int64_t n_ids, double share = 1.0) {
+  const int64_t groups = kRowThreads / lanes_of_class(lane_class_of(t->tv.dim)), wave = grid_for(t, 8), cap = wave * 8;
+  const auto blocks = [&](int64_t most, int64_t typical, int64_t per, double resident) {
+    return (uint32_t)clamp_blocks(most, per, std::max({std::min(cap, (typical + per - 1) / per), (int64_t)(resident * share), (int64_t)1}));
+  };
+  return {blocks(n_ids / 64, n_ids / 64, groups, 1.0), blocks(n_ids / 2, n_ids / 64, groups, (double)wave),
+          blocks(n_ids, n_ids / 4, kRowThreads, 2.0 * (double)wave)};
+}
+uint32_t blocks_of(const RowGrid& g) { return g.parts + g.shorts + g.singles; }
+
+// After the look-ups of a batch: its parts in order, on a stream of their own, beside the pull and the
+// first half of the push.  (While kernels are being timed one by one, everything stays on the table's stream.)
+int launch_order(mono_table* t) {
+  cudaStream_t s = t->stream, a = t->timing ? s : t->aux_stream;
+  if (a != s) {
+    CUDA_TRY(t, cudaEventRecord(t->ev_fork, s));
+    CUDA_TRY(t, cudaStreamWaitEvent(a, t->ev_fork, 0));
+  }
+  LAUNCH_ON(t, a, K_EXPAND, launch_after(expand_parts_kernel, grid_for(t, 8) * 4, 128, a, t->wk));
+  LAUNCH_ON(t, a, K_ORDER, launch_after(order_parts_kernel, 64, kWindows, a, t->wk));
+  CUDA_TRY(t, cudaGetLastError());
+  CUDA_TRY(t, cudaEventRecord(t->ev_aux, a));
   return MONO_OK;
 }
 
@@ -390,105 +434,78 @@ int launch_group(mono_table* t, cudaStream_t s, const unsigned long long* ids, i
 // push of this batch together.  Nothing in the table changes.
 int launch_prepare(mono_table* t, const unsigned long long* ids, int64_t n_ids, const long long* off, int64_t n_bags) {
   auto& ah = t->ahead;
+  Work& w = t->wk;
   if (ah.valid && ah.ids == ids && ah.n_ids == n_ids && ah.off == off && ah.n_bags == n_bags) {
-    // grouped already, beside the table's other work: the two copies of the grouping scratch change
-    // places, and the counters the grouping left come over
+    // grouped already, beside the table's other work: the two copies of the grouping scratch change places
     ah.valid = false;
     CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_ahead, 0));        // (recorded when the grouping ran on a stream of its own)
-    Work& w = t->wk;
     std::swap(w.bset, ah.bset); std::swap(w.occ, ah.occ); std::swap(w.occ_bag, ah.occ_bag);
-    std::swap(w.uid, ah.uid); std::swap(w.uslot, ah.uslot); std::swap(w.uocc, ah.uocc);
-    LAUNCH(t, K_ADOPT, launch_after(adopt_group_kernel, 1, 32, t->stream, t->tv.st, ah.st));
-    CUDA_TRY(t, cudaGetLastError());
+    std::swap(w.uid, ah.uid); std::swap(w.uslot, ah.uslot); std::swap(w.uocc, ah.uocc); std::swap(w.call, ah.call);
   } else {
-    const int rc = launch_group(t, t->stream, ids, n_ids, off, n_bags);
+    const int rc = launch_group(t, t->stream, ids, n_ids, off, n_bags, w);
     if (rc != MONO_OK) return rc;
   }
-  LAUNCH(t, K_LOOKUP, launch_after(table_update_kernel<kLookUp>, grid_for(t, 8) * 4, 256, t->stream, t->tv, t->wk, 0u));
+  const bool ordered = orders_parts(t, n_bags);
+  LAUNCH(t, K_LOOKUP, launch_after(table_update_kernel<kLookUp>, update_grid(t, n_ids), 256, t->stream, t->tv, w, 0u));
   CUDA_TRY(t, cudaGetLastError());
-  return MONO_OK;
+  t->prep = {ids, n_ids, off, n_bags, true, false, ordered};
+  return ordered ? launch_order(t) : (int)MONO_OK;
 }
 
-// grad_ready: if not null, the gradients are still being copied in; the kernels that read them wait for it
+// grad_ready: if not null, the gradients are still being copied in; the kernel that reads them waits for it
 int launch_apply(mono_table* t, const unsigned long long* ids, int64_t n_ids, const long long* off,
                  int64_t n_bags, const float* grad, uint32_t now, cudaEvent_t grad_ready = nullptr) {
   cudaStream_t s = t->stream;
   const TableView& tv = t->tv;
   const Work& wk = t->wk;
-  // grids of the grid-stride kernels: several waves of blocks per SM where that measured faster
-  // (shorter tails), one wave elsewhere.  The reduction of the short segments runs beside the long
-  // segments' chain and the insertions: with four waves of blocks instead of eight the step measured
-  // 1.9 % faster on the largest configuration (its own time is the same); the parts launch and
-  // update_singletons keep eight.
-  const int g4 = grid_for(t, 4), g8 = grid_for(t, 8);
-  int rc0 = MONO_OK;
+  int rc = MONO_OK;
+  bool ordered;
   if (is_prepared_batch(t, ids, n_ids, off, n_bags)) {
     // grouped and looked up already; filed too, if its lookup has run
     t->prep.valid = false;
-    if (!t->prep.filed) LAUNCH(t, K_FILE, launch_after(file_segments_kernel, g8, 256, s, wk, n_ids, n_bags));
-    LAUNCH(t, K_UPDATE, launch_after(table_update_kernel<kCommit>, g8 * 4, 256, s, tv, wk, now));
+    ordered = t->prep.ordered;
+    if (!t->prep.filed) LAUNCH(t, K_FILE, launch_after(file_segments_kernel, insert_grid(t, n_ids), 256, s, wk, n_ids, n_bags));
+    LAUNCH(t, K_UPDATE, launch_after(table_update_kernel<kCommit>, update_grid(t, n_ids), 256, s, tv, wk, now));
   } else {
-    if ((rc0 = discard_prepared(t)) != MONO_OK) return rc0;
+    if ((rc = discard_prepared(t)) != MONO_OK) return rc;
     if (n_ids == 0 || n_bags == 0) return MONO_OK;
-    if ((rc0 = launch_group(t, s, ids, n_ids, off, n_bags)) != MONO_OK) return rc0;
-    LAUNCH(t, K_UPDATE, launch_after(table_update_kernel<kLookUp | kCommit>, g8 * 4, 256, s, tv, wk, now));
-    LAUNCH(t, K_FILE, launch_after(file_segments_kernel, g8, 256, s, wk, n_ids, n_bags));
+    if ((rc = launch_group(t, s, ids, n_ids, off, n_bags, wk)) != MONO_OK) return rc;
+    ordered = orders_parts(t, n_bags);
+    LAUNCH(t, K_UPDATE, launch_after(table_update_kernel<kLookUp | kCommit>, update_grid(t, n_ids), 256, s, tv, wk, now));
+    if (ordered && (rc = launch_order(t)) != MONO_OK) return rc;
+    LAUNCH(t, K_FILE, launch_after(file_segments_kernel, insert_grid(t, n_ids), 256, s, wk, n_ids, n_bags));
   }
-  // The long segments (the few hottest IDs) are reduced on a stream of their own -- expand,
-  // order, the parts, fold, combine, one after the other with no event in between -- beside
-  // the kernels that work through the rest of the batch on the table's stream: the reduction
-  // of the short segments and update_singletons.  The two chains touch different rows and meet
-  // again before the call's last kernel (measured 0.9 % of a step faster than the parts on the
-  // table's stream between two event waits).  With the exact filter the insertion of the new
-  // IDs runs on a third stream beside both: their rows were settled by the commit half, so the
-  // row updates do not wait for it.  With the probabilistic filter it is the insertion that
-  // decides the rows, and it stays on the table's stream.
-  // While kernels are being timed one by one, everything stays on the table's stream.
-  cudaStream_t a = t->timing ? s : t->aux_stream;
-  const bool insert_aside = a != s && tv.sketch_depth == 0;
+  // Two kernels are left: the insertion of the new IDs and the row updates.  With the exact filter the
+  // rows of new IDs were settled by the commit half, so nothing in the row updates waits for the
+  // insertion, which runs beside them on the stream the sweep uses: a sweep that follows this call
+  // follows the insertions.  With the probabilistic filter it is the insertion that decides the rows,
+  // and it stays on the table's stream.  Whichever kernel ends last closes the call.
+  const bool insert_aside = !t->timing && tv.sketch_depth == 0;
+  const unsigned insert_blocks = insert_grid(t, n_ids);
+  const RowGrid row_grid = rows_grid(t, n_ids);
+  const unsigned total = insert_blocks + blocks_of(row_grid);
+  cudaStream_t k = insert_aside ? t->sweep_stream : s;
   if (insert_aside) {
-    // (on the stream the sweep uses: a sweep slice that follows this call follows the insertions)
-    cudaStream_t k = t->sweep_stream;
     CUDA_TRY(t, cudaEventRecord(t->ev_commit, s));
     CUDA_TRY(t, cudaStreamWaitEvent(k, t->ev_commit, 0));
-    CUDA_TRY(t, cudaStreamWaitEvent(a, t->ev_commit, 0));
-    LAUNCH_ON(t, k, K_INSERT, launch_after(table_insert_kernel, g8, 256, k, tv, wk, now));
-    CUDA_TRY(t, cudaGetLastError());
-    // the rest of the call touches rows and scratch only: a sweep may run beside it
-    CUDA_TRY(t, cudaEventRecord(t->ev_keys, k));
-  } else {
-    if (tv.sketch_depth) LAUNCH(t, K_SKETCH, launch_after(sketch_add_kernel, g8, 256, s, tv, wk));
-    LAUNCH(t, K_INSERT, launch_after(table_insert_kernel, g8, 256, s, tv, wk, now));
-    CUDA_TRY(t, cudaGetLastError());
-    CUDA_TRY(t, cudaEventRecord(t->ev_keys, s));
-    if (a != s) CUDA_TRY(t, cudaStreamWaitEvent(a, t->ev_keys, 0));
+  } else if (tv.sketch_depth) {
+    LAUNCH(t, K_SKETCH, launch_after(sketch_add_kernel, insert_blocks, 256, s, tv, wk));
   }
-  // (nobody reads the per-call set after the key-store work: its primary tier is wiped beside the rest)
-  LAUNCH_ON(t, a, K_CLEAR, launch_after(clear_primary_kernel, g8, 256, a, wk));
-  LAUNCH_ON(t, a, K_EXPAND, launch_after(expand_parts_kernel, g8 * 4, 128, a, tv, wk));
-  LAUNCH_ON(t, a, K_ORDER, launch_after(order_parts_kernel, 64, kWindows, a, tv, wk));
+  LAUNCH_ON(t, k, K_INSERT, launch_after(table_insert_kernel, insert_blocks, 256, k, tv, wk, now, total));
   CUDA_TRY(t, cudaGetLastError());
+  // the rest of the call touches rows and scratch only: a sweep may run beside it
+  CUDA_TRY(t, cudaEventRecord(t->ev_keys, k));
+  if (ordered) CUDA_TRY(t, cudaStreamWaitEvent(s, t->ev_aux, 0));
   if (grad_ready) CUDA_TRY(t, cudaStreamWaitEvent(s, grad_ready, 0));
-  const int rc = dispatch_dim(tv.dim, [&](auto g, auto nv) -> int {
+  rc = dispatch_dim(tv.dim, [&](auto g, auto nv) -> int {
     constexpr int G = decltype(g)::value, NV = decltype(nv)::value;
-    LAUNCH(t, K_REDUCE, launch_after(reduce_adagrad_kernel<G, NV>, g8 * 4, 128, s, tv, wk, grad, n_bags, kReduceShort));
-    if (grad_ready && a != s) CUDA_TRY(t, cudaStreamWaitEvent(a, grad_ready, 0));
-    LAUNCH_ON(t, a, K_REDUCE_PARTS, launch_after(reduce_adagrad_kernel<G, NV>, g8 * 8, 128, a, tv, wk, grad, n_bags, kReduceParts));
-    LAUNCH(t, K_SINGLES, launch_after(update_singletons_kernel<G, NV>, g8 * 8, 128, s, tv, wk, grad, n_bags));
+    LAUNCH(t, K_ROWS, launch_after(update_rows_kernel<G, NV>, blocks_of(row_grid), kRowThreads, s, tv, wk, grad, n_bags, (int)ordered, row_grid, total));
     return (int)MONO_OK;
   });
-  if (rc != MONO_OK) return rc;
-  LAUNCH_ON(t, a, K_FOLD, launch_after(fold_partials_kernel, g4, 256, a, tv, wk));
-  LAUNCH_ON(t, a, K_COMBINE, launch_after(combine_adagrad_kernel, g8, kCombineThreads, a, tv, wk));
-  if (a != s) {
-    CUDA_TRY(t, cudaEventRecord(t->ev_aux, a));
-    CUDA_TRY(t, cudaStreamWaitEvent(s, t->ev_aux, 0));
-  }
-  if (insert_aside) CUDA_TRY(t, cudaStreamWaitEvent(s, t->ev_keys, 0));
-  LAUNCH(t, K_FINISH, launch_after(finish_apply_kernel, 1, 256, s, tv.st, wk.win_count, 1));
   CUDA_TRY(t, cudaGetLastError());
+  if (insert_aside) CUDA_TRY(t, cudaStreamWaitEvent(s, t->ev_keys, 0));
   t->keys_idle = true;
-  return MONO_OK;
+  return rc;
 }
 
 int check_now(mono_table* t, int64_t now) {
@@ -499,14 +516,8 @@ int check_now(mono_table* t, int64_t now) {
 // ---- grouped calls: one launch over several tables -------------------------------------------
 
 enum GroupKernel {
-  GK_FILL, GK_DEDUP, GK_UPDATE, GK_INSERT, GK_FILE, GK_EXPAND, GK_ORDER, GK_POOL, GK_POOL_WIDE, GK_REDUCE, GK_REDUCE_WIDE,
-  GK_SINGLES, GK_SINGLES_WIDE, GK_FOLD, GK_COMBINE, GK_CLEAR, GK_COUNT
+  GK_FILL, GK_DEDUP, GK_UPDATE, GK_INSERT, GK_FILE, GK_POOL, GK_POOL_WIDE, GK_ROWS, GK_ROWS_WIDE, GK_COUNT
 };
-
-uint32_t lane_class_of(uint32_t dim) {
-  return dim <= 16 ? 0u : dim <= 32 ? 1u : dim <= 64 ? 2u : dim <= 128 ? 3u : dim <= 256 ? 4u : dim <= 512 ? 5u : 6u;
-}
-int lanes_of_class(uint32_t c) { return c == 0 ? 4 : c == 1 ? 8 : c == 2 ? 16 : 32; }
 
 void free_group_scratch(mono_table* t) {
   auto& g = t->grp;
@@ -517,36 +528,20 @@ void free_group_scratch(mono_table* t) {
   }
 }
 
-int64_t clamp_blocks(int64_t work, int64_t per_block, int64_t cap) {
-  int64_t b = (work + per_block - 1) / per_block;
-  if (b < 1) b = 1;
-  return b > cap ? cap : b;
-}
-
 // Blocks that table `t` contributes to grouped kernel `k` (the grid it would launch alone, but no
 // larger than its batch needs: a group may hold hundreds of small tables).
 uint32_t group_blocks(const mono_table* t, int k, const GroupItem& it) {
   const int64_t n_ids = it.n_ids, n_bags = it.n_bags;
-  const int64_t g8 = grid_for(t, 8), g4 = grid_for(t, 4);
-  const uint32_t lc = lane_class_of(t->tv.dim);
-  const int G = lanes_of_class(lc);
-  const bool wide = lc >= 4;
+  const bool wide = it.lane_class >= 4;
   switch (k) {
-    case GK_FILL: return (uint32_t)clamp_blocks(n_bags, 256, g8);
+    case GK_FILL: return (uint32_t)clamp_blocks(n_bags, 256, grid_for(t, 8));
     case GK_DEDUP: return (uint32_t)((n_ids + kTileIds - 1) / kTileIds);
-    case GK_UPDATE: return (uint32_t)clamp_blocks(n_ids, 256, g8 * 4);
-    case GK_INSERT: case GK_FILE: return (uint32_t)clamp_blocks(n_ids, 256, g8);
-    case GK_EXPAND: return (uint32_t)clamp_blocks(n_ids / kSegChunk + 1, 1, g8 * 4);
-    case GK_ORDER: return (uint32_t)clamp_blocks(n_ids / kSegChunk + 1, kWindows, 64);
+    case GK_UPDATE: return update_grid(t, n_ids);
+    case GK_INSERT: case GK_FILE: return insert_grid(t, n_ids);
     case GK_POOL: return wide ? 0u : (uint32_t)((n_bags + it.tile_bags - 1) / it.tile_bags);
     case GK_POOL_WIDE: return wide ? (uint32_t)((n_bags + it.tile_bags - 1) / it.tile_bags) : 0u;
-    case GK_REDUCE: return wide ? 0u : (uint32_t)clamp_blocks(n_ids / 2 + 1, 128 / G, g8 * 8);
-    case GK_REDUCE_WIDE: return wide ? (uint32_t)clamp_blocks(n_ids / 2 + 1, 128 / G, g8 * 8) : 0u;
-    case GK_SINGLES: return wide ? 0u : (uint32_t)clamp_blocks(n_ids, 128, g8 * 8);
-    case GK_SINGLES_WIDE: return wide ? (uint32_t)clamp_blocks(n_ids, 128, g8 * 8) : 0u;
-    case GK_FOLD: return (uint32_t)clamp_blocks(n_ids / (kSegChunk * kFoldWidth) + 1, 1, g4);
-    case GK_COMBINE: return (uint32_t)clamp_blocks(n_ids / kSegChunk + 1, 1, g8);
-    case GK_CLEAR: return (uint32_t)clamp_blocks((int64_t)t->wk.primary_mask + 1, 2048, g8);
+    case GK_ROWS: return wide ? 0u : blocks_of(it.row_grid);
+    case GK_ROWS_WIDE: return wide ? blocks_of(it.row_grid) : 0u;
     default: return 0u;
   }
 }
@@ -846,14 +841,14 @@ int mono_group_ahead(mono_table* t, const uint64_t* ids, int64_t n_ids, const in
     if (arc == MONO_OK) arc = dev_alloc(t, &ah.uid, n);
     if (arc == MONO_OK) arc = dev_alloc(t, &ah.uslot, n);
     if (arc == MONO_OK) arc = dev_alloc(t, &ah.uocc, n);
-    if (arc == MONO_OK) arc = dev_alloc(t, &ah.st, 1);
+    if (arc == MONO_OK) arc = dev_alloc(t, &ah.call, 1);
     if (arc != MONO_OK) {
-      dev_free(ah.bset); dev_free(ah.occ); dev_free(ah.occ_bag); dev_free(ah.uid); dev_free(ah.uslot); dev_free(ah.uocc); dev_free(ah.st);
+      dev_free(ah.bset); dev_free(ah.occ); dev_free(ah.occ_bag); dev_free(ah.uid); dev_free(ah.uslot); dev_free(ah.uocc); dev_free(ah.call);
       return arc;
     }
     init_bset_kernel<<<grid_for(t, 4), 256, 0, g>>>(ah.bset, slots);
     CUDA_TRY(t, cudaGetLastError());
-    CUDA_TRY(t, cudaMemsetAsync(ah.st, 0, sizeof(DevState), g));
+    CUDA_TRY(t, cudaMemsetAsync(ah.call, 0, sizeof(CallState), g));
     ah.valid = false;
   }
   if (ah.valid) {
@@ -861,13 +856,14 @@ int mono_group_ahead(mono_table* t, const uint64_t* ids, int64_t n_ids, const in
     ah.valid = false;
     init_bset_kernel<<<grid_for(t, 4), 256, 0, g>>>(ah.bset, slots);
     CUDA_TRY(t, cudaGetLastError());
-    CUDA_TRY(t, cudaMemsetAsync(ah.st, 0, sizeof(DevState), g));
+    CUDA_TRY(t, cudaMemsetAsync(ah.call, 0, sizeof(CallState), g));
   }
   if (n_ids == 0 || n_bags == 0) return MONO_OK;
   Work into = w;
   into.bset = ah.bset; into.occ = ah.occ; into.occ_bag = ah.occ_bag; into.uid = ah.uid; into.uslot = ah.uslot; into.uocc = ah.uocc;
+  into.call = ah.call;
   if ((rc = launch_group(t, g, reinterpret_cast<const unsigned long long*>(ids), n_ids,
-                         reinterpret_cast<const long long*>(slot_offsets), n_bags, &into, ah.st)) != MONO_OK) return rc;
+                         reinterpret_cast<const long long*>(slot_offsets), n_bags, into)) != MONO_OK) return rc;
   if (g != t->stream) CUDA_TRY(t, cudaEventRecord(t->ev_ahead, g));
   ah.ids = ids; ah.n_ids = n_ids; ah.off = slot_offsets; ah.n_bags = n_bags;
   ah.valid = true;
@@ -882,10 +878,8 @@ int mono_prepare_push(mono_table* t, const uint64_t* ids, int64_t n_ids, const i
   if ((rc = reserve(t, n_ids, n_bags)) != MONO_OK) return rc;
   if ((rc = discard_prepared(t)) != MONO_OK) return rc;
   if (n_ids == 0 || n_bags == 0) return MONO_OK;
-  if ((rc = launch_prepare(t, reinterpret_cast<const unsigned long long*>(ids), n_ids,
-                           reinterpret_cast<const long long*>(slot_offsets), n_bags)) != MONO_OK) return rc;
-  t->prep = {ids, n_ids, slot_offsets, n_bags, true, false};
-  return MONO_OK;
+  return launch_prepare(t, reinterpret_cast<const unsigned long long*>(ids), n_ids,
+                        reinterpret_cast<const long long*>(slot_offsets), n_bags);
 }
 
 int mono_group_prepare_push(int32_t n_tables, mono_table* const* tables, const uint64_t* const* ids,
@@ -912,7 +906,7 @@ int mono_group_prepare_push(int32_t n_tables, mono_table* const* tables, const u
   GROUP_LAUNCH(p, K_LOOKUP, GK_UPDATE, 256, group_table_update_kernel<kLookUp>);
   CUDA_TRY(p.owner, cudaGetLastError());
   for (int32_t i = 0; i < n_tables; ++i)
-    if (p.items[i].active) tables[i]->prep = {ids[i], n_ids[i], slot_offsets[i], n_bags[i], true, false};
+    if (p.items[i].active) tables[i]->prep = {ids[i], n_ids[i], slot_offsets[i], n_bags[i], true, false, false};
   return group_end(p, tables);
 }
 
@@ -962,6 +956,7 @@ int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const ui
   if (n_tables == 0) return MONO_OK;
   if (!ids || !n_ids || !slot_offsets || !n_bags || !grad_pooled) return MONO_ERR_ARG;
   bool all_prepared = true, all_filed = true;
+  int64_t all_ids = 0;
   for (int32_t i = 0; i < n_tables; ++i) {
     mono_table* t = tables[i];
     join_sweep(t);
@@ -971,6 +966,7 @@ int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const ui
     if ((rc = reserve(t, n_ids[i], n_bags[i])) != MONO_OK) return rc;
     if (n_ids[i] == 0 || n_bags[i] == 0) continue;
     const bool prepared = is_prepared_batch(t, ids[i], n_ids[i], slot_offsets[i], n_bags[i]);
+    if (prepared && t->prep.ordered) CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_aux, 0));     // (announced by a call of its own)
     all_prepared &= prepared;
     all_filed &= prepared && t->prep.filed;
   }
@@ -985,6 +981,11 @@ int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const ui
   if ((rc = group_begin(p, n_tables, tables, group_stream)) != MONO_OK) return rc;
   for (int32_t i = 0; i < n_tables; ++i)
     group_describe(p, i, tables[i], ids[i], n_ids[i], slot_offsets[i], n_bags[i], nullptr, grad_pooled[i], (uint32_t)now, all_prepared);
+  for (int32_t i = 0; i < n_tables; ++i) all_ids += n_ids[i];
+  for (int32_t i = 0; i < n_tables; ++i) {
+    p.items[i].row_grid = rows_grid(tables[i], n_ids[i], (double)n_ids[i] / (double)(all_ids ? all_ids : 1));
+    p.items[i].total_blocks = insert_grid(tables[i], n_ids[i]) + blocks_of(p.items[i].row_grid);
+  }
   if ((rc = group_upload(p, tables)) != MONO_OK) return rc;
   if (all_prepared) {
     if (!all_filed) GROUP_LAUNCH(p, K_FILE, GK_FILE, 256, group_file_segments_kernel);
@@ -996,17 +997,8 @@ int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const ui
   }
   if (p.any_sketch) GROUP_LAUNCH(p, K_SKETCH, GK_INSERT, 256, group_sketch_add_kernel);
   GROUP_LAUNCH(p, K_INSERT, GK_INSERT, 256, group_table_insert_kernel);
-  GROUP_LAUNCH(p, K_CLEAR, GK_CLEAR, 256, group_clear_primary_kernel);
-  GROUP_LAUNCH(p, K_EXPAND, GK_EXPAND, 128, group_expand_parts_kernel);
-  GROUP_LAUNCH(p, K_ORDER, GK_ORDER, kWindows, group_order_parts_kernel);
-  GROUP_LAUNCH(p, K_REDUCE, GK_REDUCE, 128, group_reduce_adagrad_kernel<0>);
-  GROUP_LAUNCH(p, K_REDUCE, GK_REDUCE_WIDE, 128, group_reduce_adagrad_kernel<1>);
-  GROUP_LAUNCH(p, K_SINGLES, GK_SINGLES, 128, group_update_singletons_kernel<0>);
-  GROUP_LAUNCH(p, K_SINGLES, GK_SINGLES_WIDE, 128, group_update_singletons_kernel<1>);
-  GROUP_LAUNCH(p, K_FOLD, GK_FOLD, 256, group_fold_partials_kernel);
-  GROUP_LAUNCH(p, K_COMBINE, GK_COMBINE, kCombineThreads, group_combine_adagrad_kernel);
-  ++p.owner->launches[K_FINISH];
-  launch_after(group_finish_apply_kernel, (unsigned)n_tables, 256, p.gs, p.d_items, (uint32_t)n_tables, 1);
+  GROUP_LAUNCH(p, K_ROWS, GK_ROWS, kRowThreads, group_update_rows_kernel<0>);
+  GROUP_LAUNCH(p, K_ROWS, GK_ROWS_WIDE, kRowThreads, group_update_rows_kernel<1>);
   CUDA_TRY(p.owner, cudaGetLastError());
   for (int32_t i = 0; i < n_tables; ++i) tables[i]->prep.valid = false;
   return group_end(p, tables);
@@ -1155,7 +1147,6 @@ int mono_lookup_pool_host(mono_table* t, const uint64_t* ids, int64_t n_ids, con
   bool prepared = false;
   if (n_ids > 0) {
     if ((rc = launch_prepare(t, t->stage_ids, n_ids, t->stage_off, n_bags)) != MONO_OK) return rc;
-    t->prep = {t->stage_ids, n_ids, t->stage_off, n_bags, true, false};
     t->staged = {ids, n_ids, slot_offsets, n_bags, true};
     prepared = true;
   }

@@ -96,19 +96,23 @@ struct DevState {
   unsigned long long sum_unique_resident;
   unsigned long long sum_new;
   unsigned long long sum_single_resident;
-  // per-call work counters, reset at the end of every mono_apply_grads
-  unsigned int n_unique;
-  unsigned int n_insert;
-  unsigned int n_long;                   // distinct IDs whose segment is split into parts
-  unsigned int n_parts;
-  unsigned int n_folds;                  // groups of kFoldWidth parts that are added up before the final combine
-  unsigned int call_bad_offsets;         // this call's offsets were malformed: occurrences are checked one by one
-  unsigned int n_valid_ids;
-  unsigned int seg_cursor;               // entries of bag_of_sorted[] handed out so far
-  unsigned int n_multi;                  // distinct IDs that occur more than once in the batch
-  unsigned int pad1;
   // export / audit scratch
   unsigned long long export_n;
+};
+
+// Counters of one batch on its way through grouping, look-up and push; all zero between calls.  They
+// belong to the scratch a batch is grouped into, not to the table: a batch that is grouped ahead has a
+// copy of its own, which changes places with the other when its turn comes.
+struct CallState {
+  unsigned long long longs;              // high word: distinct IDs whose segment is reduced in parts; low word: their parts
+  unsigned int n_unique;
+  unsigned int n_insert;
+  unsigned int n_valid_ids;
+  unsigned int n_multi;                  // distinct IDs that occur more than once in the batch
+  unsigned int seg_cursor;               // entries of bag_of_sorted[] handed out so far
+  unsigned int bad_offsets;              // this call's offsets were malformed: occurrences are checked one by one
+  unsigned int blocks_done;              // of the kernels that end a push: the last one closes the call
+  unsigned int pad;
 };
 
 // Checked build (-DMONO_DEBUG): every index the library computes for itself -- a segment
