@@ -78,17 +78,17 @@ __device__ inline void clear_primary(const Work& wk, uint32_t vblock, uint32_t v
   for (uint32_t i = vblock * blockDim.x + threadIdx.x; i < n; i += vgrid * blockDim.x)
     *reinterpret_cast<ulonglong2*>(wk.bset + i) = e;
 }
-// Sum of grad rows of bags bag_of_sorted[begin .. end) for the NV column
-// vectors this lane owns.  Eight independent row loads in flight per step.
-template <int G, int NV>
+// Sum of the grad rows of bags bag_of_sorted[begin], [begin + STEP], ... below end for the NV column
+// vectors this lane owns.  Eight independent row loads in flight per trip.
+template <int G, int NV, int STEP = 1>
 __device__ inline void reduce_segment(const Work& wk, const float* __restrict__ grad, long long n_bags,
                                       uint32_t dim, int gl, uint32_t begin, uint32_t end, D4 (&s)[NV]) {
   constexpr int kDepth = NV == 1 ? 8 : 4;
   uint32_t i = begin;
-  for (; i + kDepth <= end; i += kDepth) {
+  for (; i + (kDepth - 1) * STEP < end; i += kDepth * STEP) {
     uint32_t b[kDepth];
 #pragma unroll
-    for (int k = 0; k < kDepth; ++k) b[k] = wk.bag_of_sorted[i + k];
+    for (int k = 0; k < kDepth; ++k) b[k] = wk.bag_of_sorted[i + k * STEP];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const uint32_t c4 = gl + v * G;
@@ -107,7 +107,7 @@ __device__ inline void reduce_segment(const Work& wk, const float* __restrict__ 
     // the ragged tail, again with all its loads issued before the adds
     uint32_t b[kDepth];
 #pragma unroll
-    for (int k = 0; k < kDepth; ++k) b[k] = i + k < end ? wk.bag_of_sorted[i + k] : 0xFFFFFFFFu;
+    for (int k = 0; k < kDepth; ++k) b[k] = i + k * STEP < end ? wk.bag_of_sorted[i + k * STEP] : 0xFFFFFFFFu;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const uint32_t c4 = gl + v * G;
@@ -146,59 +146,78 @@ file_segments_kernel(Work wk, long long n_ids, long long n_bags) { after_previou
 // What bounds it: gradient rows gathered at random for the first two kinds (latency; ten blocks of 128
 // threads per SM at 48 registers: eight at 64 measured 3 % of a step slower, twelve spill), HBM for the third.
 
-// Sum of partial sums src[0], src[stride], ... (n of them, in that order) for the columns this lane owns.
-// They were written by other blocks: read past L1.
-template <int G, int NV>
-__device__ __forceinline__ void sum_partials(const double* src, uint32_t n, size_t stride, uint32_t dim, int gl, D4 (&s)[NV]) {
+// The lanes that work on one part of a long segment: PG of them, PG / G lane groups that take turns at the
+// rows to add up.
+template <int PG, int G>
+struct Team {
+  static constexpr int kGroups = PG / G;
+  int lane = threadIdx.x % PG, gl = threadIdx.x % G, grp = threadIdx.x % PG / G;
+  unsigned mask = PG == 32 ? 0xFFFFFFFFu : ((1u << (PG & 31)) - 1u) << ((threadIdx.x & 31) / PG * PG);
+
+  // the groups have each summed a share: afterwards every one of them has the whole
+  template <int NV>
+  __device__ __forceinline__ void add_groups(D4 (&s)[NV]) const {
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const uint32_t c4 = gl + v * G;
-    if (c4 * 4u < dim) {
-      const double2* p = reinterpret_cast<const double2*>(src) + c4 * 2;
-      D4 a = D4{0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
-      for (uint32_t i = 0; i < n; ++i, p += stride / 2) {
-        const double2 x = __ldcg(p), y = __ldcg(p + 1);
-        a.x += x.x; a.y += x.y; a.z += y.x; a.w += y.y;
+    for (int o = G; o < PG; o <<= 1)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        s[v].x += __shfl_xor_sync(mask, s[v].x, o);
+        s[v].y += __shfl_xor_sync(mask, s[v].y, o);
+        s[v].z += __shfl_xor_sync(mask, s[v].z, o);
+        s[v].w += __shfl_xor_sync(mask, s[v].w, o);
       }
-      s[v] = a;
+  }
+
+  // s = src[0] + src[stride] + ... (n of them).  They were written by other blocks: read past L1.
+  template <int NV>
+  __device__ __forceinline__ void sum_partials(const double* src, uint32_t n, size_t stride, uint32_t dim, D4 (&s)[NV]) const {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const uint32_t c4 = gl + v * G;
+      s[v] = D4{0.0, 0.0, 0.0, 0.0};
+      if (c4 * 4u < dim) {
+#pragma unroll 4
+        for (uint32_t i = grp; i < n; i += kGroups) {
+          const double2* p = reinterpret_cast<const double2*>(src + i * stride) + c4 * 2;
+          const double2 x = __ldcg(p), y = __ldcg(p + 1);
+          s[v].x += x.x; s[v].y += x.y; s[v].z += y.x; s[v].w += y.y;
+        }
+      }
     }
+    add_groups<NV>(s);
   }
-}
 
-// The long ID that part p belongs to: the last one whose first part is not after p.  The lanes of the
-// group look at G places at a time.
-template <int G>
-__device__ __forceinline__ uint32_t owner_of_part(const Work& wk, uint32_t n_long, uint32_t p, int gl, unsigned group_mask) {
-  uint32_t lo = 0, n = n_long;                                           // it is in [lo, lo + n)
-  while (n > 1) {
-    const uint32_t step = (n + G - 1) / G, at = gl * step;
-    const bool before = at < n && wk.long_part0[lo + at] <= p;
-    const uint32_t c = __popc(__ballot_sync(group_mask, before)) - 1;
-    lo += c * step;
-    n = min(step, n - c * step);
+  // The long ID that part p belongs to: the last one whose first part is not after p, PG places at a time.
+  __device__ __forceinline__ uint32_t owner_of_part(const Work& wk, uint32_t n_long, uint32_t p) const {
+    uint32_t lo = 0, n = n_long;                                         // it is in [lo, lo + n)
+    while (n > 1) {
+      const uint32_t step = (n + PG - 1) / PG, at = lane * step;
+      const bool before = at < n && wk.long_part0[lo + at] <= p;
+      const uint32_t c = __popc(__ballot_sync(mask, before)) - 1;
+      lo += c * step;
+      n = min(step, n - c * step);
+    }
+    return lo;
   }
-  return lo;
-}
+};
 
-// The parts of the long segments.  A lane group sums one part into fp64 partial sums in scratch.
-// Partial sums are added up in a tree: the group that finishes the last of kFanIn neighbours adds
+// The parts of the long segments.  A team of PG lanes sums one part into fp64 partial sums in scratch.
+// Partial sums are added up in a tree: the team that finishes the last of kFanIn neighbours adds
 // them up and goes on to the next level, and the one that reaches the top updates the row.  The
 // order of every addition is fixed by the parts' numbers, whoever does it.  (A tree, because one ID
 // can own a tenth of a batch: with 64 neighbours at a time and then all the rest, adding up the
 // 11 000 parts of such an ID was a serial chain of 50 us.)
-template <int G, int NV>
+template <int PG, int G, int NV>
 __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
                                     bool ordered, uint32_t vblock, uint32_t vgrid) {
   const unsigned long long longs = wk.call->longs;
   const uint32_t n_parts = (uint32_t)longs, n_long = (uint32_t)(longs >> 32);
-  const int gl = threadIdx.x % G, lane = threadIdx.x & 31;
-  const unsigned group_mask = G == 32 ? 0xFFFFFFFFu : ((1u << (G & 31)) - 1u) << (lane / G * G);
-  const uint32_t groups = (vgrid * blockDim.x) / G;
-  for (uint32_t item = (vblock * blockDim.x + threadIdx.x) / G; item < n_parts; item += groups) {
+  const Team<PG, G> team;
+  const uint32_t teams = (vgrid * blockDim.x) / PG;
+  for (uint32_t item = (vblock * blockDim.x + threadIdx.x) / PG; item < n_parts; item += teams) {
     const uint32_t p = ordered ? wk.part_order[item] : item;
     if (!MONO_INDEX_OK(wk.error_bits, p, wk.max_parts)) continue;
-    const uint32_t li = ordered ? wk.part_u[p] : owner_of_part<G>(wk, n_long, p, gl, group_mask);
+    const uint32_t li = ordered ? wk.part_u[p] : team.owner_of_part(wk, n_long, p);
     if (!MONO_INDEX_OK(wk.error_bits, li, wk.max_long)) continue;
     const uint32_t u = wk.long_u[li], p0 = wk.long_part0[li];
     const uint32_t row_word = wk.urow[u];
@@ -210,7 +229,8 @@ __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const f
     D4 s[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) s[v] = D4{0.0, 0.0, 0.0, 0.0};
-    reduce_segment<G, NV>(wk, grad, n_bags, tv.dim, gl, begin, end, s);
+    reduce_segment<G, NV, PG / G>(wk, grad, n_bags, tv.dim, team.gl, begin + team.grp, end, s);
+    team.template add_groups<NV>(s);
     const uint32_t parts = (m + kSegChunk - 1) / kSegChunk;
     bool top = true;
     for (uint32_t level = 0, step = 1; step < parts; ++level, step *= kFanIn) {
@@ -218,8 +238,8 @@ __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const f
       double* dst = wk.partials + (size_t)(p0 + k) * tv.dim;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const uint32_t c4 = gl + v * G;
-        if (c4 * 4u < tv.dim) {
+        const uint32_t c4 = team.gl + v * G;
+        if (team.grp == 0 && c4 * 4u < tv.dim) {
           reinterpret_cast<double2*>(dst)[c4 * 2] = make_double2(s[v].x, s[v].y);
           reinterpret_cast<double2*>(dst)[c4 * 2 + 1] = make_double2(s[v].z, s[v].w);
         }
@@ -228,22 +248,23 @@ __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const f
       const uint32_t want = min(kFanIn, (parts - k + step - 1) / step);
       uint32_t* counter = wk.part_done + p0 + k;                         // five bits per level: kFanIn at most
       __threadfence();
-      __syncwarp(group_mask);
+      __syncwarp(team.mask);
       uint32_t before = 0;
-      if (gl == 0) before = atomicAdd(counter, 1u << (5 * level));
-      before = __shfl_sync(group_mask, before, 0, G) >> (5 * level) & 31u;
+      if (team.lane == 0) before = atomicAdd(counter, 1u << (5 * level));
+      before = __shfl_sync(team.mask, before, 0, PG) >> (5 * level) & 31u;
       if (before != want - 1u) { top = false; break; }
       __threadfence();
-      if (gl == 0) atomicSub(counter, want << (5 * level));              // zero again for the next call
-      sum_partials<G, NV>(wk.partials + (size_t)(p0 + k) * tv.dim, want, (size_t)step * tv.dim, tv.dim, gl, s);
+      if (team.lane == 0) atomicSub(counter, want << (5 * level));       // zero again for the next call
+      team.template sum_partials<NV>(wk.partials + (size_t)(p0 + k) * tv.dim, want, (size_t)step * tv.dim, tv.dim, s);
     }
     if (!top) continue;
     const unsigned long long id = wk.uid[u];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const uint32_t c4 = gl + v * G;
-      if (c4 * 4u < tv.dim) update_row(tv, row_word, id, c4, s[v]);
+      const uint32_t c4 = team.gl + v * G;
+      if (team.grp == 0 && c4 * 4u < tv.dim) update_row(tv, row_word, id, c4, s[v]);
     }
+    __syncwarp(team.mask);
   }
 }
 
@@ -342,15 +363,21 @@ __device__ inline void update_singletons(const TableView& tv, const Work& wk, co
   if (lane == 0 && n_single) atomicAdd(&tv.st->sum_single_resident, (unsigned long long)n_single);
 }
 constexpr int kRowThreads = 128;
+constexpr uint32_t kFewParts = 4096;     // a warp for each is resident
 // How the grid is shared out: blocks [0, parts) take the parts, the next `shorts` the short segments,
 // the rest what occurs once.
 struct RowGrid { uint32_t parts, shorts, singles; };
 
-template <int G, int NV>
+template <int G, int NV, bool FEW>
 __device__ __forceinline__ void update_rows_body(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
                                                  bool ordered, const RowGrid& grid, uint32_t total_blocks, uint32_t vblock) {
   if (vblock < grid.parts) {
-    reduce_parts<G, NV>(tv, wk, grad, n_bags, ordered, vblock, grid.parts);
+    // Few parts (they are resident all at once): a warp each, because the longest chain of loads is what
+    // counts (step of 20 000 IDs 35.8 -> 28.4 us, of 135 000 56 -> 47).  Many: a lane group each, which
+    // spends nothing on adding groups up (a warp each: 1 M IDs 154 -> 160 us, 4 M drifting 351 -> 370).
+    // (A grouped call, whose tables share the SMs, has no use for it: FEW is false.)
+    if (G < 32 && (!FEW || (uint32_t)wk.call->longs > kFewParts)) reduce_parts<G, G, NV>(tv, wk, grad, n_bags, ordered, vblock, grid.parts);
+    else reduce_parts<32, G, NV>(tv, wk, grad, n_bags, ordered, vblock, grid.parts);
   } else if (vblock - grid.parts < grid.shorts) {
     reduce_short<G, NV>(tv, wk, grad, n_bags, vblock - grid.parts, grid.shorts);
   } else {
@@ -363,7 +390,7 @@ template <int G, int NV>
 __global__ void __launch_bounds__(kRowThreads, NV == 1 ? 10 : 4)
 update_rows_kernel(TableView tv, Work wk, const float* __restrict__ grad, long long n_bags, int ordered, RowGrid grid, uint32_t total_blocks) {
   after_previous_kernel();
-  update_rows_body<G, NV>(tv, wk, grad, n_bags, ordered != 0, grid, total_blocks, blockIdx.x);
+  update_rows_body<G, NV, true>(tv, wk, grad, n_bags, ordered != 0, grid, total_blocks, blockIdx.x);
 }
 
 }  // namespace mono

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kRowThreads, WIDE ? 4 : 10)
 group_update_rows_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   by_lane_class<WIDE>(it.lane_class, [&](auto g, auto nv) {
-    update_rows_body<decltype(g)::value, decltype(nv)::value>(it.tv, it.wk, it.grad, it.n_bags, false, it.row_grid, it.total_blocks, vblock);
+    update_rows_body<decltype(g)::value, decltype(nv)::value, false>(it.tv, it.wk, it.grad, it.n_bags, false, it.row_grid, it.total_blocks, vblock);
   });
 }
 

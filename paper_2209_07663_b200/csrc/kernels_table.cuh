@@ -194,8 +194,11 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
     // that the insertion that follows has nothing to tell the kernels that update rows
     const bool exact = tv.sketch_depth == 0;
     if ((MODE & kCommit) && exact && active && !hit && m >= tv.threshold) need_row = true;
-    const Reservation rv = block_reserve(tv, wk.call, &sh, need_row, (MODE & kLookUp) && m > 1, (MODE & kCommit) && active && !hit,
-                                         ((MODE & kLookUp) && m > 1) ? m : 0u);
+    // (the commit half of a batch that the table knows has nothing to reserve in most blocks)
+    Reservation rv = {kNoRow, 0u, 0u, 0u};
+    if ((MODE & kLookUp) || __syncthreads_or(need_row || (active && !hit)))
+      rv = block_reserve(tv, wk.call, &sh, need_row, (MODE & kLookUp) && m > 1, (MODE & kCommit) && active && !hit,
+                         ((MODE & kLookUp) && m > 1) ? m : 0u);
     if (!active) continue;
     if (MODE & kLookUp) {
       if (m > kSegChunk) register_long(wk, u, m);

@@ -401,8 +401,8 @@ bool orders_parts(const mono_table* t, int64_t n_bags) { return n_bags * (int64_
 unsigned update_grid(const mono_table* t, int64_t n_ids) { return (unsigned)clamp_blocks(n_ids, 256, grid_for(t, 8) * 4); }
 unsigned insert_grid(const mono_table* t, int64_t n_ids) { return (unsigned)clamp_blocks(n_ids, 256, grid_for(t, 8)); }
 // Blocks of the row updates for a batch that has `share` of the GPU (1, or its part of a grouped call).  The host
-// only knows how many IDs there are, so every share of the grid is sized for a long-tailed batch (a part per 64 IDs,
-// an ID in 64 with a short segment per lane group, one in four that occurs once per thread), and loops where that
+// only knows how many IDs there are, so every share of the grid is sized for a long-tailed batch (a part per 64 IDs, an ID
+// in 64 with a short segment, one in four that occurs once per thread), and loops where that
 // was too few: blocks that find nothing to do cost 1 ns each, 20 us of a step with eight waves of them on 1 M IDs.
 // While the batch is small enough for all of its blocks to be resident, it is spread as far as it goes instead.
 RowGrid rows_grid(const mono_table* t, int64_t n_ids, double share = 1.0) {
@@ -410,7 +410,7 @@ RowGrid rows_grid(const mono_table* t, int64_t n_ids, double share = 1.0) {
   const auto blocks = [&](int64_t most, int64_t typical, int64_t per, double resident) {
     return (uint32_t)clamp_blocks(most, per, std::max({std::min(cap, (typical + per - 1) / per), (int64_t)(resident * share), (int64_t)1}));
   };
-  return {blocks(n_ids / 64, n_ids / 64, groups, 1.0), blocks(n_ids / 2, n_ids / 64, groups, (double)wave),
+  return {blocks(n_ids / 64 * groups / 4, n_ids / 64, groups, (double)wave), blocks(n_ids / 2, n_ids / 64, groups, (double)wave),
           blocks(n_ids, n_ids / 4, kRowThreads, 2.0 * (double)wave)};
 }
 uint32_t blocks_of(const RowGrid& g) { return g.parts + g.shorts + g.singles; }
