@@ -102,19 +102,22 @@ struct mono_table {
   int64_t sketch_epoch = 0;       // time the sketch was last cleared
   int64_t max_ids = 0, max_bags = 0;
   // device staging for the host-buffer calls
-  unsigned long long* stage_ids = nullptr;
-  long long* stage_off = nullptr;
+  // (IDs and offsets twice: those of the next batch come in while the kernels still read this one's)
+  unsigned long long* stage_ids[2] = {};
+  long long* stage_off[2] = {};
+  int stage_at = 0;               // which of the two holds the batch that was staged last
   float* stage_out = nullptr;     // pooled rows on their way to the host
   float* stage_grad = nullptr;    // gradients on their way in
   // The host-buffer calls copy on two streams of their own, one per direction, so that a step's
   // gradients come in while its pooled rows still go out (the link is full duplex) and both
   // run beside the kernels.  ev_staged: the IDs or gradients have arrived; ev_out: the pooled
   // rows are ready to leave; ev_d2h: they have left; ev_stage_free: the kernels are done with
-  // the staged inputs.
+  // those staged IDs and offsets, ev_grad_free: with the staged gradients.  (Before they have
+  // been recorded for the first time, waiting for them is a no-op.)
   cudaStream_t h2d_stream = nullptr, d2h_stream = nullptr;
-  cudaEvent_t ev_staged = nullptr, ev_grad_in = nullptr, ev_out = nullptr, ev_d2h = nullptr, ev_stage_free = nullptr;
+  cudaEvent_t ev_staged = nullptr, ev_grad_in = nullptr, ev_out = nullptr, ev_d2h = nullptr, ev_grad_free = nullptr;
+  cudaEvent_t ev_stage_free[2] = {};
   bool d2h_pending = false;       // a copy to the host is in flight that `stream` has not waited for
-  bool stage_used = false;        // ev_stage_free has been recorded
   // the host batch whose IDs and offsets are on the device, staged by mono_lookup_pool_host
   struct { const void* ids; int64_t n_ids; const void* off; int64_t n_bags; bool valid; } staged = {nullptr, 0, nullptr, 0, false};
   std::string last_err;
@@ -158,7 +161,8 @@ void free_scratch(mono_table* t) {
   dev_free(w.bset); dev_free(w.occ); dev_free(w.occ_bag); dev_free(w.bag_of_sorted);
   dev_free(w.uid); dev_free(w.uslot); dev_free(w.uocc); dev_free(w.useg); dev_free(w.ulen); dev_free(w.urow); dev_free(w.ucell); dev_free(w.umeta);
   dev_free(w.multi_list); dev_free(w.ins_list); dev_free(w.long_u); dev_free(w.long_part0); dev_free(w.part_u); dev_free(w.part_order); dev_free(w.win_count); dev_free(w.partials); dev_free(w.part_done); dev_free(w.call);
-  dev_free(t->stage_ids); dev_free(t->stage_off); dev_free(t->stage_out); dev_free(t->stage_grad); dev_free(t->occ_row);
+  for (int b = 0; b < 2; ++b) { dev_free(t->stage_ids[b]); dev_free(t->stage_off[b]); }
+  dev_free(t->stage_out); dev_free(t->stage_grad); dev_free(t->occ_row);
   auto& ah = t->ahead;
   dev_free(ah.bset); dev_free(ah.occ); dev_free(ah.occ_bag); dev_free(ah.uid); dev_free(ah.uslot); dev_free(ah.uocc); dev_free(ah.call);
   ah.valid = false;
@@ -271,9 +275,8 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   ALLOC(w.long_u, w.max_long); ALLOC(w.long_part0, w.max_long); ALLOC(w.part_u, w.max_parts); ALLOC(w.part_order, w.max_parts); ALLOC(w.win_count, 2 * kWindows);
   ALLOC(w.partials, (size_t)w.max_parts * t->tv.dim);
   ALLOC(w.part_done, w.max_parts); ALLOC(w.call, 1);
-  ALLOC(t->stage_ids, n); ALLOC(t->stage_off, (size_t)max_bags + 1);
-  // (the two staging buffers of the host-buffer calls, one bag-by-dim matrix each, are allocated by the
-  // first such call: callers that keep their batches on the device never pay for them)
+  // (the staging buffers of the host-buffer calls are allocated by the first such call: callers that keep
+  // their batches on the device never pay for them)
   ALLOC(t->occ_row, n);
 #undef ALLOC
   w.primary_mask = (uint32_t)(primary - 1);
@@ -769,7 +772,7 @@ int mono_table_destroy(mono_table* t) {
   if (t->ahead_stream) { cudaStreamSynchronize(t->ahead_stream); cudaStreamDestroy(t->ahead_stream); }
   if (t->h2d_stream) { cudaStreamSynchronize(t->h2d_stream); cudaStreamDestroy(t->h2d_stream); }
   if (t->d2h_stream) { cudaStreamSynchronize(t->d2h_stream); cudaStreamDestroy(t->d2h_stream); }
-  for (cudaEvent_t e : {t->ev_staged, t->ev_grad_in, t->ev_out, t->ev_d2h, t->ev_stage_free}) if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : {t->ev_staged, t->ev_grad_in, t->ev_out, t->ev_d2h, t->ev_grad_free, t->ev_stage_free[0], t->ev_stage_free[1]}) if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : {t->ev_fork, t->ev_keys, t->ev_swept, t->ev_group, t->ev_aux, t->ev_commit, t->ev_ahead, t->ev_swap})
     if (e) cudaEventDestroy(e);
   for (auto& p : t->pending) { cudaEventDestroy(p.second.first); cudaEventDestroy(p.second.second); }
@@ -1098,29 +1101,39 @@ int mono_lookup_pool_noalloc(mono_table* t, const uint64_t* ids, int64_t n_ids, 
 }
 
 // Streams, events and staging of the host-buffer calls, made by the first of them.
-static int host_path_ready(mono_table* t, int64_t n_bags) {
+static int host_path_ready(mono_table* t) {
   if (!t->h2d_stream) {
     CUDA_TRY(t, cudaStreamCreateWithFlags(&t->h2d_stream, cudaStreamNonBlocking));
     CUDA_TRY(t, cudaStreamCreateWithFlags(&t->d2h_stream, cudaStreamNonBlocking));
-    for (cudaEvent_t* e : {&t->ev_staged, &t->ev_grad_in, &t->ev_out, &t->ev_d2h, &t->ev_stage_free})
+    for (cudaEvent_t* e : {&t->ev_staged, &t->ev_grad_in, &t->ev_out, &t->ev_d2h, &t->ev_grad_free, &t->ev_stage_free[0], &t->ev_stage_free[1]})
       CUDA_TRY(t, cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   }
   if (!t->stage_out) {                                     // sized with the rest of the scratch: max_bags rows
-    (void)n_bags;
     int rc = dev_alloc(t, &t->stage_out, (size_t)t->max_bags * t->tv.dim);
     if (rc == MONO_OK) rc = dev_alloc(t, &t->stage_grad, (size_t)t->max_bags * t->tv.dim);
-    if (rc != MONO_OK) { dev_free(t->stage_out); dev_free(t->stage_grad); return rc; }
+    for (int b = 0; b < 2 && rc == MONO_OK; ++b) {
+      rc = dev_alloc(t, &t->stage_ids[b], (size_t)t->max_ids);
+      if (rc == MONO_OK) rc = dev_alloc(t, &t->stage_off[b], (size_t)t->max_bags + 1);
+    }
+    if (rc != MONO_OK) {
+      dev_free(t->stage_out); dev_free(t->stage_grad);
+      for (int b = 0; b < 2; ++b) { dev_free(t->stage_ids[b]); dev_free(t->stage_off[b]); }
+      return rc;
+    }
   }
   return MONO_OK;
 }
 
-// IDs and offsets of a host batch to the staging buffers, on the inbound copy stream, once the
-// kernels of the previous step are done with what is there.
+// IDs and offsets of a host batch to the staging buffers that the last one does not sit in, on the inbound copy
+// stream.  They may be overwritten once the kernels of the batch before the last are done with them, so the copy
+// does not wait for this batch's push: with one set of buffers the inbound link stood idle while the push of
+// 213 000 bags of 32 columns ran.
 static int stage_batch(mono_table* t, const uint64_t* ids, int64_t n_ids, const int64_t* off, int64_t n_bags) {
   cudaStream_t c = t->h2d_stream;
-  if (t->stage_used) CUDA_TRY(t, cudaStreamWaitEvent(c, t->ev_stage_free, 0));
-  if (n_ids) CUDA_TRY(t, cudaMemcpyAsync(t->stage_ids, ids, (size_t)n_ids * 8, cudaMemcpyHostToDevice, c));
-  CUDA_TRY(t, cudaMemcpyAsync(t->stage_off, off, (size_t)(n_bags + 1) * 8, cudaMemcpyHostToDevice, c));
+  const int b = t->stage_at ^= 1;
+  CUDA_TRY(t, cudaStreamWaitEvent(c, t->ev_stage_free[b], 0));
+  if (n_ids) CUDA_TRY(t, cudaMemcpyAsync(t->stage_ids[b], ids, (size_t)n_ids * 8, cudaMemcpyHostToDevice, c));
+  CUDA_TRY(t, cudaMemcpyAsync(t->stage_off[b], off, (size_t)(n_bags + 1) * 8, cudaMemcpyHostToDevice, c));
   CUDA_TRY(t, cudaEventRecord(t->ev_staged, c));
   CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_staged, 0));
   return MONO_OK;
@@ -1134,26 +1147,26 @@ int mono_lookup_pool_host(mono_table* t, const uint64_t* ids, int64_t n_ids, con
   if (rc != MONO_OK) return rc;
   if (n_bags > 0 && !out) return MONO_ERR_ARG;
   if ((rc = reserve(t, n_ids, n_bags)) != MONO_OK) return rc;
-  if ((rc = host_path_ready(t, n_bags)) != MONO_OK) return rc;
+  if ((rc = host_path_ready(t)) != MONO_OK) return rc;
   if ((rc = discard_prepared(t)) != MONO_OK) return rc;
   t->staged.valid = false;
   cudaStream_t s = t->stream;
-  // the staging buffers must be free: the kernels that read the last staged batch have been issued on `s`
-  CUDA_TRY(t, cudaEventRecord(t->ev_stage_free, s));
-  t->stage_used = true;
   if ((rc = stage_batch(t, ids, n_ids, slot_offsets, n_bags)) != MONO_OK) return rc;
   if (n_bags == 0) return MONO_OK;
+  unsigned long long* d_ids = t->stage_ids[t->stage_at];
+  long long* d_off = t->stage_off[t->stage_at];
   // the staged batch is the one the push that follows will be given: group it and look its IDs up once for both
   bool prepared = false;
   if (n_ids > 0) {
-    if ((rc = launch_prepare(t, t->stage_ids, n_ids, t->stage_off, n_bags)) != MONO_OK) return rc;
+    if ((rc = launch_prepare(t, d_ids, n_ids, d_off, n_bags)) != MONO_OK) return rc;
     t->staged = {ids, n_ids, slot_offsets, n_bags, true};
     prepared = true;
   }
   // the previous result must have left stage_out before this one is written there
   if (t->d2h_pending) { CUDA_TRY(t, cudaStreamWaitEvent(s, t->ev_d2h, 0)); t->d2h_pending = false; }
-  if ((rc = launch_lookup(t, t->stage_ids, n_ids, t->stage_off, n_bags, t->stage_out, prepared)) != MONO_OK) return rc;
+  if ((rc = launch_lookup(t, d_ids, n_ids, d_off, n_bags, t->stage_out, prepared)) != MONO_OK) return rc;
   CUDA_TRY(t, cudaEventRecord(t->ev_out, s));
+  CUDA_TRY(t, cudaEventRecord(t->ev_stage_free[t->stage_at], s));          // (recorded again by the push, if it takes this batch)
   CUDA_TRY(t, cudaStreamWaitEvent(t->d2h_stream, t->ev_out, 0));
   CUDA_TRY(t, cudaMemcpyAsync(out, t->stage_out, (size_t)n_bags * t->tv.dim * 4, cudaMemcpyDeviceToHost, t->d2h_stream));
   CUDA_TRY(t, cudaEventRecord(t->ev_d2h, t->d2h_stream));
@@ -1170,34 +1183,32 @@ int mono_apply_grads_host(mono_table* t, const uint64_t* ids, int64_t n_ids, con
   if (n_bags > 0 && !grad_pooled) return MONO_ERR_ARG;
   if ((rc = check_now(t, now)) != MONO_OK) return rc;
   if ((rc = reserve(t, n_ids, n_bags)) != MONO_OK) return rc;
-  if ((rc = host_path_ready(t, n_bags)) != MONO_OK) return rc;
+  if ((rc = host_path_ready(t)) != MONO_OK) return rc;
   cudaStream_t s = t->stream;
   const bool reuse = t->staged.valid && t->staged.ids == ids && t->staged.n_ids == n_ids && t->staged.off == slot_offsets &&
                      t->staged.n_bags == n_bags;
   t->staged.valid = false;
   if (!reuse) {
-    // not the batch the lookup staged: bring its IDs and offsets in now (what was announced from the
-    // staging buffers is about to be overwritten)
+    // not the batch the lookup staged: bring its IDs and offsets in now
     if ((rc = discard_prepared(t)) != MONO_OK) return rc;
-    CUDA_TRY(t, cudaEventRecord(t->ev_stage_free, s));
-    t->stage_used = true;
     if ((rc = stage_batch(t, ids, n_ids, slot_offsets, n_bags)) != MONO_OK) return rc;
   }
-  // the gradients come in on the copy stream while the ID-only kernels of the push run (the previous
-  // push, the last reader of stage_grad, was issued before ev_stage_free was last recorded)
+  // the gradients come in on the copy stream while the ID-only kernels of the push run
   cudaEvent_t grad_ready = nullptr;
   if (n_bags) {
     cudaStream_t c = t->h2d_stream;
-    if (t->stage_used) CUDA_TRY(t, cudaStreamWaitEvent(c, t->ev_stage_free, 0));
+    CUDA_TRY(t, cudaStreamWaitEvent(c, t->ev_grad_free, 0));
     CUDA_TRY(t, cudaMemcpyAsync(t->stage_grad, grad_pooled, (size_t)n_bags * t->tv.dim * 4, cudaMemcpyHostToDevice, c));
     CUDA_TRY(t, cudaEventRecord(t->ev_grad_in, c));
     grad_ready = t->ev_grad_in;
   }
   t->last_now = now;
-  rc = launch_apply(t, t->stage_ids, n_ids, t->stage_off, n_bags, t->stage_grad, (uint32_t)now, grad_ready);
+  rc = launch_apply(t, t->stage_ids[t->stage_at], n_ids, t->stage_off[t->stage_at], n_bags, t->stage_grad, (uint32_t)now, grad_ready);
   if (rc != MONO_OK) return rc;
   // (an empty batch launches nothing, so nothing has waited for the gradient copy yet)
   if (grad_ready && (n_ids == 0 || n_bags == 0)) CUDA_TRY(t, cudaStreamWaitEvent(s, grad_ready, 0));
+  CUDA_TRY(t, cudaEventRecord(t->ev_stage_free[t->stage_at], s));
+  CUDA_TRY(t, cudaEventRecord(t->ev_grad_free, s));
   return MONO_OK;
 }
 
