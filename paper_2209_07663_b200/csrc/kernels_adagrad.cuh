@@ -30,8 +30,8 @@ __device__ inline void add4(D4& a, const float4 v) { a.x += (double)v.x; a.y += 
 
 // acc += G*G;  w -= lr*G/(sqrt(acc)+eps), each operation rounded to fp32 on its
 // own (no fused multiply-add), so the result does not depend on contraction.
-__device__ inline void adagrad4(float4& w, float4& a, const D4& g, float lr, float eps) {
-  const float gx = (float)g.x, gy = (float)g.y, gz = (float)g.z, gw = (float)g.w;
+__device__ inline void adagrad4(float4& w, float4& a, const float4 g, float lr, float eps) {
+  const float gx = g.x, gy = g.y, gz = g.z, gw = g.w;
   a.x = __fadd_rn(a.x, __fmul_rn(gx, gx));
   a.y = __fadd_rn(a.y, __fmul_rn(gy, gy));
   a.z = __fadd_rn(a.z, __fmul_rn(gz, gz));
@@ -56,7 +56,7 @@ __device__ inline void update_row(const TableView& tv, uint32_t row_word, unsign
     w = *pw;
     a = *pa;
   }
-  adagrad4(w, a, g, tv.lr, tv.eps);
+  adagrad4(w, a, make_float4((float)g.x, (float)g.y, (float)g.z, (float)g.w), tv.lr, tv.eps);
   *pw = w;
   *pa = a;
 }
@@ -144,7 +144,8 @@ file_segments_kernel(Work wk, long long n_ids, long long n_bags) { after_previou
 // whole step: 20 000 IDs 54 -> 36 us, 1 M IDs 180 -> 153, 4 M drifting 360 -> 348, 8 M 1404 -> 1395; against the
 // three kinds one after the other in every block, 47 / 163 / 411 / 1437.
 // What bounds it: gradient rows gathered at random for the first two kinds (latency; ten blocks of 128
-// threads per SM at 48 registers: eight at 64 measured 3 % of a step slower, twelve spill), HBM for the third.
+// threads per SM at 48 registers: eight at 64 measured 3 % of a step slower, twelve spill; rows of 132 to 256 columns
+// seven at 72, 198 -> 167 us per step against four), HBM for the third.
 
 // The lanes that work on one part of a long segment: PG of them, PG / G lane groups that take turns at the
 // rows to add up.
@@ -308,6 +309,9 @@ template <int G, int NV>
 __device__ inline void update_singletons(const TableView& tv, const Work& wk, const float* __restrict__ grad,
                                               long long n_bags, uint32_t vblock, uint32_t vgrid) {
   constexpr int kGroups = 32 / G;
+  // Two rows of a lane group in flight (1.3 M single rows of 64 columns 5 % faster, whole step 1395 -> 1380 us; 99 000 of
+  // 100 columns 137 -> 130); rows of several vectors per lane have their own loads to overlap.
+  constexpr int kRows = NV == 1 ? 2 : 1;
   const int lane = threadIdx.x & 31;
   const int gl = lane % G, grp = lane / G;
   const uint32_t n = wk.call->n_unique;
@@ -332,32 +336,54 @@ __device__ inline void update_singletons(const TableView& tv, const Work& wk, co
     unsigned todo = __ballot_sync(0xFFFFFFFFu, single);
     n_single += __popc(todo);
     while (todo) {
-      // the next kGroups flagged lanes, one per lane group
-      int src = -1;
-      unsigned rest = todo;
+      // the next kGroups * kRows flagged lanes, kRows for each lane group; all their loads before the first store
+      uint32_t rw[kRows], bg[kRows];
+      unsigned long long key[kRows];
+      bool mine[kRows];
 #pragma unroll
-      for (int g = 0; g < kGroups; ++g) {
-        const int l = rest ? __ffs(rest) - 1 : -1;
-        if (l >= 0) rest &= rest - 1;
-        if (g == grp) src = l;
+      for (int k = 0; k < kRows; ++k) {
+        int src = -1;
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) {
+          const int l = todo ? __ffs(todo) - 1 : -1;
+          if (l >= 0) todo &= todo - 1;
+          if (g == grp) src = l;
+        }
+        mine[k] = src >= 0;
+        const int from = src < 0 ? 0 : src;
+        rw[k] = __shfl_sync(0xFFFFFFFFu, row_word, from);
+        bg[k] = __shfl_sync(0xFFFFFFFFu, bag, from);
+        key[k] = __shfl_sync(0xFFFFFFFFu, id, from);
       }
-      todo = rest;
-      const int from = src < 0 ? 0 : src;
-      const uint32_t rw = __shfl_sync(0xFFFFFFFFu, row_word, from);
-      const uint32_t bg = __shfl_sync(0xFFFFFFFFu, bag, from);
-      const unsigned long long key = __shfl_sync(0xFFFFFFFFu, id, from);
-      if (src >= 0) {
-        const float4* g4 = reinterpret_cast<const float4*>(grad + (size_t)bg * tv.dim);
+      float4 x[kRows][NV], w[kRows][NV], a[kRows][NV];
+#pragma unroll
+      for (int k = 0; k < kRows; ++k)
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const uint32_t c4 = gl + v * G;
-          if (c4 * 4u < tv.dim) {
-            const float4 x = __ldg(g4 + c4);
-            const D4 g = D4{(double)x.x, (double)x.y, (double)x.z, (double)x.w};
-            update_row(tv, rw, key, c4, g);
+          if (!mine[k] || c4 * 4u >= tv.dim) continue;
+          const uint32_t row = rw[k] & ~kFreshBit;
+          x[k][v] = __ldg(reinterpret_cast<const float4*>(grad + (size_t)bg[k] * tv.dim) + c4);
+          if (!(rw[k] & kFreshBit)) {
+            w[k][v] = reinterpret_cast<const float4*>(tv.w_row(row))[c4];
+            a[k][v] = reinterpret_cast<const float4*>(tv.acc_row(row))[c4];
           }
         }
-      }
+#pragma unroll
+      for (int k = 0; k < kRows; ++k)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const uint32_t c4 = gl + v * G;
+          if (!mine[k] || c4 * 4u >= tv.dim) continue;
+          const uint32_t row = rw[k] & ~kFreshBit;
+          if (rw[k] & kFreshBit) {
+            w[k][v] = init_vec(tv, key[k], c4);
+            a[k][v] = make_float4(tv.init_acc, tv.init_acc, tv.init_acc, tv.init_acc);
+          }
+          adagrad4(w[k][v], a[k][v], x[k][v], tv.lr, tv.eps);
+          reinterpret_cast<float4*>(tv.w_row(row))[c4] = w[k][v];
+          reinterpret_cast<float4*>(tv.acc_row(row))[c4] = a[k][v];
+        }
     }
   }
   if (lane == 0 && n_single) atomicAdd(&tv.st->sum_single_resident, (unsigned long long)n_single);
@@ -387,7 +413,7 @@ __device__ __forceinline__ void update_rows_body(const TableView& tv, const Work
   block_done(tv.st, wk, total_blocks);
 }
 template <int G, int NV>
-__global__ void __launch_bounds__(kRowThreads, NV == 1 ? 10 : 4)
+__global__ void __launch_bounds__(kRowThreads, NV == 1 ? 10 : NV == 2 ? 7 : 4)
 update_rows_kernel(TableView tv, Work wk, const float* __restrict__ grad, long long n_bags, int ordered, RowGrid grid, uint32_t total_blocks) {
   after_previous_kernel();
   update_rows_body<G, NV, true>(tv, wk, grad, n_bags, ordered != 0, grid, total_blocks, blockIdx.x);
