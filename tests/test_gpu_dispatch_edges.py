@@ -1,0 +1,150 @@
+"""Edges of the launch rules: the pooling kernels' tiles and vector widths, the parts of long
+segments and the tree their partial sums go up, the host-buffer staging taken in turn."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import mono_oracle as mo
+from paper_2209_07663_b200 import binding as mb
+from paper_2209_07663_b200 import workload as wl
+from tests.parity import assert_audit_ok, assert_state_equal, assert_vectors_close
+
+pytestmark = pytest.mark.gpu
+f32 = np.float32
+
+
+def filled(dim, n=4000, capacity=4096):
+    """A table whose n IDs own rows of known values."""
+    rng = np.random.default_rng(dim)
+    ids = wl.splitmix64(np.arange(1, n + 1, dtype=np.uint64))
+    w = rng.standard_normal((n, dim)).astype(f32)
+    t = mb.MonoTable(capacity, dim, 1, 0, key_cells=1 << 14)
+    t.import_entries(ids, np.ones(n, np.uint32), np.zeros(n, np.int64), np.ones(n, np.uint8), w, np.zeros_like(w))
+    return t, ids, w
+
+
+def pulls(t, ids, w, lens, rng, offset_floats=0, break_at=None):
+    """Pull bags of these lengths (some IDs unknown), announced and not; compare with a sum in double."""
+    dim, n = t.dim, len(ids)
+    total = int(np.sum(lens))
+    pick = rng.integers(0, n + n // 8, total)                      # beyond n: an ID the table does not know
+    flat = np.where(pick < n, ids[np.minimum(pick, n - 1)], np.uint64(1) + pick.astype(np.uint64)).astype(np.uint64)
+    off = np.zeros(len(lens) + 1, np.int64)
+    off[1:] = np.cumsum(lens)
+    rows = np.where((pick < n)[:, None], w[np.minimum(pick, n - 1)], 0).astype(np.float64)
+    want = np.stack([rows[off[b]:off[b + 1]].sum(axis=0) if lens[b] else np.zeros(dim) for b in range(len(lens))])
+    if break_at is not None:                                       # one bag malformed: it and the next read as empty or as they stand
+        off[break_at + 1] = off[break_at] - 1
+        want[break_at] = 0
+        lo, hi = off[break_at + 1], off[break_at + 2]
+        want[break_at + 1] = rows[lo:hi].sum(axis=0) if lo >= 0 else 0
+    d_ids, d_off = torch.from_numpy(flat.view(np.int64)).cuda(), torch.from_numpy(off).cuda()
+    store = torch.full((len(lens) * dim + 8,), float("nan"), device="cuda")
+    out = store[offset_floats:offset_floats + len(lens) * dim]
+    for announced in (False, True):
+        out.fill_(float("nan"))
+        if announced:
+            mb.mono_prepare_push(t.handle, d_ids, total, d_off, len(lens))
+        mb.mono_lookup_pool(t.handle, d_ids, total, d_off, len(lens), out)
+        assert_vectors_close(out.cpu().numpy().reshape(-1, dim), want.astype(f32), f"dim {dim}, announced {announced}")
+
+
+@pytest.mark.parametrize("dim", [4, 12, 64, 100, 128, 132, 136, 200, 512, 520])
+def test_pull_at_every_width_and_alignment(dim):
+    t, ids, w = filled(dim)
+    rng = np.random.default_rng(1)
+    for shift in (0, 4):                                           # 32-byte and only 16-byte aligned output
+        pulls(t, ids, w, rng.integers(0, 20, 700), rng, offset_floats=shift)
+    assert t.status()["error_bits"] == 0
+
+
+@pytest.mark.parametrize("lens", [
+    [1], [0], [1024], [1025], [5000], [0] * 9 + [33], [1] * 256, [1] * 257, [2] * 8,
+    [31, 32, 33, 63, 64, 65] * 50, [1] * 300 + [1023] + [1] * 300, [700, 400] * 20, list(range(40)) * 30,
+], ids=lambda v: f"{len(v)}x{max(v)}")
+def test_pull_at_the_edges_of_tiles(lens):
+    for dim in (16, 200):
+        t, ids, w = filled(dim)
+        pulls(t, ids, w, np.array(lens), np.random.default_rng(2))
+        assert t.status()["error_bits"] == 0
+
+
+@pytest.mark.parametrize("lens", [[3] * 400, [700, 400] * 20])
+def test_pull_with_a_malformed_bag_in_a_tile(lens):
+    t, ids, w = filled(32)
+    pulls(t, ids, w, np.array(lens), np.random.default_rng(3), break_at=5)
+    assert t.status()["error_bits"] == mb.MONO_DEV_BAD_OFFSETS
+
+
+# multiplicities at the edges of parts (64) and of the levels of their tree (16, 256 and 4096 parts); the second
+# batch has more parts than get a warp each, the third more gradients than are left in the order they come
+@pytest.mark.parametrize("mult,dim,n_bags", [
+    ([63, 64, 65, 128, 1024, 1025, 1088, 16384, 16385], 32, 3000),
+    ([300000, 64 * 256 + 1, 65, 1], 8, 20000),
+    ([16385, 1024, 65, 64], 520, 40000),
+])
+@pytest.mark.parametrize("announced", [False, True])
+def test_long_segments_at_the_edges_of_the_tree(mult, dim, n_bags, announced):
+    kw = dict(init_scale=0.05, seed=9)
+    gpu, cpu = mb.MonoTable(64, dim, 1, 0, **kw), mo.OracleTable(64, dim, 1, 0, **kw)
+    rng = np.random.default_rng(4)
+    ids = rng.permutation(np.repeat(wl.splitmix64(np.arange(len(mult), dtype=np.uint64)), mult))
+    cuts = np.sort(rng.integers(0, ids.size + 1, n_bags - 1))
+    off = np.concatenate([[0], cuts, [ids.size]]).astype(np.int64)
+    for now in range(2):                                           # the second push finds counters and set as the first left them
+        grad = (rng.standard_normal((n_bags, dim)) * 0.01).astype(f32)
+        d = [torch.from_numpy(x).cuda() for x in (ids.view(np.int64), off, grad)]
+        if announced:
+            mb.mono_prepare_push(gpu.handle, d[0], ids.size, d[1], n_bags)
+        mb.mono_apply_grads(gpu.handle, d[0], ids.size, d[1], n_bags, d[2], now)
+        cpu.apply_grads(ids, off, grad, now)
+        assert_state_equal(gpu, cpu, f"push {now}")
+    assert_audit_ok(gpu)
+    assert gpu.status()["error_bits"] == 0
+
+
+def test_distinct_ids_fill_the_first_tier_of_the_call_set():
+    """Batches of distinct IDs only: the primary tier has a slot for each, and what does not find one near
+    its place overflows; both tiers have to be empty again for the next push."""
+    kw = dict(init_scale=0.05, seed=3)
+    gpu, cpu = mb.MonoTable(1 << 14, 16, 1, 0, max_ids=8192, **kw), mo.OracleTable(1 << 14, 16, 1, 0, **kw)
+    rng = np.random.default_rng(5)
+    for now in range(3):
+        ids = wl.splitmix64(np.arange(now * 1000, now * 1000 + 8192, dtype=np.uint64))
+        off = np.arange(0, 8193, 4, dtype=np.int64)
+        grad = (rng.standard_normal((2048, 16)) * 0.01).astype(f32)
+        gpu.apply_grads(ids, off, grad, now)
+        cpu.apply_grads(ids, off, grad, now)
+    assert_state_equal(gpu, cpu)
+
+
+def test_host_buffers_are_staged_in_turn():
+    """Pulls without a push, pushes of another batch, and several steps in flight: every batch has to be read from
+    the buffers it was staged in."""
+    cfg = wl.scaled(wl.CONFIGS["tiny"], n_examples=128, filter_threshold=1)
+    kw = dict(lr=cfg.lr, eps=cfg.eps, init_scale=cfg.init_scale, seed=cfg.seed)
+    gpu = mb.MonoTable(cfg.capacity, cfg.dim, 1, 0, key_cells=cfg.key_cells, max_ids=4096, max_bags=cfg.n_bags, **kw)
+    cpu = mo.OracleTable(cfg.capacity, cfg.dim, 1, 0, **kw)
+    steps = [wl.Stream(cfg).step(t) for t in range(8)]
+    host = [[torch.from_numpy(x).pin_memory() for x in (s.ids.view(np.int64), s.offsets, s.grad_pooled)] for s in steps]
+    outs, wants = [], []
+
+    def pull(k):
+        outs.append(torch.full((cfg.n_bags, cfg.dim), float("nan")).pin_memory())
+        mb.mono_lookup_pool_host(gpu.handle, host[k][0], host[k][0].numel(), host[k][1], cfg.n_bags, outs[-1])
+        wants.append(cpu.lookup_pool(steps[k].ids, steps[k].offsets))
+
+    def push(k, now):
+        mb.mono_apply_grads_host(gpu.handle, host[k][0], host[k][0].numel(), host[k][1], cfg.n_bags, host[k][2], now)
+        cpu.apply_grads(steps[k].ids, steps[k].offsets, steps[k].grad_pooled, now)
+
+    push(0, 0)
+    for now in range(1, 4):
+        pull(now), pull(now + 1), pull(now)
+        push(now, 2 * now)
+        push(now + 4, 2 * now + 1)
+    mb.mono_fence(gpu.handle)
+    torch.cuda.synchronize()
+    for k, (got, want) in enumerate(zip(outs, wants)):
+        assert_vectors_close(got.numpy(), want, f"pull {k}")
+    assert_state_equal(gpu, cpu)
