@@ -57,19 +57,14 @@ def measured_peaks():
 
 
 KERNEL_SOURCES = {
-    "probe_rows": ("kernels_forward.cuh", "table_layout.cuh"),
     "gather_pool": ("kernels_forward.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
     "fill_occ_bag": ("kernels_dedup.cuh", "table_layout.cuh"),
     "dedup_tile": ("kernels_dedup.cuh", "table_layout.cuh"),
     "table_lookup": ("kernels_table.cuh", "kernels_forward.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
     "table_update": ("kernels_table.cuh", "kernels_forward.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
     "table_insert": ("kernels_table.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
-    "update_singletons": ("kernels_adagrad.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
-    "file_segments": ("kernels_adagrad.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
-    "reduce_adagrad": ("kernels_adagrad.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
-    "reduce_parts": ("kernels_adagrad.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
-    "combine_adagrad": ("kernels_adagrad.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
-    "fold_partials": ("kernels_adagrad.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
+    "file_segments": ("kernels_adagrad.cuh", "kernels_forward.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
+    "update_rows": ("kernels_adagrad.cuh", "kernels_forward.cuh", "kernels_table.cuh", "kernels_dedup.cuh", "table_layout.cuh"),
 }
 
 
@@ -288,7 +283,6 @@ def algorithmic_bytes(n, b, u, ur, ur1, unew, d, sweep_cells=0, prepared=True, e
     the lookup instead of once per occurrence inside it.  sweep_cells: key cells the step's slice
     of the expiry sweep covers, expired: entries it removes."""
     per_kernel = {
-        "probe_rows": 0,
         # offsets, one 8-byte record per occurrence (the ID, or its place in the grouping), each distinct row once, out
         "gather_pool": 8 * (b + 1) + 8 * n + (0 if prepared else 32 * n) + 4 * d * ur + 4 * d * b,
         "fill_occ_bag": 8 * (b + 1),                         # offsets
@@ -298,11 +292,9 @@ def algorithmic_bytes(n, b, u, ur, ur1, unew, d, sweep_cells=0, prepared=True, e
         "table_insert": (16 + 8 * d) * unew,                 # key write + row/accumulator initialisation
         "sketch_add": 0,                                     # (probabilistic filter: counted with table_insert's new IDs)
         "update_singletons": 20 * d * ur1,                   # IDs seen once: gradient row, row and accumulator in and out
-        # rows of repeated IDs + the gradient rows the singletons did not read, once (the two launches of
-        # reduce_adagrad_kernel, short segments and the parts of long ones, share them; counted on the first)
-        "reduce_adagrad": 16 * d * (ur - ur1) + 4 * d * max(b - ur1, 0), "reduce_parts": 0,
-        "file_segments": 0, "clear_set": 0,
-        "expand_parts": 0, "order_parts": 0, "fold_partials": 0, "combine_adagrad": 0, "finish_apply": 0,
+        # rows of repeated IDs + the gradient rows the singletons did not read, once (update_rows_kernel does both)
+        "reduce_adagrad": 16 * d * (ur - ur1) + 4 * d * max(b - ur1, 0), "update_rows": 0,
+        "file_segments": 0, "expand_parts": 0, "order_parts": 0,
         # the sweep's 4-byte record per 4-cell bucket in order; a removed entry's bucket read (64) and its cell cleared (32)
         "expire": sweep_cells + 96 * expired,
     }
@@ -310,11 +302,9 @@ def algorithmic_bytes(n, b, u, ur, ur1, unew, d, sweep_cells=0, prepared=True, e
 
 
 KERNEL_GROUP = {
-    "probe_rows": "lookup_pool", "gather_pool": "lookup_pool",
-    "fill_occ_bag": "dedup", "dedup_tile": "dedup", "finish_apply": "dedup", "clear_set": "dedup",
-    "table_lookup": "table", "table_update": "table", "sketch_add": "table", "table_insert": "table", "expand_parts": "table", "order_parts": "table",
-    "update_singletons": "adagrad", "file_segments": "lookup_pool", "reduce_parts": "adagrad", "reduce_adagrad": "adagrad", "fold_partials": "adagrad",
-    "combine_adagrad": "adagrad", "expire": "expire",
+    "gather_pool": "lookup_pool", "file_segments": "lookup_pool", "fill_occ_bag": "dedup", "dedup_tile": "dedup",
+    "table_lookup": "table", "table_update": "table", "sketch_add": "table", "table_insert": "table",
+    "expand_parts": "adagrad", "order_parts": "adagrad", "update_rows": "adagrad", "expire": "expire",
 }
 
 
@@ -552,6 +542,8 @@ def run_ours(args):
         gone = (st_c["n_expired_total"] - st_b["n_expired_total"]) / KT
         alg_kernel, alg_total = algorithmic_bytes(n, cfg.n_bags, u, ur, ur1, unew, d, cfg.key_cells // S if S > 0 else 0,
                                                   prepared=args.prepare, expired=gone)
+        # one kernel updates the rows of IDs that occur once and of those that repeat
+        alg_kernel["update_rows"] = alg_kernel.pop("update_singletons") + alg_kernel.pop("reduce_adagrad")
         per_kernel = {}
         for name, v in tim["kernels"].items():
             if v["launches"] and name in KERNEL_GROUP:
@@ -561,12 +553,7 @@ def run_ours(args):
             g = KERNEL_GROUP[name]
             group_ms[g] = group_ms.get(g, 0.0) + v["ms_per_launch"]
             group_bytes[g] = group_bytes.get(g, 0) + alg_kernel[name]
-        # the kernel that takes the most device time (reduce_adagrad_kernel is launched twice per step, for the
-        # short segments and for the parts of the long ones: its time is the two launches together)
-        if "reduce_parts" in per_kernel and "reduce_adagrad" in per_kernel:
-            per_kernel["reduce_adagrad"]["ms_short_segments"] = per_kernel["reduce_adagrad"]["ms_per_launch"]
-            per_kernel["reduce_adagrad"]["ms_parts"] = per_kernel["reduce_parts"]["ms_per_launch"]
-            per_kernel["reduce_adagrad"]["ms_per_launch"] += per_kernel.pop("reduce_parts")["ms_per_launch"]
+        # the kernel that takes the most device time
         dom = max(per_kernel, key=lambda k: per_kernel[k]["ms_per_launch"])
         dom_bytes, dom_ms = alg_kernel[dom], per_kernel[dom]["ms_per_launch"]
         achieved = dom_bytes / (dom_ms * 1e-3) / 1e9
@@ -615,10 +602,6 @@ def run_ours(args):
                 "peak_kind": f"of {peak_kind}", "algorithmic_bytes_per_launch": dom_bytes,
                 "ms_per_launch": dom_ms,
                 "traffic": recorded_traffic(dom, args.workload),
-                **({"launches_per_step": 2,
-                    "note": "this kernel runs twice per step (short segments, then the parts of long ones); bytes, "
-                            "time and traffic are those of the two launches together"}
-                   if dom == "reduce_adagrad" and "ms_parts" in per_kernel[dom] else {}),
             },
             "whole_step": {
                 "algorithmic_bytes": alg_total, "achieved_gbs": alg_total / (step_ms * 1e-3) / 1e9,
@@ -629,8 +612,6 @@ def run_ours(args):
                                    for k, v in per_kernel.items()},
                 "frac_by_phase": {g: round(group_bytes[g] / (group_ms[g] * 1e-3) / 1e9 / peak, 3) for g in group_ms},
                 "ms_by_kernel": {k: round(v["ms_per_launch"], 4) for k, v in per_kernel.items()},
-                "reduce_adagrad_ms": {"short_segments": per_kernel.get("reduce_adagrad", {}).get("ms_short_segments"),
-                                      "parts": per_kernel.get("reduce_adagrad", {}).get("ms_parts")},
                 "expire_ms_per_launch": (tim["kernels"]["expire"]["ms"] / tim["kernels"]["expire"]["launches"]
                                          if tim["kernels"]["expire"]["launches"] else None),
             },
