@@ -128,7 +128,7 @@ __device__ inline void reduce_segment(const Work& wk, const float* __restrict__ 
 // has filed the bags, FiledRows): one pass over the occurrences.
 __device__ inline void file_segments_body(const Work& wk, long long n_ids, long long n_bags, uint32_t vblock, uint32_t vgrid) {
   const long long stride = (long long)vgrid * blockDim.x;
-  const FiledRows rows{wk, n_bags, 0u};
+  const FiledRows<1> rows{wk, n_bags, 0u};
   for (long long j = (long long)vblock * blockDim.x + threadIdx.x; j < n_ids; j += stride) (void)rows.file(j);
 }
 __global__ void __launch_bounds__(256)
@@ -221,9 +221,8 @@ __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const f
     const uint32_t li = ordered ? wk.part_u[p] : team.owner_of_part(wk, n_long, p);
     if (!MONO_INDEX_OK(wk.error_bits, li, wk.max_long)) continue;
     const uint32_t u = wk.long_u[li], p0 = wk.long_part0[li];
-    const uint32_t row_word = wk.urow[u];
+    const uint32_t row_word = wk.urow[u], m = wk.ulen[u], seg = wk.useg[u];
     if (row_word == kNoRow) continue;                                    // no row: gradient dropped, by every part
-    const uint32_t m = wk.ulen[u], seg = wk.useg[u];
     uint32_t k = p - p0;
     const uint32_t begin = seg + k * kSegChunk, end = (k + 1) * kSegChunk < m ? begin + kSegChunk : seg + m;
     if (!MONO_INDEX_OK(wk.error_bits, (unsigned long long)end - 1, wk.max_ids)) continue;

@@ -191,12 +191,13 @@ struct ProbedRows {
 // A batch that was announced: every distinct ID was looked up then, and its slot of the per-call
 // set holds its row.  While it is there, every occurrence of a repeated ID is filed for the push:
 // its bag goes into the ID's segment of bag_of_sorted[], at the occurrence's rank.
+template <int P>
 struct FiledRows {
   const Work& wk;
   long long n_bags;
   uint32_t zero_row;
-  __device__ __forceinline__ uint32_t file(long long j) const {
-    const uint2 o = wk.occ[j];
+  __device__ __forceinline__ uint32_t file(long long j) const { return file(j, wk.occ[j]); }
+  __device__ __forceinline__ uint32_t file(long long j, const uint2 o) const {
     if (o.x == kNoSlot || !MONO_INDEX_OK(wk.error_bits, o.x, wk.n_slots)) return zero_row;
     const uint4 bs = __ldg(reinterpret_cast<const uint4*>(wk.bset + o.x));       // key (x, y), segment start, row
     if (bs.z != kNoSegment) {                                                     // (an ID that occurs once has no segment)
@@ -206,7 +207,30 @@ struct FiledRows {
     return bs.w != kNoRow ? bs.w : zero_row;
   }
   __device__ __forceinline__ void resolve(long long first, uint32_t n, uint32_t* dst) const {
-    for (uint32_t i = threadIdx.x; i < n; i += kPoolThreads) dst[i] = file(first + i);
+    for (uint32_t i = threadIdx.x; i < n; i += kPoolThreads * P) {
+      uint2 o[P];
+      uint4 bs[P];
+      uint32_t bag[P];
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        const uint32_t at = i + k * kPoolThreads;
+        o[k] = at < n ? wk.occ[first + at] : make_uint2(kNoSlot, 0u);
+        bag[k] = at < n ? wk.occ_bag[first + at] : 0xFFFFFFFFu;
+      }
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        bs[k] = make_uint4(0u, 0u, kNoSegment, kNoRow);
+        if (o[k].x != kNoSlot && MONO_INDEX_OK(wk.error_bits, o[k].x, wk.n_slots)) bs[k] = __ldg(reinterpret_cast<const uint4*>(wk.bset + o[k].x));
+      }
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        const uint32_t at = i + k * kPoolThreads;
+        if (at >= n) continue;
+        if (bs[k].z != kNoSegment && bag[k] < n_bags && MONO_INDEX_OK(wk.error_bits, (unsigned long long)bs[k].z + o[k].y, wk.max_ids))
+          wk.bag_of_sorted[bs[k].z + o[k].y] = bag[k];
+        dst[at] = bs[k].w != kNoRow ? bs[k].w : zero_row;
+      }
+    }
   }
 };
 
@@ -342,7 +366,10 @@ __device__ __forceinline__ void pool_tile_body(const TableView& tv, const Rows& 
 // all the warps an SM holds (213 000 bags of 32 columns 31.5 us against 36.9 with six blocks), wider
 // ones with the registers for more rows in flight (long bags of 64 columns 22.7 against 25 us).
 template <int G, int NV, int VW> constexpr int pool_blocks_per_sm() { return NV > 1 ? 4 : G <= 8 ? 8 : 6; }
+// (Filing is a chain of two reads, a batch's own record and its ID's slot of the per-call set: four at a time, 8 M IDs of
+// 64 columns 1365 -> 1348 us per step; at the 32 registers of the narrow rows they spill, 4 M IDs 343 -> 359.)
 template <int G> constexpr int kProbesInFlight = G <= 8 ? 1 : 2;
+template <int G> constexpr int kFiledInFlight = G <= 8 ? 1 : 4;
 
 template <int G, int NV, int VW>
 __global__ void __launch_bounds__(kPoolThreads, (pool_blocks_per_sm<G, NV, VW>()))
@@ -355,7 +382,7 @@ template <int G, int NV, int VW>
 __global__ void __launch_bounds__(kPoolThreads, (pool_blocks_per_sm<G, NV, VW>()))
 gather_pool_kernel(TableView tv, Work wk, uint32_t* __restrict__ spill, long long n_ids, const long long* __restrict__ offsets,
                  long long n_bags, float* __restrict__ out, uint32_t tile_bags) { after_previous_kernel();
-  pool_tile_body<G, NV, VW>(tv, FiledRows{wk, n_bags, (uint32_t)tv.capacity}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x);
+  pool_tile_body<G, NV, VW>(tv, FiledRows<kFiledInFlight<G>>{wk, n_bags, (uint32_t)tv.capacity}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x);
 }
 
 }  // namespace mono
