@@ -8,6 +8,29 @@
 
 namespace mono {
 
+// The rest of a read-only look-up that missed the preferred cell, for pulls that are bound by latency: the
+// seven other keys of both buckets are asked for together.
+__device__ inline bool thread_lookup_rest(const TableView& tv, unsigned long long id, unsigned stash_hw, unsigned long long* meta) {
+  const unsigned long long h0 = tv.hash0(id);
+  const uint32_t first = (uint32_t)(h0 >> 62);
+  const Cell* b0 = tv.cells + (h0 & tv.bucket_mask) * kCellsPerBucket;
+  const Cell* b1 = tv.cells + tv.bucket1(id) * kCellsPerBucket;
+  unsigned long long k0[3], k1[4];
+#pragma unroll
+  for (uint32_t k = 0; k < 3; ++k) k0[k] = __ldg(&b0[(first + 1u + k) & 3u].key);
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) k1[k] = __ldg(&b1[k].key);
+  const Cell* at = nullptr;
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) if (k1[k] == id) at = b1 + k;
+#pragma unroll
+  for (uint32_t k = 0; k < 3; ++k) if (k0[k] == id) at = b0 + ((first + 1u + k) & 3u);
+  for (unsigned i = 0; at == nullptr && i < stash_hw; ++i)
+    if (__ldg(&tv.stash[i].key) == id) at = tv.stash + i;
+  if (at) *meta = __ldg(&at->meta);
+  return at != nullptr;
+}
+
 // Read-only look-up by one thread.  An insertion tries the cell named by the
 // top bits of the hash first, so that cell is read first and alone; the other
 // three cells of the bucket, the second bucket and the stash follow only on a
@@ -53,17 +76,23 @@ __device__ inline unsigned long long thread_locate(const TableView& tv, unsigned
   const uint32_t first = (uint32_t)(h0 >> 62);
   const Cell c0 = load_cell_whole(tv.cells + base0 + first);
   if (c0.key == id) { *meta = c0.meta; return base0 + first; }
+  // On a miss the keys of the other three cells are asked for together, then those of the second
+  // bucket: most of these IDs are new to the table and in neither bucket, and a warp waits for its
+  // slowest lane, so eight reads one after the other were what the look-up took (a key store at load 0.89:
+  // 50 -> 42 us for 300 000 distinct IDs; all seven keys at once read a line more than most need: 48).
+  unsigned long long at = kNoCell, k0[3], k1[4];
 #pragma unroll
-  for (uint32_t k = 1; k < kCellsPerBucket; ++k) {
-    const Cell c = load_cell_whole(tv.cells + base0 + ((first + k) & 3u));
-    if (c.key == id) { *meta = c.meta; return base0 + ((first + k) & 3u); }
-  }
-  const unsigned long long base1 = tv.bucket1(id) * kCellsPerBucket;
+  for (uint32_t k = 0; k < 3; ++k) k0[k] = tv.cells[base0 + ((first + 1u + k) & 3u)].key;
 #pragma unroll
-  for (uint32_t k = 0; k < kCellsPerBucket; ++k) {
-    const Cell c = load_cell_whole(tv.cells + base1 + k);
-    if (c.key == id) { *meta = c.meta; return base1 + k; }
+  for (uint32_t k = 0; k < 3; ++k) if (k0[k] == id) at = base0 + ((first + 1u + k) & 3u);
+  if (at == kNoCell) {
+    const unsigned long long base1 = tv.bucket1(id) * kCellsPerBucket;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) k1[k] = tv.cells[base1 + k].key;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) if (k1[k] == id) at = base1 + k;
   }
+  if (at != kNoCell) { *meta = tv.cells[at].meta; return at; }
   for (unsigned i = 0; i < stash_hw; ++i) {
     const Cell s = load_cell_whole(tv.stash + i);
     if (s.key == id) { *meta = s.meta; return (tv.bucket_mask + 1) * kCellsPerBucket + i; }
@@ -158,7 +187,7 @@ __device__ __forceinline__ void pool_bag(const float* __restrict__ rows, uint32_
 //
 // A batch that was not announced: every occurrence is looked up in the key store.  The preferred
 // cells of P occurrences are asked for together; the rest of a look-up follows only on a miss.
-template <int P>
+template <int P, bool TOGETHER>
 struct ProbedRows {
   const TableView& tv;
   const unsigned long long* __restrict__ ids;
@@ -181,7 +210,7 @@ struct ProbedRows {
       for (int k = 0; k < P; ++k) {
         if (i + k * kPoolThreads >= n) continue;
         bool found = id[k] != kEmptyKey;
-        if (found && c[k].key != id[k]) found = thread_lookup(tv, id[k], stash_hw, &c[k].meta);
+        if (found && c[k].key != id[k]) found = TOGETHER ? thread_lookup_rest(tv, id[k], stash_hw, &c[k].meta) : thread_lookup(tv, id[k], stash_hw, &c[k].meta);
         dst[i + k * kPoolThreads] = found && meta_resident(c[k].meta) ? meta_row(c[k].meta) : (uint32_t)tv.capacity;
       }
     }
@@ -371,11 +400,14 @@ template <int G, int NV, int VW> constexpr int pool_blocks_per_sm() { return NV 
 template <int G> constexpr int kProbesInFlight = G <= 8 ? 1 : 2;
 template <int G> constexpr int kFiledInFlight = G <= 8 ? 1 : 4;
 
-template <int G, int NV, int VW>
-__global__ void __launch_bounds__(kPoolThreads, (pool_blocks_per_sm<G, NV, VW>()))
+// TOGETHER (launch_pool): of a look-up that misses the preferred cell, the rest at once.  It needs
+// the registers of six blocks per SM, which narrow rows only have to spare in a batch of one wave of blocks
+// (one request of 208 bags 5.7 -> 4.8 us; 213 000 bags 31.8 -> 32.8, so larger ones look on bucket by bucket).
+template <int G, int NV, int VW, bool TOGETHER>
+__global__ void __launch_bounds__(kPoolThreads, (TOGETHER && G <= 8 ? 6 : pool_blocks_per_sm<G, NV, VW>()))
 probe_pool_kernel(TableView tv, const unsigned long long* __restrict__ ids, uint32_t* __restrict__ spill, long long n_ids,
                   const long long* __restrict__ offsets, long long n_bags, float* __restrict__ out, uint32_t tile_bags) { after_previous_kernel();
-  pool_tile_body<G, NV, VW>(tv, ProbedRows<kProbesInFlight<G>>{tv, ids, tv.st->stash_hw}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x);
+  pool_tile_body<G, NV, VW>(tv, ProbedRows<kProbesInFlight<G>, TOGETHER>{tv, ids, tv.st->stash_hw}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x);
 }
 
 template <int G, int NV, int VW>

@@ -123,7 +123,7 @@ struct AnyRows {
   const GroupItem& it;
   __device__ __forceinline__ void resolve(long long first, uint32_t n, uint32_t* dst) const {
     if (it.prepared) FiledRows<1>{it.wk, it.n_bags, (uint32_t)it.tv.capacity}.resolve(first, n, dst);
-    else ProbedRows<1>{it.tv, it.ids, it.tv.st->stash_hw}.resolve(first, n, dst);
+    else ProbedRows<1, false>{it.tv, it.ids, it.tv.st->stash_hw}.resolve(first, n, dst);
   }
 };
 

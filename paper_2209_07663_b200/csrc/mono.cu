@@ -358,7 +358,8 @@ int launch_pool(mono_table* t, const unsigned long long* ids, uint32_t* spill, i
     const uint32_t tile = pool_tile(n_ids, n_bags, grid_for(t, pool_blocks_per_sm<G, NV, VW>()), kPoolThreads / G);
     const unsigned blocks = (unsigned)((n_bags + tile - 1) / tile);
     if (filed) LAUNCH(t, K_POOL, launch_after(gather_pool_kernel<G, NV, VW>, blocks, kPoolThreads, t->stream, t->tv, t->wk, spill, n_ids, off, n_bags, out, tile));
-    else LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
+    else if (G > 8 || (int64_t)blocks <= grid_for(t, 6)) LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW, true>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
+    else LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW, (G > 8)>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
     CUDA_TRY(t, cudaGetLastError());
     return (int)MONO_OK;
   });
