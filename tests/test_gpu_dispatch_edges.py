@@ -148,3 +148,27 @@ def test_host_buffers_are_staged_in_turn():
     for k, (got, want) in enumerate(zip(outs, wants)):
         assert_vectors_close(got.numpy(), want, f"pull {k}")
     assert_state_equal(gpu, cpu)
+
+
+@pytest.mark.parametrize("dim", [16, 64])
+@pytest.mark.parametrize("repeats", [1, 64])
+def test_look_ups_find_entries_wherever_they_sit(dim, repeats):
+    """A key store at load 0.97: entries in their preferred cell, elsewhere in either bucket, and in the overflow
+    stash; unknown IDs too.  One batch is one wave of blocks, the other several."""
+    n = 3970
+    ids = wl.splitmix64(np.arange(1, n + 1, dtype=np.uint64))
+    w = np.random.default_rng(7).standard_normal((n, dim)).astype(f32)
+    t = mb.MonoTable(4096, dim, 1, 0, key_cells=4096, seed=5)
+    t.import_entries(ids, np.ones(n, np.uint32), np.zeros(n, np.int64), np.ones(n, np.uint8), w, np.zeros_like(w))
+    assert t.status()["error_bits"] == 0 and t.status()["n_evictions_total"] > 0
+    known = np.tile(ids, repeats)
+    flat = np.concatenate([known, wl.splitmix64(np.arange(10 ** 6, 10 ** 6 + 500, dtype=np.uint64))])
+    want = torch.from_numpy(np.concatenate([np.tile(w, (repeats, 1)), np.zeros((500, dim), f32)])).cuda()
+    d_ids = torch.from_numpy(flat.view(np.int64)).cuda()
+    d_off = torch.arange(flat.size + 1, device="cuda")
+    for announced in (False, True):
+        out = torch.full((flat.size, dim), float("nan"), device="cuda")
+        if announced:
+            mb.mono_prepare_push(t.handle, d_ids, flat.size, d_off, flat.size)
+        mb.mono_lookup_pool(t.handle, d_ids, flat.size, d_off, flat.size, out)
+        assert torch.equal(out, want), announced
