@@ -8,8 +8,11 @@
 #include <Python.h>
 
 #include <cstdint>
+#include <exception>
+#include <new>
 #include <vector>
 
+#include <ATen/PythonTorchFunctionTLS.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 namespace {
@@ -53,20 +56,34 @@ bool expects(Py_ssize_t got, Py_ssize_t want) {
   return false;
 }
 
-// Raw address of a tensor / int / None / anything binding._ptr knows.
+// A reference that is given back whichever way its scope is left.
+struct Owned {
+  PyObject* o;
+  explicit Owned(PyObject* p) : o(p) {}
+  Owned(const Owned&) = delete;
+  Owned& operator=(const Owned&) = delete;
+  ~Owned() { Py_XDECREF(o); }
+};
+
+// Whether x is a torch.Tensor (or Parameter) itself, with nobody listening to its methods: only then may its
+// fields be read here.  A subclass may answer for itself, and so may a torch function mode.
+bool plain_tensor(PyObject* x) { return THPVariable_CheckExact(x) && !at::impl::torch_function_mode_enabled(); }
+
+// Raw address of a tensor / int / None / anything binding._ptr knows.  What a plain tensor refuses
+// (one without storage: inside vmap, grad or jvp, sparse, opaque) is asked for again through Python, which says why.
 bool address(PyObject* x, ptr* out) {
-  if (THPVariable_Check(x)) {
-    const at::Tensor& t = THPVariable_Unpack(x);
-    if (!t.is_contiguous()) { PyErr_SetString(PyExc_ValueError, "tensors passed to the C ABI must be contiguous"); return false; }
-    *out = t.data_ptr();
-    return true;
+  if (plain_tensor(x)) {
+    try {
+      const at::Tensor& t = THPVariable_Unpack(x);
+      if (t.is_contiguous()) { *out = t.data_ptr(); return true; }
+    } catch (const std::exception&) {
+    }
   }
   if (x == Py_None) { *out = nullptr; return true; }
   if (!PyLong_Check(x)) {
-    PyObject* r = PyObject_CallOneArg(g_address_of, x);
-    if (!r) return false;
-    *out = PyLong_AsVoidPtr(r);
-    Py_DECREF(r);
+    const Owned r(PyObject_CallOneArg(g_address_of, x));
+    if (!r.o) return false;
+    *out = PyLong_AsVoidPtr(r.o);
     return !PyErr_Occurred();
   }
   *out = PyLong_AsVoidPtr(x);
@@ -80,11 +97,29 @@ bool integer(PyObject* x, i64* out) {
 
 template <typename C>
 PyObject* without_gil(C&& call) {
+  struct Released {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Released() { PyEval_RestoreThread(state); }
+  };
   int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = call();
-  Py_END_ALLOW_THREADS
+  { const Released released; rc = call(); }
   return PyLong_FromLong(rc);
+}
+
+// Every method is entered through this: a C++ exception that left one would end the process.
+using Method = PyObject* (*)(PyObject*, PyObject* const*, Py_ssize_t);
+template <Method F>
+PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t n) noexcept {
+  try {
+    return F(self, args, n);
+  } catch (const std::bad_alloc&) {
+    return PyErr_NoMemory();
+  } catch (const std::exception& e) {
+    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+  } catch (...) {
+    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
+  }
+  return nullptr;
 }
 
 // (t, ids, n_ids, offsets, n_bags)
@@ -141,21 +176,27 @@ PyObject* fence(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 // Pulls with the arguments of MonoTable.lookup_pool as they are: returns None, having done nothing,
-// unless ids and offsets are contiguous 64-bit tensors on the table's device, and out a tensor.
+// unless ids and offsets are contiguous 64-bit tensors on the table's device, and out a tensor, all of them plain.
 // (handle, device, ids, offsets, out)
 PyObject* table_pull(PyObject*, PyObject* const* a, Py_ssize_t n) {
   ptr t, out;
   i64 device;
   if (!expects(n, 5) || !address(a[0], &t) || !integer(a[1], &device)) return nullptr;
-  if (!THPVariable_Check(a[2]) || !THPVariable_Check(a[3]) || !THPVariable_Check(a[4])) Py_RETURN_NONE;
-  const at::Tensor &ids = THPVariable_Unpack(a[2]), &off = THPVariable_Unpack(a[3]);
-  for (const at::Tensor* x : {&ids, &off}) {
-    const bool words = x->scalar_type() == at::kLong || x->scalar_type() == at::kUInt64;
-    if (!words || !x->is_cuda() || x->get_device() != device || !x->is_contiguous()) Py_RETURN_NONE;
+  if (!plain_tensor(a[2]) || !plain_tensor(a[3]) || !plain_tensor(a[4])) Py_RETURN_NONE;
+  ptr pi, po;
+  i64 n_ids, n_bags;
+  try {
+    const at::Tensor &ids = THPVariable_Unpack(a[2]), &off = THPVariable_Unpack(a[3]);
+    for (const at::Tensor* x : {&ids, &off}) {
+      const bool words = x->scalar_type() == at::kLong || x->scalar_type() == at::kUInt64;
+      if (!words || !x->is_cuda() || x->get_device() != device || !x->is_contiguous()) Py_RETURN_NONE;
+    }
+    pi = ids.data_ptr(), po = off.data_ptr();
+    n_ids = ids.numel(), n_bags = off.numel() - 1;
+  } catch (const std::exception&) {
+    Py_RETURN_NONE;                                          // (no storage: the Python way says why)
   }
   if (!address(a[4], &out)) return nullptr;
-  ptr pi = ids.data_ptr(), po = off.data_ptr();
-  const i64 n_ids = ids.numel(), n_bags = off.numel() - 1;
   return without_gil([&] { return fn<int (*)(ptr, ptr, i64, ptr, i64, ptr)>(F_LOOKUP)(t, pi, n_ids, po, n_bags, out); });
 }
 
@@ -166,7 +207,8 @@ struct Group {
 };
 
 bool entries(PyObject* list, size_t n, std::vector<ptr>* p, std::vector<i64>* numel, i64 less) {
-  PyObject* seq = PySequence_Fast(list, "grouped calls take lists, one entry per table");
+  const Owned own(PySequence_Fast(list, "grouped calls take lists, one entry per table"));
+  PyObject* const seq = own.o;
   if (!seq) return false;
   bool ok = (size_t)PySequence_Fast_GET_SIZE(seq) == n;
   if (!ok) PyErr_SetString(PyExc_ValueError, "grouped calls take one batch per table");
@@ -176,13 +218,11 @@ bool entries(PyObject* list, size_t n, std::vector<ptr>* p, std::vector<i64>* nu
     PyObject* x = PySequence_Fast_GET_ITEM(seq, i);
     ok = address(x, &(*p)[i]);
     if (!ok || !numel) continue;
-    if (THPVariable_Check(x)) { (*numel)[i] = THPVariable_Unpack(x).numel() - less; continue; }
-    PyObject* r = PyObject_CallMethod(x, "numel", nullptr);
-    ok = r && integer(r, &(*numel)[i]);
-    Py_XDECREF(r);
+    if (plain_tensor(x)) { (*numel)[i] = THPVariable_Unpack(x).numel() - less; continue; }
+    const Owned r(PyObject_CallMethod(x, "numel", nullptr));
+    ok = r.o && integer(r.o, &(*numel)[i]);
     (*numel)[i] -= less;
   }
-  Py_DECREF(seq);
   return ok;
 }
 
@@ -226,7 +266,7 @@ PyObject* group_push(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
-#define FAST(f) reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(static_cast<PyObject* (*)(PyObject*, PyObject* const*, Py_ssize_t)>(f))), METH_FASTCALL, nullptr
+#define FAST(f) reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(static_cast<Method>(guarded<f>))), METH_FASTCALL, nullptr
 PyMethodDef kMethods[] = {
   {"bind", FAST(bind)},
   {"lookup_pool", FAST(pull<F_LOOKUP>)},
