@@ -886,9 +886,11 @@ int mono_prepare_push(mono_table* t, const uint64_t* ids, int64_t n_ids, const i
                         reinterpret_cast<const long long*>(slot_offsets), n_bags);
 }
 
+// (The grouped calls describe their tables in host vectors, which may not be there to be had: no C++ exception
+// may leave a C entry.)
 int mono_group_prepare_push(int32_t n_tables, mono_table* const* tables, const uint64_t* const* ids,
                             const int64_t* n_ids, const int64_t* const* slot_offsets, const int64_t* n_bags,
-                            void* group_stream) {
+                            void* group_stream) try {
   MONO_API_RANGE();
   int rc = group_check(n_tables, tables);
   if (rc != MONO_OK) return rc;
@@ -912,11 +914,13 @@ int mono_group_prepare_push(int32_t n_tables, mono_table* const* tables, const u
   for (int32_t i = 0; i < n_tables; ++i)
     if (p.items[i].active) tables[i]->prep = {ids[i], n_ids[i], slot_offsets[i], n_bags[i], true, false, false};
   return group_end(p, tables);
+} catch (const std::bad_alloc&) {
+  return MONO_ERR_NOMEM;
 }
 
 int mono_group_lookup_pool(int32_t n_tables, mono_table* const* tables, const uint64_t* const* ids,
                            const int64_t* n_ids, const int64_t* const* slot_offsets, const int64_t* n_bags,
-                           float* const* out, void* group_stream) {
+                           float* const* out, void* group_stream) try {
   MONO_API_RANGE();
   int rc = group_check(n_tables, tables);
   if (rc != MONO_OK) return rc;
@@ -949,11 +953,13 @@ int mono_group_lookup_pool(int32_t n_tables, mono_table* const* tables, const ui
   for (int32_t i = 0; i < n_tables; ++i)
     if (p.items[i].prepared && p.items[i].n_ids > 0) tables[i]->prep.filed = true;
   return group_end(p, tables);
+} catch (const std::bad_alloc&) {
+  return MONO_ERR_NOMEM;
 }
 
 int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const uint64_t* const* ids,
                            const int64_t* n_ids, const int64_t* const* slot_offsets, const int64_t* n_bags,
-                           const float* const* grad_pooled, int64_t now, void* group_stream) {
+                           const float* const* grad_pooled, int64_t now, void* group_stream) try {
   MONO_API_RANGE();
   int rc = group_check(n_tables, tables);
   if (rc != MONO_OK) return rc;
@@ -1006,6 +1012,8 @@ int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const ui
   CUDA_TRY(p.owner, cudaGetLastError());
   for (int32_t i = 0; i < n_tables; ++i) tables[i]->prep.valid = false;
   return group_end(p, tables);
+} catch (const std::bad_alloc&) {
+  return MONO_ERR_NOMEM;
 }
 
 static int expire_range(mono_table* t, int64_t now, uint32_t slice, uint32_t n_slices) {

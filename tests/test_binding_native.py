@@ -7,6 +7,8 @@ import sys
 
 import pytest
 
+from paper_2209_07663_b200 import binding as mb
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 # Every case runs in a process of its own, forked after the imports, because what is tested for is that it lives on.
@@ -100,3 +102,34 @@ def test_what_has_no_address_is_a_python_error(call, what, want):
 
 def test_a_torch_function_mode_hears_of_the_tensors():
     assert outcomes()["listened"] == "LookupError 3"
+
+
+# 2^23 tables (a block of zeros stands for each: nothing is read of it but its device) and room for half of the first
+# host vector that describes them.
+STARVED = """
+import ctypes, resource
+from paper_2209_07663_b200 import binding as mb
+lib = mb.load_library()
+n = 1 << 23
+mb.mono_group_prepare_push([], [], [])
+zeros = ctypes.create_string_buffer(1 << 16)
+tables = (ctypes.c_void_p * n)(*([ctypes.addressof(zeros)] * n))
+handles = [0] * n
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + 4 * n, resource.getrlimit(resource.RLIMIT_AS)[1]))
+empty = ctypes.c_void_p()
+print(lib.mono_group_prepare_push(n, tables, empty, empty, empty, empty, empty))
+print(lib.mono_group_lookup_pool(n, tables, empty, empty, empty, empty, empty, empty))
+print(lib.mono_group_apply_grads(n, tables, empty, empty, empty, empty, empty, 0, empty))
+try:
+    mb.mono_group_prepare_push(handles, handles, handles)
+except MemoryError:
+    print("MemoryError")
+"""
+
+
+def test_a_grouped_call_without_host_memory_is_an_error():
+    r = subprocess.run([sys.executable, "-c", STARVED], capture_output=True, text=True, timeout=600,
+                       env=dict(os.environ, PYTHONPATH=ROOT, CUDA_VISIBLE_DEVICES=""), cwd=ROOT)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split() == [str(mb.MONO_ERR_NOMEM)] * 3 + ["MemoryError"]
