@@ -53,7 +53,7 @@ enum {
   MONO_ERR_ARG = -1,    /* null or misaligned pointer, size out of range, bad option */
   MONO_ERR_TIME = -2,   /* `now` decreased or is outside [0, MONO_MAX_NOW] */
   MONO_ERR_CUDA = -3,   /* a CUDA runtime call failed; see mono_last_cuda_error */
-  MONO_ERR_NOMEM = -4,  /* device allocation failed */
+  MONO_ERR_NOMEM = -4,  /* device allocation failed, or the host memory a grouped call describes its tables in */
   MONO_ERR_SIZE = -5,   /* caller buffer too small (mono_export) */
   MONO_ERR_LIMIT = -6   /* the call is larger than the fixed maximum of an entry point that
                            never allocates (mono_lookup_pool_noalloc) */

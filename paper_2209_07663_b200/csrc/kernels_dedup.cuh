@@ -50,9 +50,11 @@ struct Work {
   // is small enough to stay in L2 for a batch with the usual share of repeats;
   // an ID that finds no free slot among its first kPrimaryProbes positions there
   // goes to the secondary tier, which alone can hold a batch of all-distinct IDs.
-  BatchSlot* bset;           // [primary_mask + 1 + secondary_mask + 1]
-  uint32_t primary_mask;     // primary tier: slots [0, primary_mask]
-  uint32_t secondary_mask;   // secondary tier: slots primary_mask + 1 + [0, secondary_mask]
+  BatchSlot* bset;           // [n_slots()]
+  uint32_t primary_mask;     // primary tier: slots [0, primary_mask]; goes by the batch (primary_mask_for on the host), so that a
+                             //               small one in a large reservation wipes only what it may have used
+  uint32_t secondary_base;   // secondary tier: slots secondary_base + [0, secondary_mask], behind the primary tier of the
+                             //               largest batch
   uint2* occ;                // [max_ids] per occurrence: x = slot of its ID (kNoSlot if padding / outside bags),
                              //           y = rank of the occurrence among those of its ID
   uint32_t* occ_bag;         // [max_ids] bag of each occurrence
@@ -77,8 +79,9 @@ struct Work {
   uint32_t* part_done;       // [max_parts] partial sums that are there, counted at the first of the kFanIn that belong together; zero between calls
   uint32_t max_long, max_parts;
   uint32_t max_ids;          // entries of the per-occurrence and per-distinct-ID arrays
-  uint32_t n_slots;          // slots of bset, both tiers
+  uint32_t secondary_mask;
   unsigned int* error_bits;  // the table's sticky condition bits (the checked build reports through them)
+  __host__ __device__ unsigned long long n_slots() const { return (unsigned long long)secondary_base + secondary_mask + 1; }
 };
 
 // A bag is well formed when 0 <= offsets[b] <= offsets[b+1] <= n_ids; any other bag is
@@ -223,7 +226,7 @@ __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long*
     if (!placed) {
       // secondary tier: it has at least twice as many slots as a call has IDs, so
       // an empty slot is always reached; the bound only guards against misuse
-      const uint32_t base2 = wk.primary_mask + 1u;
+      const uint32_t base2 = wk.secondary_base;
       uint32_t q = (uint32_t)(mix_a(id ^ seed) >> 24) & wk.secondary_mask;
       for (uint32_t probe = 0; probe <= wk.secondary_mask; ++probe) {
         kk = *reinterpret_cast<volatile unsigned long long*>(&wk.bset[base2 + q].key);

@@ -227,7 +227,7 @@ struct FiledRows {
   uint32_t zero_row;
   __device__ __forceinline__ uint32_t file(long long j) const { return file(j, wk.occ[j]); }
   __device__ __forceinline__ uint32_t file(long long j, const uint2 o) const {
-    if (o.x == kNoSlot || !MONO_INDEX_OK(wk.error_bits, o.x, wk.n_slots)) return zero_row;
+    if (o.x == kNoSlot || !MONO_INDEX_OK(wk.error_bits, o.x, wk.n_slots())) return zero_row;
     const uint4 bs = __ldg(reinterpret_cast<const uint4*>(wk.bset + o.x));       // key (x, y), segment start, row
     if (bs.z != kNoSegment) {                                                     // (an ID that occurs once has no segment)
       const uint32_t bag = wk.occ_bag[j];
@@ -249,7 +249,7 @@ struct FiledRows {
 #pragma unroll
       for (int k = 0; k < P; ++k) {
         bs[k] = make_uint4(0u, 0u, kNoSegment, kNoRow);
-        if (o[k].x != kNoSlot && MONO_INDEX_OK(wk.error_bits, o[k].x, wk.n_slots)) bs[k] = __ldg(reinterpret_cast<const uint4*>(wk.bset + o[k].x));
+        if (o[k].x != kNoSlot && MONO_INDEX_OK(wk.error_bits, o[k].x, wk.n_slots())) bs[k] = __ldg(reinterpret_cast<const uint4*>(wk.bset + o[k].x));
       }
 #pragma unroll
       for (int k = 0; k < P; ++k) {

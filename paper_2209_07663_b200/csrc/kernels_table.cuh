@@ -164,7 +164,7 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
       id = wk.uid[u];
       if (MODE & kLookUp) {
         slot = wk.uslot[u];
-        if (!MONO_INDEX_OK(wk.error_bits, slot, wk.n_slots)) slot = 0;
+        if (!MONO_INDEX_OK(wk.error_bits, slot, wk.n_slots())) slot = 0;
         m = wk.bset[slot].a;
         cell = thread_locate(tv, id, stash_hw, &meta);
       } else {

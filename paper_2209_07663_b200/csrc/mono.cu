@@ -231,12 +231,35 @@ void join_sweep(mono_table* t) {
 int discard_prepared(mono_table* t) {
   if (!t->prep.valid) return MONO_OK;
   t->prep.valid = false;
-  const uint64_t slots = (uint64_t)t->wk.primary_mask + 1 + (uint64_t)t->wk.secondary_mask + 1;
   if (t->prep.ordered) CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_aux, 0));
-  init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(t->wk.bset, slots);
+  init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(t->wk.bset, t->wk.n_slots());
   forget_call_kernel<<<1, 256, 0, t->stream>>>(t->tv.st, t->wk);
   CUDA_TRY(t, cudaGetLastError());
   return MONO_OK;
+}
+
+// Slots of the primary tier of the per-call set for a batch.  It holds the distinct IDs, a quarter to all of the
+// batch's IDs.  Up to 2^21 IDs a slot per ID still fits L2 (at most 32 MB); beyond, two slots per five IDs, which
+// long-tailed batches of that size fill to a half: more would leave L2 and take longer to wipe.  (297 000 IDs
+// with 129 000 distinct ones filled 2^17 slots to the brim: dedup_tile 31 us there, 16 us with 2^19.)
+uint64_t primary_slots(int64_t n_ids) {
+  const uint64_t slots = next_pow2(n_ids <= (1 << 21) ? (uint64_t)n_ids : ((uint64_t)n_ids * 2) / 5);
+  return slots < 1024 ? 1024 : slots;
+}
+
+// The scratch as a batch of n_ids uses it: the same for its grouping, its pull and its push.  A batch below the
+// reservation gets up to eight times its own tier of the reserved one, while that is at most 16 MB: the emptier, the fewer
+// collisions, and the wipe of 16 MB does not show yet.  (20 600 IDs, reserved 2^18: 36.2 us a step, against 39.4 with a slot
+// per ID; 164 000 IDs 51.3 with 32 MB, 48.3 with 16.)  More is all wipe, by the few blocks of a small batch: 168 IDs in a
+// reservation of 2^21 took 294 us with the whole tier, 28 with their own.
+uint32_t primary_mask_for(const Work& w, int64_t n_ids) {
+  const uint64_t own = primary_slots(n_ids), roomy = std::max(own, std::min<uint64_t>(8 * own, 1 << 20));
+  return (uint32_t)std::min<uint64_t>(roomy, w.secondary_base) - 1u;
+}
+Work work_for(const mono_table* t, int64_t n_ids) {
+  Work w = t->wk;
+  w.primary_mask = primary_mask_for(w, n_ids);
+  return w;
 }
 
 int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
@@ -256,12 +279,7 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   free_scratch(t);
   Work& w = t->wk;
   const size_t n = (size_t)max_ids;
-  // The primary tier holds the distinct IDs of a batch, a quarter to all of its IDs.  Up to 2^21 IDs
-  // a slot per ID still fits L2 (at most 32 MB); beyond, two slots per five IDs, which long-tailed
-  // batches of that size fill to a half: more would leave L2 and take longer to wipe.  (297 000 IDs
-  // with 129 000 distinct ones filled 2^17 slots to the brim: dedup_tile 31 us there, 16 us with 2^19.)
-  uint64_t primary = next_pow2(max_ids <= (1 << 21) ? (uint64_t)max_ids : ((uint64_t)max_ids * 2) / 5);
-  if (primary < 1024) primary = 1024;
+  const uint64_t primary = primary_slots(max_ids);
   const uint64_t secondary = next_pow2(2 * (uint64_t)max_ids);
   const uint64_t slots = primary + secondary;
   int rc;
@@ -280,9 +298,9 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   ALLOC(t->occ_row, n);
 #undef ALLOC
   w.primary_mask = (uint32_t)(primary - 1);
+  w.secondary_base = (uint32_t)primary;
   w.secondary_mask = (uint32_t)(secondary - 1);
   w.max_ids = (uint32_t)max_ids;
-  w.n_slots = (uint32_t)slots;
   w.error_bits = &t->tv.st->error_bits;
   init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(w.bset, slots);
   CUDA_TRY(t, cudaGetLastError());
@@ -446,7 +464,7 @@ int launch_prepare(mono_table* t, const unsigned long long* ids, int64_t n_ids, 
     std::swap(w.bset, ah.bset); std::swap(w.occ, ah.occ); std::swap(w.occ_bag, ah.occ_bag);
     std::swap(w.uid, ah.uid); std::swap(w.uslot, ah.uslot); std::swap(w.uocc, ah.uocc); std::swap(w.call, ah.call);
   } else {
-    const int rc = launch_group(t, t->stream, ids, n_ids, off, n_bags, w);
+    const int rc = launch_group(t, t->stream, ids, n_ids, off, n_bags, work_for(t, n_ids));
     if (rc != MONO_OK) return rc;
   }
   const bool ordered = orders_parts(t, n_bags);
@@ -461,7 +479,7 @@ int launch_apply(mono_table* t, const unsigned long long* ids, int64_t n_ids, co
                  int64_t n_bags, const float* grad, uint32_t now, cudaEvent_t grad_ready = nullptr) {
   cudaStream_t s = t->stream;
   const TableView& tv = t->tv;
-  const Work& wk = t->wk;
+  const Work wk = work_for(t, n_ids);
   int rc = MONO_OK;
   bool ordered;
   if (is_prepared_batch(t, ids, n_ids, off, n_bags)) {
@@ -611,6 +629,7 @@ void group_describe(GroupPlan& p, int32_t i, mono_table* t, const uint64_t* ids,
                     int64_t n_bags, float* out, const float* grad, uint32_t now, bool prepared) {
   GroupItem& it = p.items[i];
   it.tv = t->tv; it.wk = t->wk;
+  it.wk.primary_mask = primary_mask_for(t->wk, n_ids);
   it.ids = reinterpret_cast<const unsigned long long*>(ids);
   it.off = reinterpret_cast<const long long*>(off);
   it.n_ids = n_ids; it.n_bags = n_bags; it.out = out; it.grad = grad; it.now = now;
@@ -828,8 +847,7 @@ int mono_group_ahead(mono_table* t, const uint64_t* ids, int64_t n_ids, const in
   auto& ah = t->ahead;
   // while kernels are being timed one by one, the grouping runs on the table's stream like everything else
   cudaStream_t g = t->timing ? t->stream : t->ahead_stream;
-  const Work& w = t->wk;
-  const uint64_t slots = (uint64_t)w.primary_mask + 1 + (uint64_t)w.secondary_mask + 1;
+  const uint64_t slots = t->wk.n_slots();
   // The grouping follows what the table's stream holds so far: whatever fills the batch's arrays,
   // and the kernels that still use the copy of the scratch handed back at the last exchange.
   if (g != t->stream) {
@@ -863,7 +881,7 @@ int mono_group_ahead(mono_table* t, const uint64_t* ids, int64_t n_ids, const in
     CUDA_TRY(t, cudaMemsetAsync(ah.call, 0, sizeof(CallState), g));
   }
   if (n_ids == 0 || n_bags == 0) return MONO_OK;
-  Work into = w;
+  Work into = work_for(t, n_ids);
   into.bset = ah.bset; into.occ = ah.occ; into.occ_bag = ah.occ_bag; into.uid = ah.uid; into.uslot = ah.uslot; into.uocc = ah.uocc;
   into.call = ah.call;
   if ((rc = launch_group(t, g, reinterpret_cast<const unsigned long long*>(ids), n_ids,
