@@ -1,6 +1,6 @@
 """B200-native collisionless embedding table (the hot path of Monolith, arXiv 2209.07663).
 
-`binding` is the thin ctypes layer over the C ABI of include/mono.h;
+`binding` is the thin layer over the C ABI of include/mono.h;
 `workload` draws seeded synthetic ID streams; `build` compiles the CUDA library.
 """
 from . import workload  # noqa: F401

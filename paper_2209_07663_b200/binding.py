@@ -1,16 +1,19 @@
-"""ctypes binding of the C ABI in include/mono.h.
+"""Binding of the C ABI in include/mono.h.
 
 Marshals arguments only: tensors become raw pointers, options become the C
 structs, return codes become exceptions.  Every step of the table's work runs in
 the CUDA library.  There is no fallback: if libmono.so is missing, loading
 raises.  The calls that a training or serving loop makes each step go through a
 small CPython extension (csrc/binding_native.cpp) instead of ctypes: on a small
-batch the host is what bounds them.
+batch the host is what bounds them.  A program that has not imported torch has no
+tensors to pass; it needs neither torch nor the extension, and all its calls go
+through ctypes.
 """
 from __future__ import annotations
 
 import ctypes
 import os
+import sys
 from typing import Optional
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
@@ -84,11 +87,12 @@ def _struct_dict(s: ctypes.Structure) -> dict:
 
 _lib = None
 _native = None          # csrc/binding_native.cpp, bound to the functions of the loaded library
+_portable = None        # the same calls through ctypes, for a program without torch
 
 
 def load_library(path: Optional[str] = None):
     """Load libmono.so and declare its prototypes.  Raises if it is not there."""
-    global _lib, _native
+    global _lib, _native, _portable
     if _lib is not None and path is None:
         return _lib
     path = path or LIB_PATH
@@ -134,13 +138,11 @@ def load_library(path: Optional[str] = None):
     for name, (res, args) in proto.items():
         fn = getattr(L, name)
         fn.restype, fn.argtypes = res, args
-    native = _load_native()
-    native.bind({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in proto}, _ptr)
-    _lib, _native = L, native
+    _lib, _native, _portable = L, None, None
     return L
 
 
-def _load_native():
+def _load_native(L):
     import importlib.util
     path = os.path.join(_PKG, "_binding_native.so")
     if not os.path.exists(path):
@@ -149,14 +151,50 @@ def _load_native():
     spec = importlib.util.spec_from_file_location("_binding_native", path)
     module = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(module)
+    module.bind({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in EXPORTS}, _ptr)
     return module
 
 
+class _Portable:
+    """The methods of csrc/binding_native.cpp through ctypes."""
+
+    def __init__(self, L):
+        for name in ("lookup_pool", "lookup_pool_noalloc", "lookup_pool_host", "apply_grads", "apply_grads_host",
+                     "prepare_push", "group_ahead", "expire", "expire_slice", "fence"):
+            fn = getattr(L, "mono_" + name)
+            setattr(self, name, lambda *args, fn=fn: fn(*map(_ptr, args)))
+        self._lib = L
+
+    @staticmethod
+    def _group(handles, ids, slot_offsets, vectors):
+        n = len(handles)
+        if not (len(ids) == len(slot_offsets) == len(vectors) == n):
+            raise ValueError("grouped calls take one batch per table")
+        ptrs, i64s = ctypes.c_void_p * n, ctypes.c_int64 * n
+        return (n, ptrs(*handles), ptrs(*map(_ptr, ids)), i64s(*[x.numel() for x in ids]),
+                ptrs(*map(_ptr, slot_offsets)), i64s(*[x.numel() - 1 for x in slot_offsets]), ptrs(*map(_ptr, vectors)))
+
+    def group_prepare_push(self, handles, ids, slot_offsets, stream):
+        return self._lib.mono_group_prepare_push(*self._group(handles, ids, slot_offsets, ids)[:-1], stream or None)
+
+    def group_lookup_pool(self, handles, ids, slot_offsets, outs, stream):
+        return self._lib.mono_group_lookup_pool(*self._group(handles, ids, slot_offsets, outs), stream or None)
+
+    def group_apply_grads(self, handles, ids, slot_offsets, grads, now, stream):
+        return self._lib.mono_group_apply_grads(*self._group(handles, ids, slot_offsets, grads), now, stream or None)
+
+
 def _hot():
-    """The native module, loading the library first if nothing has."""
-    if _native is None:
-        load_library()
-    return _native
+    """The hot calls of the loaded library (which is loaded first if nothing has): native in a program that has
+    imported torch, through ctypes in one that has not, or not yet."""
+    global _native, _portable
+    L = load_library()
+    if sys.modules.get("torch") is not None:
+        _native = _load_native(L)
+        return _native
+    if _portable is None:
+        _portable = _Portable(L)
+    return _portable
 
 
 def error_string(code: int) -> str:
@@ -426,7 +464,7 @@ class MonoTable:
     def lookup_pool(self, ids, offsets, out=None):
         if out is not None:
             # tensors that are where and what the call needs go straight to it (None: they are not)
-            rc = _native.table_pull(self.handle, self._device, ids, offsets, out)
+            rc = (_native or _hot()).table_pull(self.handle, self._device, ids, offsets, out)
             if rc is not None:
                 if rc:
                     _check("mono_lookup_pool", rc, self.handle)

@@ -133,3 +133,44 @@ def test_a_grouped_call_without_host_memory_is_an_error():
                        env=dict(os.environ, PYTHONPATH=ROOT, CUDA_VISIBLE_DEVICES=""), cwd=ROOT)
     assert r.returncode == 0, r.stderr[-2000:]
     assert r.stdout.split() == [str(mb.MONO_ERR_NOMEM)] * 3 + ["MemoryError"]
+
+
+# What a caller with arrays and addresses needs is the library alone.
+WITHOUT_TORCH = """
+import os, sys
+if sys.argv[1] == "absent":
+    sys.modules["torch"] = None                     # import torch raises
+import numpy as np
+from paper_2209_07663_b200 import binding as mb
+mb.load_library()
+ids, off, out = np.zeros(4, np.uint64), np.array([0, 4]), np.zeros(4, np.float32)
+calls = [lambda: mb.mono_lookup_pool_host(0, ids, 4, off, 1, out), lambda: mb.mono_apply_grads_host(0, ids, 4, off, 1, out, 0),
+         lambda: mb.mono_lookup_pool(0, 4096, 4, 4096, 1, 4096), lambda: mb.mono_lookup_pool_noalloc(0, ids, 4, off, 1, out),
+         lambda: mb.mono_apply_grads(0, ids, 4, off, 1, out, 0), lambda: mb.mono_prepare_push(0, ids, 4, off, 1),
+         lambda: mb.mono_group_ahead(0, ids, 4, off, 1), lambda: mb.mono_expire(0, 1), lambda: mb.mono_expire_slice(0, 1, 0, 4),
+         lambda: mb.mono_fence(0), lambda: mb.mono_apply_grads(0, ids[::2], 2, off, 1, out, 0)]
+def all_of_them():
+    for call in calls:
+        try:
+            call()
+        except Exception as e:
+            print(type(e).__name__)
+all_of_them()
+mb.mono_group_prepare_push([], [], [])
+mb.mono_group_lookup_pool([], [], [], [])
+mb.mono_group_apply_grads([], [], [], [], 0)
+print(sys.modules.get("torch") is None, mb._native is None)
+if sys.argv[1] == "later":
+    import torch
+    all_of_them()
+    print(sys.modules.get("torch") is None, mb._native is None)
+"""
+
+
+@pytest.mark.parametrize("torch_is", ["absent", "later"])
+def test_arrays_need_neither_torch_nor_the_extension(torch_is):
+    r = subprocess.run([sys.executable, "-c", WITHOUT_TORCH, torch_is], capture_output=True, text=True, timeout=600,
+                       env=dict(os.environ, PYTHONPATH=ROOT, CUDA_VISIBLE_DEVICES=""), cwd=ROOT)
+    assert r.returncode == 0, r.stderr[-2000:]
+    each = ["MonoError"] * 10 + ["ValueError"]
+    assert r.stdout.split() == each + ["True", "True"] + (each + ["False", "False"] if torch_is == "later" else [])
