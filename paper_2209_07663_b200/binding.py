@@ -144,10 +144,10 @@ def load_library(path: Optional[str] = None):
 
 def _load_native(L):
     import importlib.util
-    path = os.path.join(_PKG, "_binding_native.so")
+    from .build import native_path
+    path = native_path()
     if not os.path.exists(path):
         raise RuntimeError(f"{path} is missing: build it with `python -m paper_2209_07663_b200.build`")
-    import torch  # noqa: F401  (the extension links against its libraries)
     spec = importlib.util.spec_from_file_location("_binding_native", path)
     module = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(module)

@@ -174,3 +174,21 @@ def test_arrays_need_neither_torch_nor_the_extension(torch_is):
     assert r.returncode == 0, r.stderr[-2000:]
     each = ["MonoError"] * 10 + ["ValueError"]
     assert r.stdout.split() == each + ["True", "True"] + (each + ["False", "False"] if torch_is == "later" else [])
+
+
+def test_another_torch_gets_an_extension_of_its_own(monkeypatch):
+    from paper_2209_07663_b200 import build
+    import torch
+    mine, made = build.build_native(), []
+
+    def compiler(cmd):
+        made.append(cmd[cmd.index("-o") + 1])
+        open(made[-1], "w").close()
+    monkeypatch.setattr(build.subprocess, "check_call", compiler)
+    assert build.build_native() == mine and not made           # up to date
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    theirs = build.build_native()
+    os.unlink(theirs)
+    assert made and theirs != mine
+    with pytest.raises(RuntimeError, match="missing"):
+        mb._load_native(mb.load_library())
