@@ -393,8 +393,11 @@ __device__ __forceinline__ void pool_tile_body(const TableView& tv, const Rows& 
 
 // Blocks per SM and look-ups in flight per thread: narrow rows, whose groups are small, do best with
 // all the warps an SM holds (213 000 bags of 32 columns 31.5 us against 36.9 with six blocks), wider
-// ones with the registers for more rows in flight (long bags of 64 columns 22.7 against 25 us).
-template <int G, int NV, int VW> constexpr int pool_blocks_per_sm() { return NV > 1 ? 4 : G <= 8 ? 8 : 6; }
+// ones with the registers for more rows in flight (long bags of 64 columns 22.7 against 25 us).  Rows of more than
+// 512 columns in 32-byte accesses need 80 registers, three blocks: at the 64 of four they spill, and the pull of 2048 bags of
+// up to 64 IDs of 1024 columns took 54 us against 40, of 65 536 bags of up to 8 IDs 106 against 98.  (In 16-byte
+// accesses four stay: three are 50 -> 40 us for the long bags of 516 columns, but 72.7 -> 76.8 for the many short ones.)
+template <int G, int NV, int VW> constexpr int pool_blocks_per_sm() { return NV * VW == 32 && VW == 8 ? 3 : NV > 1 ? 4 : G <= 8 ? 8 : 6; }
 // (Filing is a chain of two reads, a batch's own record and its ID's slot of the per-call set: four at a time, 8 M IDs of
 // 64 columns 1365 -> 1348 us per step; at the 32 registers of the narrow rows they spill, 4 M IDs 343 -> 359.)
 template <int G> constexpr int kProbesInFlight = G <= 8 ? 1 : 2;

@@ -127,8 +127,11 @@ struct AnyRows {
   }
 };
 
+// (Three blocks per SM for the wide rows, whose bodies share the widest one's registers: eight tables of 260 to 512 columns
+// 72 -> 65 us with 8192 short bags each, 35 -> 33 with long bags, of 516 to 1024 columns 118 -> 107 and 59 -> 53,
+// of 132 to 256 49 -> 47 and 22.5, against four.)
 template <int WIDE>
-__global__ void __launch_bounds__(kPoolThreads, WIDE ? 4 : 6)
+__global__ void __launch_bounds__(kPoolThreads, WIDE ? 3 : 6)
 group_pool_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   const auto pool = [&](auto g, auto nv, auto vw) {
