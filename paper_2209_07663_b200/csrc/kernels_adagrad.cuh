@@ -129,7 +129,7 @@ __device__ inline void reduce_segment(const Work& wk, const float* __restrict__ 
 __device__ inline void file_segments_body(const Work& wk, long long n_ids, long long n_bags, uint32_t vblock, uint32_t vgrid) {
   const long long stride = (long long)vgrid * blockDim.x;
   const FiledRows<1> rows{wk, n_bags, 0u};
-  for (long long j = (long long)vblock * blockDim.x + threadIdx.x; j < n_ids; j += stride) (void)rows.file(j);
+  for (long long j = (long long)vblock * blockDim.x + threadIdx.x; j < n_ids; j += stride) rows.file(j);
 }
 __global__ void __launch_bounds__(256)
 file_segments_kernel(Work wk, long long n_ids, long long n_bags) { after_previous_kernel();

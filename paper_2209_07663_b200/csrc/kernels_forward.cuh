@@ -225,15 +225,20 @@ struct FiledRows {
   const Work& wk;
   long long n_bags;
   uint32_t zero_row;
-  __device__ __forceinline__ uint32_t file(long long j) const { return file(j, wk.occ[j]); }
-  __device__ __forceinline__ uint32_t file(long long j, const uint2 o) const {
-    if (o.x == kNoSlot || !MONO_INDEX_OK(wk.error_bits, o.x, wk.n_slots())) return zero_row;
-    const uint4 bs = __ldg(reinterpret_cast<const uint4*>(wk.bset + o.x));       // key (x, y), segment start, row
-    if (bs.z != kNoSegment) {                                                     // (an ID that occurs once has no segment)
-      const uint32_t bag = wk.occ_bag[j];
-      if (bag < n_bags && MONO_INDEX_OK(wk.error_bits, (unsigned long long)bs.z + o.y, wk.max_ids)) wk.bag_of_sorted[bs.z + o.y] = bag;
-    }
-    return bs.w != kNoRow ? bs.w : zero_row;
+  // An occurrence's slot of the per-call set: key (x, y), start of the ID's segment, row.
+  __device__ __forceinline__ uint4 slot_of(const uint2 o) const {
+    if (o.x == kNoSlot || !MONO_INDEX_OK(wk.error_bits, o.x, wk.n_slots())) return make_uint4(0u, 0u, kNoSegment, kNoRow);
+    return __ldg(reinterpret_cast<const uint4*>(wk.bset + o.x));
+  }
+  __device__ __forceinline__ void file(const uint2 o, const uint4 bs, uint32_t bag) const {
+    if (bs.z != kNoSegment && bag < n_bags && MONO_INDEX_OK(wk.error_bits, (unsigned long long)bs.z + o.y, wk.max_ids))
+      wk.bag_of_sorted[bs.z + o.y] = bag;                                         // (an ID that occurs once has no segment)
+  }
+  // The filing alone, of one occurrence.
+  __device__ __forceinline__ void file(long long j) const {
+    const uint2 o = wk.occ[j];
+    const uint4 bs = slot_of(o);
+    if (bs.z != kNoSegment) file(o, bs, wk.occ_bag[j]);
   }
   __device__ __forceinline__ void resolve(long long first, uint32_t n, uint32_t* dst) const {
     for (uint32_t i = threadIdx.x; i < n; i += kPoolThreads * P) {
@@ -247,16 +252,12 @@ struct FiledRows {
         bag[k] = at < n ? wk.occ_bag[first + at] : 0xFFFFFFFFu;
       }
 #pragma unroll
-      for (int k = 0; k < P; ++k) {
-        bs[k] = make_uint4(0u, 0u, kNoSegment, kNoRow);
-        if (o[k].x != kNoSlot && MONO_INDEX_OK(wk.error_bits, o[k].x, wk.n_slots())) bs[k] = __ldg(reinterpret_cast<const uint4*>(wk.bset + o[k].x));
-      }
+      for (int k = 0; k < P; ++k) bs[k] = slot_of(o[k]);
 #pragma unroll
       for (int k = 0; k < P; ++k) {
         const uint32_t at = i + k * kPoolThreads;
         if (at >= n) continue;
-        if (bs[k].z != kNoSegment && bag[k] < n_bags && MONO_INDEX_OK(wk.error_bits, (unsigned long long)bs[k].z + o[k].y, wk.max_ids))
-          wk.bag_of_sorted[bs[k].z + o[k].y] = bag[k];
+        file(o[k], bs[k], bag[k]);
         dst[at] = bs[k].w != kNoRow ? bs[k].w : zero_row;
       }
     }
@@ -269,8 +270,9 @@ struct FiledRows {
 //      many in flight as the block has threads;
 //   2. lane groups of G (chosen from dim, so that a lane owns NV vectors of VW floats) each add up
 //      a bag at a time, in ID order, so that the fp32 sum has one fixed order.
-// Bound by the latency of scattered reads (of 32 warp-cycles per issue 22 wait for memory; DRAM at
-// 45 % and L1 at 55 % of their peaks on the largest batch), so everything here is about reads in flight:
+// Bound by the latency of scattered reads (more than half of the warp-cycles per issue wait for memory, with DRAM at
+// about half and L1 at two thirds of their peaks on the largest announced batch: profiles/), so everything here
+// is about reads in flight:
 //  - blocks of one kernel are in both steps at any time, which two kernels one after the other never
 //    are, and the rows' indices do not travel through memory;
 //  - the tile's bags are put in order of length (a counting sort of at most 256 entries in shared
@@ -399,7 +401,7 @@ __device__ __forceinline__ void pool_tile_body(const TableView& tv, const Rows& 
 // accesses four stay: three are 50 -> 40 us for the long bags of 516 columns, but 72.7 -> 76.8 for the many short ones.)
 template <int G, int NV, int VW> constexpr int pool_blocks_per_sm() { return NV * VW == 32 && VW == 8 ? 3 : NV > 1 ? 4 : G <= 8 ? 8 : 6; }
 // (Filing is a chain of two reads, a batch's own record and its ID's slot of the per-call set: four at a time, 8 M IDs of
-// 64 columns 1365 -> 1348 us per step; at the 32 registers of the narrow rows they spill, 4 M IDs 343 -> 359.)
+// 64 columns 1365 -> 1346 us per step, timed in turn; at the 32 registers of the narrow rows they spill, 4 M IDs 343 -> 359.)
 template <int G> constexpr int kProbesInFlight = G <= 8 ? 1 : 2;
 template <int G> constexpr int kFiledInFlight = G <= 8 ? 1 : 4;
 
