@@ -292,7 +292,8 @@ def algorithmic_bytes(n, b, u, ur, ur1, unew, d, sweep_cells=0, prepared=True, e
         "table_insert": (16 + 8 * d) * unew,                 # key write + row/accumulator initialisation
         "sketch_add": 0,                                     # (probabilistic filter: counted with table_insert's new IDs)
         "update_singletons": 20 * d * ur1,                   # IDs seen once: gradient row, row and accumulator in and out
-        # rows of repeated IDs + the gradient rows the singletons did not read, once (update_rows_kernel does both)
+        # rows of repeated IDs + the gradient rows the singletons did not read, once (update_rows_kernel does both kinds,
+        # and is given the sum of the two where they are compared with its time)
         "reduce_adagrad": 16 * d * (ur - ur1) + 4 * d * max(b - ur1, 0), "update_rows": 0,
         "file_segments": 0, "expand_parts": 0, "order_parts": 0,
         # the sweep's 4-byte record per 4-cell bucket in order; a removed entry's bucket read (64) and its cell cleared (32)

@@ -338,7 +338,8 @@ int mono_expire_slice(mono_table* t, int64_t now, uint32_t slice, uint32_t n_sli
  *    pointers and sizes as the mono_lookup_pool_host call directly before it reuses that copy
  *    and that announcement -- the contents must not have changed in between; given anything
  *    else it copies its own.
- *  - The two bag-by-dim staging matrices are allocated by the first host-buffer call.
+ *  - The staging buffers (two bag-by-dim matrices, two sets of IDs and offsets that batches
+ *    take in turn) are allocated by the first host-buffer call.
  * All pointers HOST.
  */
 int mono_lookup_pool_host(mono_table* t, const uint64_t* ids, int64_t n_ids,
@@ -354,11 +355,12 @@ int mono_apply_grads_host(mono_table* t, const uint64_t* ids, int64_t n_ids,
  * Who needs it: code that runs where cudaMalloc is off limits -- inside a
  * serving loop whose memory budget was fixed at start-up, under an allocator
  * that owns the whole device, or in a process that has handed every spare
- * byte to other tenants.  mono_lookup_pool keeps its per-ID scratch (the row
- * index of every ID of the batch) in a buffer it grows with cudaMalloc when a
- * larger batch arrives; this entry point keeps the same scratch in a fixed
- * array that is part of the library image instead, so it never calls
- * cudaMalloc, cudaFree or anything else that allocates.
+ * byte to other tenants.  mono_lookup_pool keeps its per-ID scratch (a row
+ * index per ID, used by runs of bags with more IDs than a block's shared
+ * memory holds) in a buffer it grows with cudaMalloc when a larger batch
+ * arrives; this entry point keeps the same scratch in a fixed array that is
+ * part of the library image instead, so it never calls cudaMalloc, cudaFree or
+ * anything else that allocates.
  *
  *  - Same arguments, same result and same error codes as mono_lookup_pool.
  *  - n_ids may be at most MONO_NOALLOC_MAX_IDS; a larger batch is refused with
@@ -372,7 +374,7 @@ int mono_apply_grads_host(mono_table* t, const uint64_t* ids, int64_t n_ids,
  *  - The table's device must be the current device (MONO_ERR_ARG otherwise:
  *    another device's copy of the array would be the wrong memory).
  *  - With mono_timing_enable switched on, the call creates CUDA events for its
- *    two launches like every other hot call; leave timing off where even that
+ *    launch like every other hot call; leave timing off where even that
  *    is unwelcome.
  *  - All tables and all calls on a device share the one array, and it keeps
  *    whatever the previous call left in it.  Nothing in it needs clearing --

@@ -78,7 +78,7 @@ struct mono_table {
   cudaEvent_t ev_ahead = nullptr;   // the grouping on ahead_stream is done
   cudaEvent_t ev_swap = nullptr;    // what `stream` held when mono_group_ahead was called: the batch's arrays are
                                     // ready, and the copy of the scratch handed back at the last exchange is let go of
-  uint32_t* occ_row = nullptr;    // scratch of the two-kernel lookup: row of every occurrence
+  uint32_t* occ_row = nullptr;    // rows of the occurrences of a pull's tiles that do not fit their block's shared memory
   int device = 0;                 // the device the table lives on
   uint64_t scratch_reallocs = 0;  // times a hot call had to grow the scratch
   // Grouped calls (one launch over several tables): the first table of a group keeps the
