@@ -210,8 +210,7 @@ struct Team {
 // 11 000 parts of such an ID was a serial chain of 50 us.)
 template <int PG, int G, int NV>
 __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
-                                    bool ordered, uint32_t vblock, uint32_t vgrid) {
-  const unsigned long long longs = wk.call->longs;
+                                    bool ordered, unsigned long long longs, uint32_t vblock, uint32_t vgrid) {
   const uint32_t n_parts = (uint32_t)longs, n_long = (uint32_t)(longs >> 32);
   const Team<PG, G> team;
   const uint32_t teams = (vgrid * blockDim.x) / PG;
@@ -273,8 +272,7 @@ __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const f
 // of a step faster on the largest configuration.)
 template <int G, int NV>
 __device__ inline void reduce_short(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
-                                    uint32_t vblock, uint32_t vgrid) {
-  const uint32_t n = wk.call->n_multi;
+                                    uint32_t n, uint32_t vblock, uint32_t vgrid) {
   const int gl = threadIdx.x % G;
   const uint32_t groups = (vgrid * blockDim.x) / G;
   for (uint32_t item = (vblock * blockDim.x + threadIdx.x) / G; item < n; item += groups) {
@@ -306,14 +304,13 @@ __device__ inline void reduce_short(const TableView& tv, const Work& wk, const f
 // back updated.
 template <int G, int NV>
 __device__ inline void update_singletons(const TableView& tv, const Work& wk, const float* __restrict__ grad,
-                                              long long n_bags, uint32_t vblock, uint32_t vgrid) {
+                                              long long n_bags, uint32_t n, uint32_t vblock, uint32_t vgrid) {
   constexpr int kGroups = 32 / G;
   // Two rows of a lane group in flight (1.3 M single rows of 64 columns 5 % faster, whole step 1395 -> 1380 us; 99 000 of
   // 100 columns 137 -> 130); rows of several vectors per lane have their own loads to overlap.
   constexpr int kRows = NV == 1 ? 2 : 1;
   const int lane = threadIdx.x & 31;
   const int gl = lane % G, grp = lane / G;
-  const uint32_t n = wk.call->n_unique;
   const uint32_t n_warps = (vgrid * blockDim.x) >> 5;
   const uint32_t n_rounds = (n + 31) / 32;
   unsigned int n_single = 0;
@@ -396,20 +393,22 @@ struct RowGrid { uint32_t parts, shorts, singles; };
 template <int G, int NV, bool FEW>
 __device__ __forceinline__ void update_rows_body(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
                                                  bool ordered, const RowGrid& grid, uint32_t total_blocks, uint32_t vblock) {
+  __shared__ CheckIn call;
+  check_in(wk, &call);
   if (vblock < grid.parts) {
     // Few parts (they are resident all at once): a warp each, because the longest chain of loads is what
     // counts (step of 20 000 IDs 35.8 -> 28.4 us, of 135 000 56 -> 47).  Many: a lane group each, which
     // spends nothing on adding groups up (a warp each: 1 M IDs 154 -> 160 us, 4 M drifting 351 -> 370).
     // (A grouped call, whose tables share the SMs, has no use for it: FEW is false.)
-    if (G < 32 && (!FEW || (uint32_t)wk.call->longs > kFewParts)) reduce_parts<G, G, NV>(tv, wk, grad, n_bags, ordered, vblock, grid.parts);
-    else reduce_parts<32, G, NV>(tv, wk, grad, n_bags, ordered, vblock, grid.parts);
+    if (G < 32 && (!FEW || (uint32_t)call.longs > kFewParts)) reduce_parts<G, G, NV>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
+    else reduce_parts<32, G, NV>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
   } else if (vblock - grid.parts < grid.shorts) {
-    reduce_short<G, NV>(tv, wk, grad, n_bags, vblock - grid.parts, grid.shorts);
+    reduce_short<G, NV>(tv, wk, grad, n_bags, call.n_multi, vblock - grid.parts, grid.shorts);
   } else {
-    update_singletons<G, NV>(tv, wk, grad, n_bags, vblock - grid.parts - grid.shorts, grid.singles);
+    update_singletons<G, NV>(tv, wk, grad, n_bags, call.n_unique, vblock - grid.parts - grid.shorts, grid.singles);
     clear_primary(wk, vblock - grid.parts - grid.shorts, grid.singles);
   }
-  block_done(tv.st, wk, total_blocks);
+  check_out(tv.st, wk, &call, total_blocks);
 }
 template <int G, int NV>
 __global__ void __launch_bounds__(kRowThreads, NV == 1 ? 10 : NV == 2 ? 7 : 4)

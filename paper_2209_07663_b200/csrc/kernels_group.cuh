@@ -83,8 +83,7 @@ group_sketch_add_kernel(const GroupItem* __restrict__ items, const uint32_t* __r
 __global__ void __launch_bounds__(256)
 group_table_insert_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
-  table_insert_body(it.tv, it.wk, it.now, vblock, vgrid);
-  block_done(it.tv.st, it.wk, it.total_blocks);
+  table_insert_body(it.tv, it.wk, it.now, it.total_blocks, vblock, vgrid);
 }
 
 // (of a push whose batch was not pulled since it was announced, or not announced)

@@ -233,7 +233,7 @@ int discard_prepared(mono_table* t) {
   t->prep.valid = false;
   if (t->prep.ordered) CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_aux, 0));
   init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(t->wk.bset, t->wk.n_slots());
-  forget_call_kernel<<<1, 256, 0, t->stream>>>(t->tv.st, t->wk);
+  forget_call_kernel<<<1, 32, 0, t->stream>>>(t->tv.st, t->wk);
   CUDA_TRY(t, cudaGetLastError());
   return MONO_OK;
 }

@@ -111,7 +111,7 @@ struct CallState {
   unsigned int n_multi;                  // distinct IDs that occur more than once in the batch
   unsigned int seg_cursor;               // entries of bag_of_sorted[] handed out so far
   unsigned int bad_offsets;              // this call's offsets were malformed: occurrences are checked one by one
-  unsigned int blocks_done;              // of the kernels that end a push: the last one closes the call
+  unsigned int blocks_in;                // of the kernels that end a push: the last one closes the call
   unsigned int pad;
 };
 
