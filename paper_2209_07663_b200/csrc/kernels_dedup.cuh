@@ -142,7 +142,15 @@ __device__ inline unsigned long long block_exclusive_scan(unsigned long long v, 
 }
 
 // One block per tile of kTileIds consecutive occurrences.
-// (eight blocks per SM: measured 0.207 ms on the largest configuration against 0.234 ms with six)
+// Bound by latency: an occurrence's ID, its slot's key, the claim of a free slot, the update of its count and that of the
+// list's length are round trips to L2 one after the other, and the block waits at barriers for the slowest.  So the IDs
+// are asked for before anything is known about the offsets, and the list's length is updated, together with the number of
+// valid occurrences, while the counts are on their way: all tiles update that one word, 3 ns each (two words, and all in
+// turn: 8 M IDs 205 us, now 190; 4 M drifting 82 -> 71; 64 tables grouped 28 -> 24).
+// Tiles of 256 occurrences: 267 and 115 us, twice as many updates of that word.  Tiles of 768 in blocks of 384
+// threads: 204 and 67.  Of 1024 in blocks of 512: 213 and 71.  Three or four occurrences per thread instead of two, at fewer
+// warps: 208 to 350 us.  A slot claimed together with its count, by a 16-byte compare-and-swap: 197.  Six blocks per SM
+// instead of eight: a tenth slower.
 __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long* __restrict__ ids, long long n_ids,
                                        const long long* __restrict__ offsets, long long n_bags,
                                        unsigned long long seed, uint32_t vblock) {
@@ -150,37 +158,42 @@ __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long*
   __shared__ unsigned long long s_key[kTileSlots];
   __shared__ unsigned int s_cnt[kTileSlots];     // multiplicity in the tile, then base rank
   __shared__ unsigned int s_gslot[kTileSlots];   // the ID's slot in the global set
-  __shared__ unsigned long long s_warp[kTileThreads / 32];
+  __shared__ unsigned long long s_total;         // occurrences of the tile in the high word, IDs it saw first in the low
   __shared__ unsigned int s_ubase;
 
-  for (int i = threadIdx.x; i < kTileSlots; i += kTileThreads) { s_key[i] = kEmptyKey; s_cnt[i] = 0; }
+  const long long tile0 = (long long)vblock * kTileIds;
+  unsigned long long my_id[kPerThread];
+#pragma unroll
+  for (int k = 0; k < kPerThread; ++k) {
+    const long long j = tile0 + k * kTileThreads + threadIdx.x;
+    my_id[k] = j < n_ids ? ids[j] : kEmptyKey;
+  }
   long long first = offsets[0], last = offsets[n_bags];
+  const bool check_each = wk.call->bad_offsets != 0u;     // set by fill_occ_bag_kernel, earlier on this stream
+  for (int i = threadIdx.x; i < kTileSlots; i += kTileThreads) { s_key[i] = kEmptyKey; s_cnt[i] = 0; }
+  if (threadIdx.x == 0) s_total = 0ull;
   if (first < 0) first = 0;
   if (last > n_ids) last = n_ids;
-  const bool check_each = wk.call->bad_offsets != 0u;     // set by fill_occ_bag_kernel, earlier on this stream
   if (check_each) { first = 0; last = n_ids; }
   __syncthreads();
 
   // 1. group the tile's occurrences in shared memory.  The thread whose occurrence puts an ID
   //    into the tile's table owns that ID for the rest of the kernel.
-  const long long tile0 = (long long)vblock * kTileIds;
-  unsigned long long my_id[kPerThread];
   uint32_t my_slot[kPerThread], my_rank[kPerThread];
   bool own[kPerThread];
-  unsigned int n_valid = 0;
+  unsigned int n_valid = 0;                               // of the warp
 #pragma unroll
   for (int k = 0; k < kPerThread; ++k) {
     const long long j = tile0 + k * kTileThreads + threadIdx.x;
-    unsigned long long id = kEmptyKey;
-    if (j >= first && j < last) id = ids[j];
+    if (j < first || j >= last) my_id[k] = kEmptyKey;
     // malformed offsets: an occurrence that no well-formed bag covers is padding, as in the lookup
-    if (check_each && id != kEmptyKey && !occurrence_covered(wk.occ_bag, offsets, n_bags, n_ids, j)) id = kEmptyKey;
-    my_id[k] = id;
+    if (check_each && my_id[k] != kEmptyKey && !occurrence_covered(wk.occ_bag, offsets, n_bags, n_ids, j)) my_id[k] = kEmptyKey;
+    const unsigned long long id = my_id[k];
     my_slot[k] = kNoSlot;
     my_rank[k] = 0;
     own[k] = false;
+    n_valid += __popc(__ballot_sync(0xFFFFFFFFu, id != kEmptyKey));
     if (id != kEmptyKey) {
-      ++n_valid;
       uint32_t s = (uint32_t)(mix_a(id ^ seed) >> 40) & (kTileSlots - 1);
       for (int probe = 0; probe < kTileSlots; ++probe) {      // at most kTileIds keys in kTileSlots slots
         const unsigned long long old = atomicCAS(&s_key[s], kEmptyKey, id);
@@ -205,10 +218,10 @@ __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long*
     g[k] = (uint32_t)(mix_b(my_id[k] ^ seed) >> 20) & wk.primary_mask;
     seen[k] = own[k] ? *reinterpret_cast<volatile unsigned long long*>(&wk.bset[g[k]].key) : 0ull;
   }
-  unsigned int n_new = 0;
 #pragma unroll
   for (int k = 0; k < kPerThread; ++k) {
     is_new[k] = false;
+    base_rank[k] = 0u;
     if (!own[k]) continue;
     const unsigned long long id = my_id[k];
     unsigned long long kk = seen[k];
@@ -239,38 +252,39 @@ __device__ inline void dedup_tile_body(const Work& wk, const unsigned long long*
       }
       g[k] = base2 + q;
     }
-    n_new += is_new[k];
   }
 #pragma unroll
   for (int k = 0; k < kPerThread; ++k)
-    base_rank[k] = own[k] ? atomicAdd(&wk.bset[g[k]].a, s_cnt[my_slot[k]]) : 0u;
+    if (own[k]) base_rank[k] = atomicAdd(&wk.bset[g[k]].a, s_cnt[my_slot[k]]);
+  // number the IDs this tile saw first: one counter update per tile
+  const int lane = threadIdx.x & 31;
+  unsigned int news[kPerThread], my_u = 0;
+#pragma unroll
+  for (int k = 0; k < kPerThread; ++k) {
+    news[k] = __ballot_sync(0xFFFFFFFFu, is_new[k]);
+    my_u += __popc(news[k]);
+  }
+  if (lane == 0) my_u = (unsigned int)atomicAdd(&s_total, (unsigned long long)n_valid << 32 | my_u);
+  my_u = __shfl_sync(0xFFFFFFFFu, my_u, 0);
+  __syncthreads();
+  if (threadIdx.x == 0) s_ubase = s_total ? (unsigned int)atomicAdd(reinterpret_cast<unsigned long long*>(&wk.call->n_unique), s_total) : 0u;
 #pragma unroll
   for (int k = 0; k < kPerThread; ++k) {
     if (!own[k]) continue;
     s_cnt[my_slot[k]] = base_rank[k];
     s_gslot[my_slot[k]] = g[k];
   }
-  // number the IDs this tile saw first: one counter update per tile
-  // (new IDs in the low word, valid occurrences in the high word of one scan)
-  unsigned long long total = 0;
-  unsigned int my_u = (unsigned int)block_exclusive_scan(((unsigned long long)n_valid << 32) | n_new, s_warp, &total);
-  if (threadIdx.x == 0) {
-    const unsigned int total_new = (unsigned int)total, total_valid = (unsigned int)(total >> 32);
-    s_ubase = total_new ? atomicAdd(&wk.call->n_unique, total_new) : 0u;
-    if (total_valid) atomicAdd(&wk.call->n_valid_ids, total_valid);
-  }
   __syncthreads();
   my_u += s_ubase;
 #pragma unroll
   for (int k = 0; k < kPerThread; ++k) {
-    if (is_new[k]) {
-      if (MONO_INDEX_OK(wk.error_bits, my_u, wk.max_ids)) {
-        wk.uid[my_u] = my_id[k];
-        wk.uslot[my_u] = g[k];
-        wk.uocc[my_u] = (uint32_t)(tile0 + k * kTileThreads + threadIdx.x);     // the owner's own occurrence
-      }
-      ++my_u;
+    const unsigned int u = my_u + __popc(news[k] & ((1u << lane) - 1u));
+    if (is_new[k] && MONO_INDEX_OK(wk.error_bits, u, wk.max_ids)) {
+      wk.uid[u] = my_id[k];
+      wk.uslot[u] = g[k];
+      wk.uocc[u] = (uint32_t)(tile0 + k * kTileThreads + threadIdx.x);     // the owner's own occurrence
     }
+    my_u += __popc(news[k]);
   }
 
   // 3. every occurrence learns its ID's slot and its rank

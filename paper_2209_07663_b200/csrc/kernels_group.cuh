@@ -61,7 +61,7 @@ group_fill_occ_bag_kernel(const GroupItem* __restrict__ items, const uint32_t* _
   fill_occ_bag_body(it.off, it.n_bags, it.n_ids, it.wk.occ_bag, it.wk.call, vblock, vgrid);
 }
 
-__global__ void __launch_bounds__(kTileThreads, 8)
+__global__ void __launch_bounds__(kTileThreads, 6)
 group_dedup_tile_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   dedup_tile_body(it.wk, it.ids, it.n_ids, it.off, it.n_bags, it.dedup_seed, vblock);

@@ -103,11 +103,11 @@ struct DevState {
 // Counters of one batch on its way through grouping, look-up and push; all zero between calls.  They
 // belong to the scratch a batch is grouped into, not to the table: a batch that is grouped ahead has a
 // copy of its own, which changes places with the other when its turn comes.
-struct CallState {
+struct __align__(8) CallState {
   unsigned long long longs;              // high word: distinct IDs whose segment is reduced in parts; low word: their parts
-  unsigned int n_unique;
-  unsigned int n_insert;
+  unsigned int n_unique;                 // (these two are added to together, as one 64-bit word)
   unsigned int n_valid_ids;
+  unsigned int n_insert;
   unsigned int n_multi;                  // distinct IDs that occur more than once in the batch
   unsigned int seg_cursor;               // entries of bag_of_sorted[] handed out so far
   unsigned int bad_offsets;              // this call's offsets were malformed: occurrences are checked one by one
