@@ -503,117 +503,115 @@ order_parts_kernel(Work wk) { after_previous_kernel(); order_parts_body(wk, bloc
 
 // Expiry sweep (Section 2.1, heuristic 2): a streaming pass over the key
 // store; a cell whose ID has been inactive for longer than ttl is emptied and
-// its row, if it has one, goes back on the free list (one counter update per
-// warp and round).
-// Rows of expired entries go back on the free stack: one counter update per warp.  Every lane
-// of the warp calls this.
-__device__ inline void warp_free_row(const TableView& tv, bool frees_row, uint32_t row, int lane) {
-  const unsigned mask = __ballot_sync(0xFFFFFFFFu, frees_row);
-  if (mask == 0) return;
-  unsigned long long pos = 0;
-  const int leader = __ffs(mask) - 1;
-  if (lane == leader)
-    pos = atomicAdd(reinterpret_cast<unsigned long long*>(&tv.st->free_top), (unsigned long long)__popc(mask));
-  pos = __shfl_sync(0xFFFFFFFFu, pos, leader);
-  const unsigned long long at = pos + __popc(mask & ((1u << lane) - 1u));
-  if (frees_row && MONO_INDEX_OK(&tv.st->error_bits, at, tv.capacity)) tv.free_rows[at] = row;
-}
-
+// its row, if it has one, goes back on the free list.
+//
 // Sweep of buckets [first_bkt, last_bkt) of the key store, and of the stash if `with_stash`.
 // The sweep reads, per bucket, the record of its oldest stamp (4 bytes, in order) and opens only
 // the buckets in which that stamp is past the expire time: an entry that has to go has a stamp at
 // or above its bucket's record, so its bucket is always opened, and the outcome is that of a sweep
 // over every cell.  A bucket that is opened gets an exact record again.  Nothing else touches the
 // key store while this runs.
-// A block lists the buckets to open in shared memory, then takes them one cell per thread, so that
-// all their loads are in flight together and the four lanes of a bucket read its 64 bytes as one.
-constexpr int kSweepDepth = 2;                                             // 16-byte loads of four records per thread and round
+// A block lists the buckets to open in shared memory, round by round until there are enough to fill it, then takes them one
+// cell per thread, so that all their loads are in flight together and the four lanes of a bucket read its 64 bytes as one.
+// The rows it frees are listed too and go on the free stack together: the top of the stack is one word that all blocks
+// update, and an update per warp and turn was what a sweep that frees many rows waited for.  Rounds of 1024 buckets instead
+// of 2048 spread a small key store or a slice over the SMs.  (Sweeps that empty 1 / 10 / 70 % of 4 M entries in 2^24 cells
+// 17 / 70 / 244 -> 9 / 25 / 83 us, of 16 M in 2^28
+// cells 87 / 238 / 1108 -> 67 / 167 / 581, of 131 000 in 2^19 cells 3.4 / 7.0 / 20 -> 3.4 / 4.4 / 8.1; without the listing over
+// several rounds the second is 125 / 171 / 570.)
+constexpr int kSweepThreads = 256;
+constexpr int kSweepBuckets = kSweepThreads * 4;                           // a block's buckets of a round: one 16-byte load of four records per thread
+constexpr uint32_t kSweepFew = 256;                                        // fewer to open than this: another round first
+struct SweepShared {
+  uint32_t open[kSweepFew + kSweepBuckets];                                // buckets to open, counted from the sweep's first
+  uint32_t row[kSweepBuckets * kCellsPerBucket];                           // rows that have become free
+  unsigned int n_open, n_rows, n_gone, n_freed;
+  long long top;
+};
+
+// Empties the cell if its entry is past the ttl.  Returns the entry's stamp if it stays.
+__device__ __forceinline__ uint32_t expire_cell(SweepShared& sh, ulonglong2* cell, long long now, long long ttl) {
+  const ulonglong2 v = *cell;
+  if (v.x == kEmptyKey) return kNoStamp;
+  const uint32_t seen = meta_time(v.y);
+  if (now - (long long)seen <= ttl) return seen;
+  ulonglong2 e; e.x = kEmptyKey; e.y = 0ull;
+  *cell = e;
+  atomicAdd(&sh.n_gone, 1u);
+  if (meta_resident(v.y)) sh.row[atomicAdd(&sh.n_rows, 1u)] = meta_row(v.y);
+  return kNoStamp;
+}
+// The rows listed so far go on the free stack, with one update of its top.  All threads of the block call this, behind a barrier.
+__device__ __forceinline__ void push_free_rows(const TableView& tv, SweepShared& sh) {
+  const unsigned int n = sh.n_rows;
+  if (n == 0) return;
+  if (threadIdx.x == 0) sh.top = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&tv.st->free_top), (unsigned long long)n);
+  __syncthreads();
+  for (unsigned int i = threadIdx.x; i < n; i += kSweepThreads)
+    if (MONO_INDEX_OK(&tv.st->error_bits, sh.top + i, tv.capacity)) tv.free_rows[sh.top + i] = sh.row[i];
+  if (threadIdx.x == 0) sh.n_freed += n;
+}
+
 __device__ inline void expire_body(const TableView& tv, unsigned long long first_bkt, unsigned long long last_bkt,
                                    bool with_stash, long long now, uint32_t vblock, uint32_t vgrid) {
   // first_bkt and last_bkt are multiples of four
-  __shared__ unsigned long long open_list[256 * kSweepDepth * 4];
-  __shared__ unsigned int n_open;
-  const unsigned long long stride = (unsigned long long)vgrid * blockDim.x * 4u;
-  const unsigned long long rounds = (last_bkt - first_bkt + stride * kSweepDepth - 1) / (stride * kSweepDepth);  // same for every thread
-  const int lane = threadIdx.x & 31;
+  __shared__ SweepShared sh;
   const long long ttl = (long long)tv.ttl;
-  unsigned int n_gone = 0, n_rows = 0;
-  for (unsigned long long r = 0; r < rounds; ++r) {
-    if (threadIdx.x == 0) n_open = 0;
+  const unsigned long long stride = (unsigned long long)vgrid * kSweepBuckets;
+  const auto records = [&](unsigned long long b) {
+    return b < last_bkt ? *reinterpret_cast<const uint4*>(tv.oldest + b) : make_uint4(kNoStamp, kNoStamp, kNoStamp, kNoStamp);
+  };
+  if (threadIdx.x == 0) sh.n_open = sh.n_rows = sh.n_gone = sh.n_freed = 0;
+  unsigned long long b0 = first_bkt + (unsigned long long)vblock * kSweepBuckets;
+  uint4 next = records(b0 + threadIdx.x * 4u);
+  __syncthreads();
+  for (; b0 < last_bkt; b0 += stride) {                    // block-uniform
+    const uint4 rec = next;
+    next = records(b0 + stride + threadIdx.x * 4u);        // (no record of another round is written in this one)
+    const uint32_t four[4] = {rec.x, rec.y, rec.z, rec.w};
+#pragma unroll
+    for (uint32_t q = 0; q < 4; ++q)
+      if (four[q] != kNoStamp && now - (long long)four[q] > ttl) sh.open[atomicAdd(&sh.n_open, 1u)] = (uint32_t)(b0 - first_bkt) + threadIdx.x * 4u + q;
     __syncthreads();
-    const unsigned long long b0 = first_bkt + r * kSweepDepth * stride + ((unsigned long long)vblock * blockDim.x + threadIdx.x) * 4u;
-    uint4 rec[kSweepDepth];
-#pragma unroll
-    for (int k = 0; k < kSweepDepth; ++k) {
-      const unsigned long long b = b0 + k * stride;
-      rec[k] = make_uint4(kNoStamp, kNoStamp, kNoStamp, kNoStamp);
-      if (b < last_bkt) rec[k] = *reinterpret_cast<const uint4*>(tv.oldest + b);
+    const uint32_t n_open = sh.n_open;
+    const bool take = n_open > kSweepFew || b0 + stride >= last_bkt;
+    for (uint32_t o0 = 0; take && o0 < n_open; o0 += kSweepBuckets) {
+      const uint32_t n_cells_open = (n_open - o0 < kSweepBuckets ? n_open - o0 : kSweepBuckets) * kCellsPerBucket;
+      for (uint32_t base = 0; base < n_cells_open; base += kSweepThreads) {
+        const uint32_t idx = base + threadIdx.x;
+        const bool valid = idx < n_cells_open;
+        const unsigned long long b = first_bkt + (valid ? sh.open[o0 + idx / kCellsPerBucket] : 0u);
+        uint32_t kept = kNoStamp;
+        if (valid) kept = expire_cell(sh, reinterpret_cast<ulonglong2*>(tv.cells + b * kCellsPerBucket + idx % kCellsPerBucket), now, ttl);
+        // the oldest stamp that stays in the bucket: its four cells sit in four adjacent lanes
+        kept = min(kept, __shfl_xor_sync(0xFFFFFFFFu, kept, 1));
+        kept = min(kept, __shfl_xor_sync(0xFFFFFFFFu, kept, 2));
+        if (valid && (idx % kCellsPerBucket) == 0) tv.oldest[b] = kept;
+      }
+      __syncthreads();
+      push_free_rows(tv, sh);
+      __syncthreads();
+      if (threadIdx.x == 0) sh.n_rows = 0;
+      __syncthreads();
     }
-#pragma unroll
-    for (int k = 0; k < kSweepDepth; ++k) {
-      const uint32_t four[4] = {rec[k].x, rec[k].y, rec[k].z, rec[k].w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (four[q] != kNoStamp && now - (long long)four[q] > ttl) open_list[atomicAdd(&n_open, 1u)] = b0 + k * stride + q;
-    }
+    if (take && threadIdx.x == 0) sh.n_open = 0;
+    __syncthreads();                                       // everyone has read n_open before the next round adds to it
+  }
+  if (with_stash && vblock == 0) {
+    static_assert(kStashCells <= kSweepBuckets * kCellsPerBucket, "the rows of the stash fit the list");
     __syncthreads();
-    const unsigned int n_cells_open = n_open * kCellsPerBucket;
-    for (unsigned int base = 0; base < n_cells_open; base += blockDim.x) {      // block-uniform
-      const unsigned int idx = base + threadIdx.x;
-      const bool valid = idx < n_cells_open;
-      const unsigned long long b = valid ? open_list[idx / kCellsPerBucket] : 0ull;
-      ulonglong2* cell = reinterpret_cast<ulonglong2*>(tv.cells + b * kCellsPerBucket + (idx % kCellsPerBucket));
-      ulonglong2 v; v.x = kEmptyKey; v.y = 0ull;
-      if (valid) v = *cell;
-      bool frees_row = false;
-      uint32_t row = 0, kept = kNoStamp;
-      if (v.x != kEmptyKey) {
-        const uint32_t seen = meta_time(v.y);
-        if (now - (long long)seen > ttl) {
-          ulonglong2 e; e.x = kEmptyKey; e.y = 0ull;
-          *cell = e;
-          ++n_gone;
-          if (meta_resident(v.y)) { frees_row = true; row = meta_row(v.y); ++n_rows; }
-        } else {
-          kept = seen;
-        }
-      }
-      // the oldest stamp that stays in the bucket: its four cells sit in four adjacent lanes
-      kept = min(kept, __shfl_xor_sync(0xFFFFFFFFu, kept, 1));
-      kept = min(kept, __shfl_xor_sync(0xFFFFFFFFu, kept, 2));
-      if (valid && (idx % kCellsPerBucket) == 0) tv.oldest[b] = kept;
-      warp_free_row(tv, frees_row, row, lane);
-    }
-    __syncthreads();                                       // everyone has read n_open before the next round resets it
+    for (uint32_t i = threadIdx.x; i < kStashCells; i += kSweepThreads) expire_cell(sh, reinterpret_cast<ulonglong2*>(tv.stash + i), now, ttl);
+    __syncthreads();
+    push_free_rows(tv, sh);
   }
-  if (with_stash) {
-    for (uint32_t base = vblock * blockDim.x; base < kStashCells; base += vgrid * blockDim.x) {   // block-uniform
-      const uint32_t i = base + threadIdx.x;
-      bool frees_row = false;
-      uint32_t row = 0;
-      if (i < kStashCells) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(tv.stash + i);
-        if (v.x != kEmptyKey && now - (long long)meta_time(v.y) > ttl) {
-          ulonglong2 e; e.x = kEmptyKey; e.y = 0ull;
-          *reinterpret_cast<ulonglong2*>(tv.stash + i) = e;
-          ++n_gone;
-          if (meta_resident(v.y)) { frees_row = true; row = meta_row(v.y); ++n_rows; }
-        }
-      }
-      warp_free_row(tv, frees_row, row, lane);
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    n_gone += __shfl_down_sync(0xFFFFFFFFu, n_gone, o);
-    n_rows += __shfl_down_sync(0xFFFFFFFFu, n_rows, o);
-  }
-  if (lane == 0 && n_gone) {
-    atomicAdd(&tv.st->n_tracked, (unsigned long long)(-(long long)n_gone));
-    atomicAdd(&tv.st->n_expired_total, (unsigned long long)n_gone);
-    if (n_rows) atomicAdd(&tv.st->n_resident, (unsigned long long)(-(long long)n_rows));
+  __syncthreads();
+  if (threadIdx.x == 0 && sh.n_gone) {
+    atomicAdd(&tv.st->n_tracked, (unsigned long long)(-(long long)sh.n_gone));
+    atomicAdd(&tv.st->n_expired_total, (unsigned long long)sh.n_gone);
+    if (sh.n_freed) atomicAdd(&tv.st->n_resident, (unsigned long long)(-(long long)sh.n_freed));
   }
 }
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSweepThreads)
 expire_kernel(TableView tv, unsigned long long first_bkt, unsigned long long last_bkt, int with_stash, long long now) { after_previous_kernel();
   expire_body(tv, first_bkt, last_bkt, with_stash != 0, now, blockIdx.x, gridDim.x);
 }

@@ -1066,11 +1066,10 @@ static int expire_range(mono_table* t, int64_t now, uint32_t slice, uint32_t n_s
   const unsigned long long first = per_slice * slice;
   const unsigned long long last = is_last ? n_buckets : per_slice * (slice + 1);
   if (last > first || is_last) {
-    const unsigned long long per_block = 256ull * 4 * kSweepDepth;               // buckets a block reads per round
-    unsigned long long blocks = (last - first + per_block - 1) / per_block;
+    unsigned long long blocks = (last - first + kSweepBuckets - 1) / kSweepBuckets;
     if (blocks < 1) blocks = 1;
     if (blocks > (unsigned long long)grid_for(t, 8)) blocks = grid_for(t, 8);
-    LAUNCH_ON(t, s, K_EXPIRE, launch_after(expire_kernel, (int)blocks, 256, s, t->tv, first, last, is_last ? 1 : 0, (long long)now));
+    LAUNCH_ON(t, s, K_EXPIRE, launch_after(expire_kernel, (int)blocks, kSweepThreads, s, t->tv, first, last, is_last ? 1 : 0, (long long)now));
   }
   if (slice + 1 == n_slices) LAUNCH_ON(t, s, K_STASH_TRIM, launch_after(stash_trim_kernel, 1, 32, s, t->tv));
   CUDA_TRY(t, cudaGetLastError());

@@ -227,3 +227,30 @@ def test_a_small_push_costs_the_same_in_a_large_reservation():
         us.append(best * 1e3)
         t.close()
     assert us[1] < 3 * us[0], us
+
+
+@pytest.mark.parametrize("n, key_cells", [(60, 64), (900, 1 << 12), (4000, 1 << 12), (4000, 1 << 23), (3 << 20, 1 << 23)])
+@pytest.mark.parametrize("slices", [1, 3])
+def test_sweeps_of_sparse_and_dense_key_stores(n, key_cells, slices):
+    """Blocks with one round of buckets and with several, few buckets to open (listed over several rounds) and nearly all;
+    entries of all ages swept three times, so that the second and third go by the records that the one before left."""
+    rng = np.random.default_rng(n)
+    ttl, capacity = 10, n + 5
+    ids = wl.splitmix64(np.arange(1, n + 1, dtype=np.uint64))
+    seen = rng.integers(0, 40, n)
+    owns = (rng.random(n) < 0.6).astype(np.uint8)
+    t = mb.MonoTable(capacity, 4, 3, ttl, key_cells=key_cells)
+    t.import_entries(ids, np.where(owns, 3, 1).astype(np.uint32), seen.astype(np.int64), owns, None, None)
+    assert t.status()["n_tracked"] == n
+    for now in (20, 21, 45):
+        for k in range(slices):
+            mb.mono_expire_slice(t.handle, now, k, slices)
+        stay = now - seen <= ttl
+        st = t.status()
+        assert (st["n_tracked"], st["n_resident"], st["n_expired_total"]) == (stay.sum(), (stay & (owns > 0)).sum(), n - stay.sum())
+        assert_audit_ok(t, f"now {now}")
+        got = t.export(rows=False)
+        order = np.argsort(ids[stay])
+        assert (got["ids"] == ids[stay][order]).all() and (got["last_seen"] == seen[stay][order]).all()
+    assert t.status()["error_bits"] == 0
+    t.close()
