@@ -35,6 +35,7 @@ struct __align__(16) BatchSlot {
 
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 constexpr uint32_t kNoSegment = 0xFFFFFFFFu;
+constexpr unsigned long long kNoMeta = 0xFFFFFFFFFFFFFFFFull;   // (no time is 2^32 - 1)
 constexpr uint32_t kSegChunk = 64;             // longest segment one lane group reduces alone
 constexpr uint32_t kFanIn = 16;                // partial sums that are added up at a time
 constexpr int kTileIds = 512;                  // occurrences per block of dedup_tile_kernel
@@ -66,8 +67,8 @@ struct Work {
   uint32_t* ulen;            // [max_ids] multiplicity of the ID in this batch
   uint32_t* urow;            // [max_ids] row word per distinct ID (kNoRow / row | kFreshBit)
   unsigned long long* ucell; // [max_ids] where the key store holds the ID (kNoCell: nowhere) and
-  unsigned long long* umeta; // [max_ids] the metadata found there, from the look-up that mono_prepare_push does
-                             //           ahead of the push
+  unsigned long long* umeta; // [max_ids] the metadata found there (kNoMeta: nowhere), from the look-up that mono_prepare_push
+                             //           does ahead of the push
   uint32_t* ins_list;        // [max_ids] distinct IDs that are not in the key store yet
   uint32_t* multi_list;      // [max_ids / 2 + 1] numbers of the distinct IDs that occur more than once
   uint32_t* long_u;          // [max_long] distinct IDs whose segment is reduced in parts

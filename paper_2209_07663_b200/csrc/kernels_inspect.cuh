@@ -39,7 +39,7 @@ probe_kernel(TableView tv, const unsigned long long* __restrict__ ids, long long
       }
       count[i] = c;
     }
-    if (last_seen) last_seen[i] = p ? (long long)meta_time(meta) : -1LL;
+    if (last_seen) last_seen[i] = p ? (long long)tv.last_seen(meta) : -1LL;
   }
 }
 
@@ -77,7 +77,7 @@ export_kernel(TableView tv, unsigned long long n_cells, unsigned long long* ids,
     const bool res = meta_resident(c.meta);
     ids[k] = c.key;
     if (count) count[k] = res ? tv.threshold : meta_low(c.meta);
-    if (last_seen) last_seen[k] = (long long)meta_time(c.meta);
+    if (last_seen) last_seen[k] = (long long)tv.last_seen(c.meta);
     if (resident) resident[k] = res ? 1 : 0;
     for (uint32_t col = 0; col < tv.dim; ++col) {
       if (w) w[k * (long long)tv.dim + col] = res ? tv.w_row(meta_row(c.meta))[col] : 0.f;

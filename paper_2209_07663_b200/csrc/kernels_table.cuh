@@ -136,7 +136,9 @@ __device__ inline void register_long(const Work& wk, uint32_t u, uint32_t m) {
 //           threshold), last_seen = now, and a row if the count has reached the threshold; an ID
 //           the key store does not hold is queued for insertion.  With kLookUp in an earlier
 //           kernel, the cell and its metadata are the remembered ones: the kernel reads its
-//           inputs in order and only scatters the new metadata words.
+//           inputs in order, and of an ID that owned a row before the metadata alone, and only scatters the rows' stamps.
+//           The cell of such an ID is written when that says something new: the mark that the row was trained
+//           since the last export, or a time before the cell's.
 //
 // Both halves in one kernel is the push that was not announced.  No cell moves during either
 // half, so the thread whose ID sits in a cell owns it.
@@ -158,22 +160,30 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
   for (uint32_t base = vblock * blockDim.x; base < n; base += vgrid * blockDim.x) {   // block-uniform
     const uint32_t u = base + threadIdx.x;
     const bool active = u < n;
-    unsigned long long id = kEmptyKey, meta = 0, cell = kNoCell;
+    unsigned long long id = kEmptyKey, meta = kNoMeta, cell = kNoCell;
     uint32_t m = 0, slot = 0;
+    bool settled = false;                  // it owned a row, and its cell stays as it is
+    const auto stays = [&] { return meta_touched(meta) && meta_time(meta) <= now; };
     if (active) {
-      id = wk.uid[u];
       if (MODE & kLookUp) {
+        id = wk.uid[u];
         slot = wk.uslot[u];
         if (!MONO_INDEX_OK(wk.error_bits, slot, wk.n_slots())) slot = 0;
         m = wk.bset[slot].a;
         cell = thread_locate(tv, id, stash_hw, &meta);
+        settled = cell != kNoCell && stays();
       } else {
         // nothing has changed the table since the look-up (every call that could forgets the
         // announcement), so the cell and its metadata are as remembered
-        m = wk.ulen[u];
-        cell = wk.ucell[u];
         meta = wk.umeta[u];
+        settled = meta != kNoMeta && stays();
+        if (!settled) {
+          m = wk.ulen[u];
+          cell = wk.ucell[u];
+        }
 #ifdef MONO_DEBUG
+        id = wk.uid[u];
+        cell = wk.ucell[u];
         if (cell != kNoCell) {
           const Cell c = load_cell_whole(cell_address(tv, cell, n_cells));
           if (c.key != id || c.meta != meta) { atomicOr(&tv.st->error_bits, 16u /* MONO_DEV_INTERNAL */); cell = thread_locate(tv, id, stash_hw, &meta); }
@@ -181,7 +191,7 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
 #endif
       }
     }
-    const bool hit = cell != kNoCell;
+    const bool hit = meta != kNoMeta;
     uint32_t low = meta_low(meta);
     const bool resident = hit && (low & kResidentBit) != 0;
     bool need_row = false;
@@ -216,14 +226,17 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
         // every ID of the batch that has a row is trained in this call: mark it for the next sync
         if (resident) { row_word = low & kRowMask; low |= kTouchedBit; }
         else if (rv.row != kNoRow) { low = kResidentBit | kTouchedBit | rv.row; row_word = rv.row | kFreshBit; }
-        cell_address(tv, cell, n_cells)->meta = make_meta(now, low);
+        if (!settled) cell_address(tv, cell, n_cells)->meta = make_meta(now, low);
         wk.urow[u] = row_word;
-        if (row_word != kNoRow) ++n_res;
+        if (row_word != kNoRow) {
+          if (MONO_INDEX_OK(&tv.st->error_bits, row_word & ~kFreshBit, tv.capacity)) tv.seen[row_word & ~kFreshBit] = now;
+          ++n_res;
+        }
       } else {
         if (exact) {
           const uint32_t row_word = rv.row != kNoRow ? (rv.row | kFreshBit) : kNoRow;
           wk.urow[u] = row_word;
-          if (row_word != kNoRow) ++n_res;
+          if (row_word != kNoRow) { tv.seen[rv.row] = now; ++n_res; }
         }
         if (MONO_INDEX_OK(wk.error_bits, rv.ins_pos, wk.max_ids)) wk.ins_list[rv.ins_pos] = u;
       }
@@ -418,7 +431,7 @@ __device__ inline void table_insert_body(const TableView& tv, const Work& wk, ui
       if (!todo) continue;
       if (rv.row != kNoRow) row_word = rv.row | kFreshBit;
       wk.urow[u] = row_word;
-      if (row_word != kNoRow) ++n_res;
+      if (row_word != kNoRow) { tv.seen[rv.row] = now; ++n_res; }
       if (row_word == kNoRow) continue;                // below the estimate (or no row left): not stored
     } else {
       if (!todo) continue;
@@ -518,9 +531,10 @@ order_parts_kernel(Work wk) { after_previous_kernel(); order_parts_body(wk, bloc
 // of 2048 spread a small key store or a slice over the SMs.  (Sweeps that empty 1 / 10 / 70 % of 4 M entries in 2^24 cells
 // 17 / 70 / 244 -> 9 / 25 / 83 us, of 16 M in 2^28
 // cells 87 / 238 / 1108 -> 67 / 167 / 581, of 131 000 in 2^19 cells 3.4 / 7.0 / 20 -> 3.4 / 4.4 / 8.1; without the listing over
-// several rounds the second is 125 / 171 / 570.)
+// several rounds the second is 125 / 171 / 570.  With the rows' stamps read: 10 / 28 / 96, 65 / 191 / 748, 4.2 / 4.5 / 8.4.)
 constexpr int kSweepThreads = 256;
 constexpr int kSweepBuckets = kSweepThreads * 4;                           // a block's buckets of a round: one 16-byte load of four records per thread
+constexpr int kSweepCells = 2;                                             // cells of a thread in flight (with their rows' stamps: one 17.2 us, two 16.4 in a drifting step)
 constexpr uint32_t kSweepFew = 256;                                        // fewer to open than this: another round first
 struct SweepShared {
   uint32_t open[kSweepFew + kSweepBuckets];                                // buckets to open, counted from the sweep's first
@@ -529,17 +543,41 @@ struct SweepShared {
   long long top;
 };
 
-// Empties the cell if its entry is past the ttl.  Returns the entry's stamp if it stays.
-__device__ __forceinline__ uint32_t expire_cell(SweepShared& sh, ulonglong2* cell, long long now, long long ttl) {
-  const ulonglong2 v = *cell;
-  if (v.x == kEmptyKey) return kNoStamp;
-  const uint32_t seen = meta_time(v.y);
-  if (now - (long long)seen <= ttl) return seen;
-  ulonglong2 e; e.x = kEmptyKey; e.y = 0ull;
-  *cell = e;
-  atomicAdd(&sh.n_gone, 1u);
-  if (meta_resident(v.y)) sh.row[atomicAdd(&sh.n_rows, 1u)] = meta_row(v.y);
-  return kNoStamp;
+// Empties each of N cells (null: none) if its entry is past the ttl; kept: the entry's stamp if it stays.  The reads of all
+// come before their writes, so that they are in flight together.
+template <int N>
+__device__ __forceinline__ void expire_cells(const TableView& tv, SweepShared& sh, ulonglong2* const (&cell)[N], long long now, long long ttl,
+                                             uint32_t (&kept)[N]) {
+  ulonglong2 v[N];
+  uint32_t seen[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    v[k].x = kEmptyKey;
+    v[k].y = 0ull;
+    if (cell[k]) v[k] = *cell[k];
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    // a cell that is past the ttl and owns a row: its time is only a bound, the row has the exact one
+    seen[k] = meta_time(v[k].y);
+    if (v[k].x != kEmptyKey && meta_resident(v[k].y) && now - (long long)seen[k] > ttl && MONO_INDEX_OK(&tv.st->error_bits, meta_row(v[k].y), tv.capacity))
+      seen[k] = tv.seen[meta_row(v[k].y)];
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    kept[k] = kNoStamp;
+    if (v[k].x == kEmptyKey) continue;
+    if (now - (long long)seen[k] <= ttl) {
+      kept[k] = seen[k];
+      // (into the cell too, so that the bucket is not opened for it again before its time)
+      if (seen[k] != meta_time(v[k].y)) cell[k]->y = make_meta(seen[k], meta_low(v[k].y));
+      continue;
+    }
+    ulonglong2 e; e.x = kEmptyKey; e.y = 0ull;
+    *cell[k] = e;
+    atomicAdd(&sh.n_gone, 1u);
+    if (meta_resident(v[k].y)) sh.row[atomicAdd(&sh.n_rows, 1u)] = meta_row(v[k].y);
+  }
 }
 // The rows listed so far go on the free stack, with one update of its top.  All threads of the block call this, behind a barrier.
 __device__ __forceinline__ void push_free_rows(const TableView& tv, SweepShared& sh) {
@@ -577,16 +615,24 @@ __device__ inline void expire_body(const TableView& tv, unsigned long long first
     const bool take = n_open > kSweepFew || b0 + stride >= last_bkt;
     for (uint32_t o0 = 0; take && o0 < n_open; o0 += kSweepBuckets) {
       const uint32_t n_cells_open = (n_open - o0 < kSweepBuckets ? n_open - o0 : kSweepBuckets) * kCellsPerBucket;
-      for (uint32_t base = 0; base < n_cells_open; base += kSweepThreads) {
-        const uint32_t idx = base + threadIdx.x;
-        const bool valid = idx < n_cells_open;
-        const unsigned long long b = first_bkt + (valid ? sh.open[o0 + idx / kCellsPerBucket] : 0u);
-        uint32_t kept = kNoStamp;
-        if (valid) kept = expire_cell(sh, reinterpret_cast<ulonglong2*>(tv.cells + b * kCellsPerBucket + idx % kCellsPerBucket), now, ttl);
-        // the oldest stamp that stays in the bucket: its four cells sit in four adjacent lanes
-        kept = min(kept, __shfl_xor_sync(0xFFFFFFFFu, kept, 1));
-        kept = min(kept, __shfl_xor_sync(0xFFFFFFFFu, kept, 2));
-        if (valid && (idx % kCellsPerBucket) == 0) tv.oldest[b] = kept;
+      for (uint32_t base = 0; base < n_cells_open; base += kSweepThreads * kSweepCells) {
+        unsigned long long b[kSweepCells];
+        ulonglong2* cell[kSweepCells];
+        uint32_t kept[kSweepCells];
+#pragma unroll
+        for (int k = 0; k < kSweepCells; ++k) {
+          const uint32_t idx = base + k * kSweepThreads + threadIdx.x;
+          b[k] = first_bkt + (idx < n_cells_open ? sh.open[o0 + idx / kCellsPerBucket] : 0u);
+          cell[k] = idx < n_cells_open ? reinterpret_cast<ulonglong2*>(tv.cells + b[k] * kCellsPerBucket + idx % kCellsPerBucket) : nullptr;
+        }
+        expire_cells<kSweepCells>(tv, sh, cell, now, ttl, kept);
+        // the oldest stamp that stays in a bucket: its four cells sit in four adjacent lanes
+#pragma unroll
+        for (int k = 0; k < kSweepCells; ++k) {
+          kept[k] = min(kept[k], __shfl_xor_sync(0xFFFFFFFFu, kept[k], 1));
+          kept[k] = min(kept[k], __shfl_xor_sync(0xFFFFFFFFu, kept[k], 2));
+          if (cell[k] && threadIdx.x % kCellsPerBucket == 0) tv.oldest[b[k]] = kept[k];
+        }
       }
       __syncthreads();
       push_free_rows(tv, sh);
@@ -600,7 +646,11 @@ __device__ inline void expire_body(const TableView& tv, unsigned long long first
   if (with_stash && vblock == 0) {
     static_assert(kStashCells <= kSweepBuckets * kCellsPerBucket, "the rows of the stash fit the list");
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < kStashCells; i += kSweepThreads) expire_cell(sh, reinterpret_cast<ulonglong2*>(tv.stash + i), now, ttl);
+    for (uint32_t i = threadIdx.x; i < kStashCells; i += kSweepThreads) {
+      ulonglong2* const cell[1] = {reinterpret_cast<ulonglong2*>(tv.stash + i)};
+      uint32_t kept[1];
+      expire_cells<1>(tv, sh, cell, now, ttl, kept);
+    }
     __syncthreads();
     push_free_rows(tv, sh);
   }
@@ -611,7 +661,7 @@ __device__ inline void expire_body(const TableView& tv, unsigned long long first
     if (sh.n_freed) atomicAdd(&tv.st->n_resident, (unsigned long long)(-(long long)sh.n_freed));
   }
 }
-__global__ void __launch_bounds__(kSweepThreads)
+__global__ void __launch_bounds__(kSweepThreads, 8)
 expire_kernel(TableView tv, unsigned long long first_bkt, unsigned long long last_bkt, int with_stash, long long now) { after_previous_kernel();
   expire_body(tv, first_bkt, last_bkt, with_stash != 0, now, blockIdx.x, gridDim.x);
 }
@@ -700,7 +750,7 @@ import_insert_kernel(TableView tv, const unsigned long long* __restrict__ ids, c
     uint32_t low = count[i] < tv.threshold ? count[i] : tv.threshold;
     if (resident[i]) {
       const uint32_t row = alloc_row(tv);
-      if (row != kNoRow) { low = kResidentBit | row; row_word[i] = row; }
+      if (row != kNoRow) { low = kResidentBit | row; row_word[i] = row; tv.seen[row] = (uint32_t)seen; }
       else low = tv.threshold;
     }
     Cell item; item.key = id; item.meta = make_meta((uint32_t)seen, low);

@@ -92,7 +92,7 @@ struct mono_table {
   } grp;
   // device-resident snapshot (mono_snapshot_save)
   struct {
-    Cell* cells = nullptr; Cell* stash = nullptr; float* rows = nullptr; uint32_t* free_rows = nullptr;
+    Cell* cells = nullptr; Cell* stash = nullptr; float* rows = nullptr; uint32_t* free_rows = nullptr; uint32_t* seen = nullptr;
     uint32_t* oldest = nullptr; DevState* st = nullptr; unsigned int* sketch = nullptr;
     uint64_t key_cells = 0; int64_t last_now = -1, sketch_epoch = 0; bool valid = false;
   } snap;
@@ -172,7 +172,7 @@ void free_scratch(mono_table* t) {
 
 void free_snapshot(mono_table* t) {
   auto& sn = t->snap;
-  dev_free(sn.cells); dev_free(sn.stash); dev_free(sn.oldest); dev_free(sn.rows); dev_free(sn.free_rows); dev_free(sn.st); dev_free(sn.sketch);
+  dev_free(sn.cells); dev_free(sn.stash); dev_free(sn.oldest); dev_free(sn.rows); dev_free(sn.free_rows); dev_free(sn.seen); dev_free(sn.st); dev_free(sn.sketch);
   sn.valid = false;
 }
 
@@ -758,6 +758,7 @@ int mono_table_create(mono_table** out, uint64_t capacity, uint32_t dim, uint32_
   if (cudaMemsetAsync(tv.rows + (size_t)capacity * 2 * dim, 0, (size_t)2 * dim * sizeof(float), t->stream) != cudaSuccess)
     return fail(MONO_ERR_CUDA);
   if ((rc = dev_alloc(t, &tv.free_rows, capacity)) != MONO_OK) return fail(rc);
+  if ((rc = dev_alloc(t, &tv.seen, capacity)) != MONO_OK) return fail(rc);
   if ((rc = dev_alloc(t, &tv.st, 1)) != MONO_OK) return fail(rc);
   tv.sketch_depth = o.sketch_depth;
   tv.sketch_seed = o.seed;
@@ -800,7 +801,7 @@ int mono_table_destroy(mono_table* t) {
   free_scratch(t);
   free_snapshot(t);
   free_group_scratch(t);
-  dev_free(t->tv.cells); dev_free(t->tv.stash); dev_free(t->tv.oldest); dev_free(t->tv.rows); dev_free(t->tv.free_rows); dev_free(t->tv.st); dev_free(t->tv.sketch);
+  dev_free(t->tv.cells); dev_free(t->tv.stash); dev_free(t->tv.oldest); dev_free(t->tv.rows); dev_free(t->tv.free_rows); dev_free(t->tv.seen); dev_free(t->tv.st); dev_free(t->tv.sketch);
   delete t;
   return MONO_OK;
 }
@@ -1263,6 +1264,7 @@ int mono_snapshot_save(mono_table* t) {
     if (rc == MONO_OK) rc = dev_alloc(t, &sn.oldest, t->key_cells / kCellsPerBucket);
     if (rc == MONO_OK) rc = dev_alloc(t, &sn.rows, row_floats);
     if (rc == MONO_OK) rc = dev_alloc(t, &sn.free_rows, tv.capacity);
+    if (rc == MONO_OK) rc = dev_alloc(t, &sn.seen, tv.capacity);
     if (rc == MONO_OK) rc = dev_alloc(t, &sn.st, 1);
     if (rc == MONO_OK && counters) rc = dev_alloc(t, &sn.sketch, counters);
     if (rc != MONO_OK) { free_snapshot(t); return rc; }
@@ -1275,6 +1277,7 @@ int mono_snapshot_save(mono_table* t) {
   CUDA_TRY(t, cudaMemcpyAsync(sn.oldest, tv.oldest, t->key_cells / kCellsPerBucket * sizeof(uint32_t), dd, s));
   CUDA_TRY(t, cudaMemcpyAsync(sn.rows, tv.rows, row_floats * sizeof(float), dd, s));
   CUDA_TRY(t, cudaMemcpyAsync(sn.free_rows, tv.free_rows, tv.capacity * sizeof(uint32_t), dd, s));
+  CUDA_TRY(t, cudaMemcpyAsync(sn.seen, tv.seen, tv.capacity * sizeof(uint32_t), dd, s));
   CUDA_TRY(t, cudaMemcpyAsync(sn.st, tv.st, sizeof(DevState), dd, s));
   if (counters) CUDA_TRY(t, cudaMemcpyAsync(sn.sketch, tv.sketch, counters * sizeof(unsigned int), dd, s));
   sn.last_now = t->last_now;
@@ -1301,6 +1304,7 @@ int mono_snapshot_restore(mono_table* t) {
   CUDA_TRY(t, cudaMemcpyAsync(tv.oldest, sn.oldest, t->key_cells / kCellsPerBucket * sizeof(uint32_t), dd, s));
   CUDA_TRY(t, cudaMemcpyAsync(tv.rows, sn.rows, row_floats * sizeof(float), dd, s));
   CUDA_TRY(t, cudaMemcpyAsync(tv.free_rows, sn.free_rows, tv.capacity * sizeof(uint32_t), dd, s));
+  CUDA_TRY(t, cudaMemcpyAsync(tv.seen, sn.seen, tv.capacity * sizeof(uint32_t), dd, s));
   CUDA_TRY(t, cudaMemcpyAsync(tv.st, sn.st, sizeof(DevState), dd, s));
   if (counters) CUDA_TRY(t, cudaMemcpyAsync(tv.sketch, sn.sketch, counters * sizeof(unsigned int), dd, s));
   t->last_now = sn.last_now;

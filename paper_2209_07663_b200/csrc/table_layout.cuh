@@ -17,7 +17,8 @@ namespace mono {
 // 16-byte loads from adjacent lanes (one 64-byte request, two DRAM sectors).
 //
 // meta, high 32 bits: last_seen (time of the last mono_apply_grads that held
-//                     the ID);
+//                     the ID); of an ID that owns a row, a time not after that one:
+//                     the row's own stamp (TableView::seen) has the exact time;
 // meta, low 32 bits : bit 31 set   -> the ID owns row (low 30 bits); bit 30 then marks a row
 //                     trained since the last mono_export_touched;
 //                     bit 31 clear -> still filtered, low 31 bits = occurrences
@@ -147,6 +148,12 @@ struct TableView {
   uint32_t* oldest;            // [n_buckets]: no entry of the bucket was last seen before this time (kNoStamp:
                                // none can be there); what the expiry sweep reads instead of the cells
   float* rows;                 // [capacity][2][dim]: weights then accumulator
+  // [capacity]: last_seen of the ID that owns the row.  Renewing the stamp of a batch's IDs in their cells is a line read and a
+  // line written per ID, scattered over the key store (2.3 M IDs: 104 us, the rate at which HBM moves lines); the rows' stamps
+  // are 4 bytes each, so a line serves several IDs (that kernel 104 -> 46 us, 8 M IDs 1323 -> 1269 per step, 1 M 142 -> 140).  The
+  // sweep pays a part of it back: of an entry whose cell's time is past the ttl it reads the row's (4 M entries of
+  // which 70 % go 82 -> 96 us).
+  uint32_t* seen;
   uint32_t* free_rows;         // [capacity]
   DevState* st;
   unsigned long long bucket_mask;   // n_buckets - 1
@@ -183,6 +190,8 @@ struct TableView {
     }
     return est;
   }
+  // last_seen of a tracked ID, from its cell's metadata
+  __device__ inline uint32_t last_seen(unsigned long long meta) const { return meta_resident(meta) ? seen[meta_row(meta)] : meta_time(meta); }
   __device__ inline float* w_row(uint32_t row) const { return rows + (size_t)row * 2u * dim; }
   __device__ inline float* acc_row(uint32_t row) const { return rows + (size_t)row * 2u * dim + dim; }
 };

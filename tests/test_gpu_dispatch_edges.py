@@ -254,3 +254,62 @@ def test_sweeps_of_sparse_and_dense_key_stores(n, key_cells, slices):
         assert (got["ids"] == ids[stay][order]).all() and (got["last_seen"] == seen[stay][order]).all()
     assert t.status()["error_bits"] == 0
     t.close()
+
+
+@pytest.mark.parametrize("announced", [False, True])
+@pytest.mark.parametrize("imported_at", [0, 40])
+def test_times_of_ids_that_own_rows(announced, imported_at):
+    """Their exact time is kept with the row, their cell's is a bound: pushes that leave the cell alone, that have to
+    mark it again after an export, and that come before the time in it (imported at 40); sweeps that open buckets for
+    cells whose rows were renewed; a snapshot, a rehash."""
+    n, ttl, dim = 300, 5, 4
+    ids = wl.splitmix64(np.arange(1, n + 1, dtype=np.uint64))
+    t = mb.MonoTable(512, dim, 1, ttl, key_cells=512)
+    t.import_entries(ids, np.ones(n, np.uint32), np.full(n, imported_at, np.int64), np.ones(n, np.uint8), None, None)
+    last = np.full(n, imported_at)
+
+    def check(what):
+        got = t.export(rows=False)
+        order = np.argsort(ids[last >= 0])
+        assert (got["ids"] == ids[last >= 0][order]).all(), what
+        assert (got["last_seen"] == last[last >= 0][order]).all(), what
+        d = torch.from_numpy(ids.view(np.int64)).cuda()
+        seen = torch.empty(n, dtype=torch.int64, device="cuda")
+        mb.mono_probe(t.handle, d, n, None, None, seen)
+        assert (seen.cpu().numpy() == last).all(), what
+        assert_audit_ok(t, what) if imported_at == 0 else None     # (a time that runs back leaves the sweep's record behind)
+
+    def push(which, now):
+        d = torch.from_numpy(ids[which].view(np.int64)).cuda()
+        off = torch.arange(d.numel() + 1, device="cuda")
+        if announced:
+            mb.mono_prepare_push(t.handle, d, d.numel(), off, d.numel())
+        mb.mono_apply_grads(t.handle, d, d.numel(), off, d.numel(), torch.zeros((d.numel(), dim), device="cuda"), now)
+        last[which] = now
+
+    k = np.arange(n)
+    push(k % 3 == 0, 1)
+    push(k % 3 == 0, 2)
+    push(k % 2 == 0, 4)
+    check("pushed")
+    assert t.export_touched()["found"] == int(((k % 3 == 0) | (k % 2 == 0)).sum())
+    push(k % 5 == 0, 5)
+    assert set(t.export_touched()["ids"]) == set(ids[k % 5 == 0])
+    mb.mono_snapshot_save(t.handle)
+    kept = last.copy()
+    push(k % 4 == 0, 6)
+    check("pushed again")
+    mb.mono_snapshot_restore(t.handle)
+    last[:] = kept
+    check("restored")
+    mb.mono_rehash(t.handle, 1024, 9)
+    check("rehashed")
+    if imported_at == 0:
+        for now in (6, 8, 10, 11):
+            t.expire(now)
+            last[(last >= 0) & (now - last > ttl)] = -1
+            check(f"swept at {now}")
+            if now == 8:
+                push((k % 7 == 0) & (last >= 0), 9)
+        assert (last >= 0).any() and (last < 0).any()
+    assert t.status()["error_bits"] == 0
