@@ -300,8 +300,7 @@ struct PoolTile {
 template <int G, int NV, int VW, typename Rows>
 __device__ __forceinline__ void pool_tile_body(const TableView& tv, const Rows& rows, uint32_t* __restrict__ spill, long long n_ids,
                                                const long long* __restrict__ offsets, long long n_bags, float* __restrict__ out,
-                                               uint32_t tile_bags, uint32_t vblock) {
-  __shared__ PoolTile sh;
+                                               uint32_t tile_bags, uint32_t vblock, PoolTile& sh) {
   constexpr int kGroups = 32 / G;
   const int lane = threadIdx.x & 31, gl = lane % G, grp = lane / G;
   const uint32_t dim = tv.dim;
@@ -412,14 +411,16 @@ template <int G, int NV, int VW, bool TOGETHER>
 __global__ void __launch_bounds__(kPoolThreads, (TOGETHER && G <= 8 ? 6 : pool_blocks_per_sm<G, NV, VW>()))
 probe_pool_kernel(TableView tv, const unsigned long long* __restrict__ ids, uint32_t* __restrict__ spill, long long n_ids,
                   const long long* __restrict__ offsets, long long n_bags, float* __restrict__ out, uint32_t tile_bags) { after_previous_kernel();
-  pool_tile_body<G, NV, VW>(tv, ProbedRows<kProbesInFlight<G>, TOGETHER>{tv, ids, tv.st->stash_hw}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x);
+  __shared__ PoolTile sh;
+  pool_tile_body<G, NV, VW>(tv, ProbedRows<kProbesInFlight<G>, TOGETHER>{tv, ids, tv.st->stash_hw}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x, sh);
 }
 
 template <int G, int NV, int VW>
 __global__ void __launch_bounds__(kPoolThreads, (pool_blocks_per_sm<G, NV, VW>()))
 gather_pool_kernel(TableView tv, Work wk, uint32_t* __restrict__ spill, long long n_ids, const long long* __restrict__ offsets,
                  long long n_bags, float* __restrict__ out, uint32_t tile_bags) { after_previous_kernel();
-  pool_tile_body<G, NV, VW>(tv, FiledRows<kFiledInFlight<G>>{wk, n_bags, (uint32_t)tv.capacity}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x);
+  __shared__ PoolTile sh;
+  pool_tile_body<G, NV, VW>(tv, FiledRows<kFiledInFlight<G>>{wk, n_bags, (uint32_t)tv.capacity}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x, sh);
 }
 
 }  // namespace mono

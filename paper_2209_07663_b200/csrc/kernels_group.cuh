@@ -36,13 +36,17 @@ struct GroupItem {
 };
 
 // Which table a block of a grouped launch belongs to: start[i] .. start[i+1] are table i's
-// blocks.  Returns the table and the block's number within it.
+// blocks.  Returns the table and the block's number within it.  Every warp searches, 32 places at a time: one at a time was
+// six reads one after the other for 64 tables, in every block of seven kernels (180 -> 176 us per step).
 __device__ inline uint32_t find_table(const uint32_t* __restrict__ start, uint32_t n_tables, uint32_t block,
                                       uint32_t* vblock, uint32_t* vgrid) {
-  uint32_t lo = 0, hi = n_tables;                        // start[lo] <= block < start[hi]
-  while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (__ldg(start + mid) <= block) lo = mid; else hi = mid;
+  uint32_t lo = 0, n = n_tables;                         // it is in [lo, lo + n), where start[lo] <= block
+  while (n > 1) {
+    const uint32_t step = (n + 31) / 32, at = (threadIdx.x & 31) * step;
+    const bool before = at < n && __ldg(start + lo + at) <= block;
+    const uint32_t c = __popc(__ballot_sync(0xFFFFFFFFu, before)) - 1;
+    lo += c * step;
+    n = min(step, n - c * step);
   }
   const uint32_t s0 = __ldg(start + lo), s1 = __ldg(start + lo + 1);
   *vblock = block - s0;
@@ -50,10 +54,25 @@ __device__ inline uint32_t find_table(const uint32_t* __restrict__ start, uint32
   return lo;
 }
 
+// A grouped call's descriptors and block maps, from the host's pinned copy.  (A copy by the DMA engine, and the way to it and
+// from there to the next kernel, left the GPU idle for ten microseconds: 64 tables 199.5 -> 180 us per step, three calls.)
+__global__ void __launch_bounds__(256)
+group_upload_kernel(uint4* __restrict__ dst, const uint4* src, uint32_t n) { after_previous_kernel();
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) dst[i] = __ldcv(src + i);
+}
+
+// A block's table: its descriptor, `it`, is copied to shared memory (read where it lies, in global memory, its fields
+// filled the registers and the kernels spilled: 64 tables 180.4 -> 178.9 us per step).
 #define MONO_GROUP_PROLOGUE                                                              \
   after_previous_kernel();                                                               \
   uint32_t vblock, vgrid;                                                                \
-  const GroupItem& it = items[find_table(start, n_tables, blockIdx.x, &vblock, &vgrid)]
+  __shared__ GroupItem it;                                                               \
+  {                                                                                      \
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(items + find_table(start, n_tables, blockIdx.x, &vblock, &vgrid)); \
+    for (uint32_t i = threadIdx.x; i < sizeof(GroupItem) / 8; i += blockDim.x) reinterpret_cast<unsigned long long*>(&it)[i] = __ldg(src + i); \
+  }                                                                                      \
+  __syncthreads()
 
 __global__ void __launch_bounds__(256)
 group_fill_occ_bag_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
@@ -133,9 +152,10 @@ template <int WIDE>
 __global__ void __launch_bounds__(kPoolThreads, WIDE ? 3 : 6)
 group_pool_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
+  __shared__ PoolTile sh;                                // (one for all widths: a block has one)
   const auto pool = [&](auto g, auto nv, auto vw) {
     pool_tile_body<decltype(g)::value, decltype(nv)::value, decltype(vw)::value>(it.tv, AnyRows{it}, it.occ_row, it.n_ids, it.off, it.n_bags, it.out,
-                                                                                 it.tile_bags, vblock);
+                                                                                 it.tile_bags, vblock, sh);
   };
   if (WIDE && it.pool_wide) {
     using W = std::integral_constant<int, 32>;
@@ -152,7 +172,7 @@ group_pool_kernel(const GroupItem* __restrict__ items, const uint32_t* __restric
 }
 
 template <int WIDE>
-__global__ void __launch_bounds__(kRowThreads, WIDE ? 4 : 10)
+__global__ void __launch_bounds__(kRowThreads, WIDE ? 4 : 8)
 group_update_rows_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   by_lane_class<WIDE>(it.lane_class, [&](auto g, auto nv) {

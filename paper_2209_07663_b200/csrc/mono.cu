@@ -678,7 +678,9 @@ int group_upload(GroupPlan& p, mono_table* const* tables) {
   }
   std::memcpy(g.host[slot], p.items.data(), p.items.size() * sizeof(GroupItem));
   std::memcpy(g.host[slot] + items_bytes, p.starts.data(), p.starts.size() * sizeof(uint32_t));
-  CUDA_TRY(p.owner, cudaMemcpyAsync(g.dev, g.host[slot], bytes, cudaMemcpyHostToDevice, p.gs));
+  const uint32_t words = (uint32_t)((bytes + 15) / 16);                  // (both buffers are larger)
+  launch_after(group_upload_kernel, (words + 255) / 256, 256, p.gs, reinterpret_cast<uint4*>(g.dev), reinterpret_cast<const uint4*>(g.host[slot]), words);
+  CUDA_TRY(p.owner, cudaGetLastError());
   CUDA_TRY(p.owner, cudaEventRecord(g.used[slot], p.gs));
   p.d_items = reinterpret_cast<const GroupItem*>(g.dev);
   p.d_starts = reinterpret_cast<const uint32_t*>(g.dev + items_bytes);
@@ -1011,8 +1013,9 @@ int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const ui
   for (int32_t i = 0; i < n_tables; ++i)
     group_describe(p, i, tables[i], ids[i], n_ids[i], slot_offsets[i], n_bags[i], nullptr, grad_pooled[i], (uint32_t)now, all_prepared);
   for (int32_t i = 0; i < n_tables; ++i) all_ids += n_ids[i];
+  // (half a table's share of the resident blocks: a block's preparations cost more here; 64 tables 63.3 -> 60.5 us, a quarter the same)
   for (int32_t i = 0; i < n_tables; ++i) {
-    p.items[i].row_grid = rows_grid(tables[i], n_ids[i], (double)n_ids[i] / (double)(all_ids ? all_ids : 1));
+    p.items[i].row_grid = rows_grid(tables[i], n_ids[i], 0.5 * (double)n_ids[i] / (double)(all_ids ? all_ids : 1));
     p.items[i].total_blocks = insert_grid(tables[i], n_ids[i]) + blocks_of(p.items[i].row_grid);
   }
   if ((rc = group_upload(p, tables)) != MONO_OK) return rc;

@@ -313,3 +313,39 @@ def test_times_of_ids_that_own_rows(announced, imported_at):
                 push((k % 7 == 0) & (last >= 0), 9)
         assert (last >= 0).any() and (last < 0).any()
     assert t.status()["error_bits"] == 0
+
+
+@pytest.mark.parametrize("n_tables", [1, 2, 31, 32, 33, 65, 150])
+def test_grouped_calls_find_every_block_its_table(n_tables):
+    """Numbers of tables around those that a warp searches at once; batches of very different size, every fifth empty.
+    Against the single-table calls on tables of their own."""
+    rng = np.random.default_rng(n_tables)
+    dims = [4, 20, 64, 128, 132]
+    pair, batch = [[], []], []
+    for i in range(n_tables):
+        for side in pair:
+            side.append(mb.MonoTable(256, dims[i % 5], 1, 0, key_cells=1024, init_scale=0.1, seed=i))
+        bags = 0 if i % 5 == 4 and i else int(rng.integers(1, 60)) if i % 7 else 900
+        ids = wl.splitmix64(rng.integers(0, 200, bags * 3).astype(np.uint64))
+        grad = (rng.standard_normal((bags, dims[i % 5])) * 0.01).astype(f32)
+        batch.append([torch.from_numpy(x).cuda() for x in (ids.view(np.int64), np.arange(0, 3 * bags + 1, 3), grad)])
+    ids, off, grad = ([b[k] for b in batch] for k in range(3))
+    grouped, single = [[t.handle for t in side] for side in pair]
+    for now in range(3):
+        out = [torch.full((b[1].numel() - 1, t.dim), float("nan"), device="cuda") for b, t in zip(batch, pair[0])]
+        if now:
+            mb.mono_group_prepare_push(grouped, ids, off)
+        mb.mono_group_lookup_pool(grouped, ids, off, out)
+        mb.mono_group_apply_grads(grouped, ids, off, grad, now)
+        for i, t in enumerate(single):
+            want = torch.zeros_like(out[i])
+            bags = off[i].numel() - 1
+            mb.mono_lookup_pool(t, ids[i], ids[i].numel(), off[i], bags, want)
+            mb.mono_apply_grads(t, ids[i], ids[i].numel(), off[i], bags, grad[i], now)
+            assert_vectors_close(out[i].cpu().numpy(), want.cpu().numpy(), f"table {i}, step {now}")
+    for g, s in zip(*pair):
+        a, b = g.export(), s.export()
+        assert (a["ids"] == b["ids"]).all() and (a["count"] == b["count"]).all() and (a["last_seen"] == b["last_seen"]).all()
+        assert_vectors_close(a["w"], b["w"], "rows")
+        assert_vectors_close(a["acc"], b["acc"], "accumulators")
+        assert g.status()["error_bits"] == 0
