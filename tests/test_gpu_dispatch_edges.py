@@ -349,3 +349,27 @@ def test_grouped_calls_find_every_block_its_table(n_tables):
         assert_vectors_close(a["w"], b["w"], "rows")
         assert_vectors_close(a["acc"], b["acc"], "accumulators")
         assert g.status()["error_bits"] == 0
+
+
+@pytest.mark.parametrize("repeated", [1, 255, 256, 4096, 4097])
+@pytest.mark.parametrize("dim", [4, 20, 64, 100, 132])
+@pytest.mark.parametrize("grouped", [False, True])
+def test_segments_of_every_length_in_small_and_large_numbers(repeated, dim, grouped):
+    """IDs that occur 1 to 66 times, so many of them repeated that a warp, or a lane group, takes each; alone and in a
+    grouped call."""
+    kw = dict(init_scale=0.05, seed=4)
+    gpu, cpu = mb.MonoTable(1 << 14, dim, 1, 0, **kw), mo.OracleTable(1 << 14, dim, 1, 0, **kw)
+    rng = np.random.default_rng(repeated + dim)
+    times = np.concatenate([np.arange(repeated) % 65 + 2, np.ones(50, np.int64)])
+    ids = rng.permutation(np.repeat(wl.splitmix64(np.arange(1, times.size + 1, dtype=np.uint64)), times))
+    off = np.unique(np.concatenate([[0, ids.size], rng.integers(0, ids.size, ids.size // 3)])).astype(np.int64)
+    grad = (rng.standard_normal((off.size - 1, dim)) * 0.01).astype(f32)
+    d = [torch.from_numpy(x).cuda() for x in (ids.view(np.int64), off, grad)]
+    for now in range(2):
+        if grouped:
+            mb.mono_group_apply_grads([gpu.handle], [d[0]], [d[1]], [d[2]], now)
+        else:
+            mb.mono_apply_grads(gpu.handle, d[0], ids.size, d[1], off.size - 1, d[2], now)
+        cpu.apply_grads(ids, off, grad, now)
+    assert_state_equal(gpu, cpu)
+    assert gpu.status()["error_bits"] == 0
