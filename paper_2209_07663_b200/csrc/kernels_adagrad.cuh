@@ -124,6 +124,41 @@ __device__ inline void reduce_segment(const Work& wk, const float* __restrict__ 
   }
 }
 
+// The same for one lane group of a grouped call's block, whose pointers are not constants of the launch: the lanes read the
+// bags' numbers together and hand them round, a load and its address less per row (64 tables: the row updates 60.5 ->
+// 56 us; a table's own launch, whose pointers are, gains nothing: 8 M IDs 642 -> 655, 1 M the same).
+template <int G, int NV>
+__device__ __forceinline__ void reduce_segment_together(const Work& wk, const float* __restrict__ grad, long long n_bags, uint32_t dim,
+                                                        int gl, uint32_t begin, uint32_t end, D4 (&s)[NV]) {
+  constexpr int kDepth = NV == 1 ? 8 : 4;
+  constexpr int kEach = kDepth > G ? kDepth / G : 1;                      // numbers a lane reads per chunk
+  const unsigned mask = G == 32 ? 0xFFFFFFFFu : ((1u << (G & 31)) - 1u) << ((threadIdx.x & 31) / G * G);
+  for (uint32_t i = begin; i < end; i += G * kEach) {                     // the same for the group
+    uint32_t mine[kEach];
+#pragma unroll
+    for (int r = 0; r < kEach; ++r) mine[r] = i + r * G + gl < end ? wk.bag_of_sorted[i + r * G + gl] : 0xFFFFFFFFu;
+#pragma unroll 1
+    for (int k0 = 0; k0 < G * kEach && i + k0 < end; k0 += kDepth) {
+      uint32_t b[kDepth];
+#pragma unroll
+      for (int k = 0; k < kDepth; ++k) b[k] = __shfl_sync(mask, mine[kEach > 1 ? k / G : 0], kEach > 1 ? k % G : k0 + k, G);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const uint32_t c4 = gl + v * G;
+        if (c4 * 4u < dim) {
+          float4 x[kDepth];
+#pragma unroll
+          for (int k = 0; k < kDepth; ++k)
+            x[k] = b[k] < n_bags ? __ldg(reinterpret_cast<const float4*>(grad + (size_t)b[k] * dim) + c4)
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int k = 0; k < kDepth; ++k) add4(s[v], x[k]);
+        }
+      }
+    }
+  }
+}
+
 // The filing pass of a push whose batch was not announced, or not pulled since (otherwise the pull
 // has filed the bags, FiledRows): one pass over the occurrences.
 __device__ inline void file_segments_body(const Work& wk, long long n_ids, long long n_bags, uint32_t vblock, uint32_t vgrid) {
@@ -208,7 +243,7 @@ struct Team {
 // order of every addition is fixed by the parts' numbers, whoever does it.  (A tree, because one ID
 // can own a tenth of a batch: with 64 neighbours at a time and then all the rest, adding up the
 // 11 000 parts of such an ID was a serial chain of 50 us.)
-template <int PG, int G, int NV>
+template <int PG, int G, int NV, bool TOGETHER>
 __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
                                     bool ordered, unsigned long long longs, uint32_t vblock, uint32_t vgrid) {
   const uint32_t n_parts = (uint32_t)longs, n_long = (uint32_t)(longs >> 32);
@@ -228,7 +263,8 @@ __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const f
     D4 s[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) s[v] = D4{0.0, 0.0, 0.0, 0.0};
-    reduce_segment<G, NV, PG / G>(wk, grad, n_bags, tv.dim, team.gl, begin + team.grp, end, s);
+    if constexpr (TOGETHER) reduce_segment_together<G, NV>(wk, grad, n_bags, tv.dim, team.gl, begin, end, s);
+    else reduce_segment<G, NV, PG / G>(wk, grad, n_bags, tv.dim, team.gl, begin + team.grp, end, s);
     team.template add_groups<NV>(s);
     const uint32_t parts = (m + kSegChunk - 1) / kSegChunk;
     bool top = true;
@@ -270,7 +306,7 @@ __device__ inline void reduce_parts(const TableView& tv, const Work& wk, const f
 // The repeated IDs: a team of PG lanes each, which reduces the segment, if it is short, and updates the row.
 // (Measured against one packed record per repeated ID, read a trip ahead: the separate arrays were 2 %
 // of a step faster on the largest configuration.)
-template <int PG, int G, int NV>
+template <int PG, int G, int NV, bool TOGETHER>
 __device__ inline void reduce_short(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
                                     uint32_t n, uint32_t vblock, uint32_t vgrid) {
   const Team<PG, G> team;
@@ -285,7 +321,8 @@ __device__ inline void reduce_short(const TableView& tv, const Work& wk, const f
     D4 s[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) s[v] = D4{0.0, 0.0, 0.0, 0.0};
-    reduce_segment<G, NV, PG / G>(wk, grad, n_bags, tv.dim, team.gl, begin + team.grp, begin + m, s);
+    if constexpr (TOGETHER) reduce_segment_together<G, NV>(wk, grad, n_bags, tv.dim, team.gl, begin, begin + m, s);
+    else reduce_segment<G, NV, PG / G>(wk, grad, n_bags, tv.dim, team.gl, begin + team.grp, begin + m, s);
     team.template add_groups<NV>(s);
     const unsigned long long id = wk.uid[u];
 #pragma unroll
@@ -402,14 +439,14 @@ __device__ __forceinline__ void update_rows_body(const TableView& tv, const Work
     // counts (step of 20 000 IDs 35.8 -> 28.4 us, of 135 000 56 -> 47).  Many: a lane group each, which
     // spends nothing on adding groups up (a warp each: 1 M IDs 154 -> 160 us, 4 M drifting 351 -> 370).
     // (A grouped call, whose tables share the SMs, has no use for it: FEW is false.)
-    if (G < 32 && (!FEW || (uint32_t)call.longs > kFewParts)) reduce_parts<G, G, NV>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
-    else reduce_parts<32, G, NV>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
+    if (G < 32 && (!FEW || (uint32_t)call.longs > kFewParts)) reduce_parts<G, G, NV, !FEW>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
+    else reduce_parts<32, G, NV, !FEW && G == 32>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
   } else if (vblock - grid.parts < grid.shorts) {
     // Likewise: up to 64 bags, eight or four at a time by a small lane group, are the longest chain of a small batch (20 000 IDs of 16
     // columns 10.1 -> 8.6 us, of 32 13.6 -> 13.2; with up to 8192 of them a warp each, 1 M IDs 55.3 -> 58.7).  Where
     // hardly any ID is repeated, adding the groups up is all it adds (160 IDs 6.1 -> 6.7).
-    if (G < 32 && (!FEW || call.n_multi > kFewParts || call.n_multi < kHardlyAny)) reduce_short<G, G, NV>(tv, wk, grad, n_bags, call.n_multi, vblock - grid.parts, grid.shorts);
-    else reduce_short<32, G, NV>(tv, wk, grad, n_bags, call.n_multi, vblock - grid.parts, grid.shorts);
+    if (G < 32 && (!FEW || call.n_multi > kFewParts || call.n_multi < kHardlyAny)) reduce_short<G, G, NV, !FEW>(tv, wk, grad, n_bags, call.n_multi, vblock - grid.parts, grid.shorts);
+    else reduce_short<32, G, NV, !FEW && G == 32>(tv, wk, grad, n_bags, call.n_multi, vblock - grid.parts, grid.shorts);
   } else {
     update_singletons<G, NV>(tv, wk, grad, n_bags, call.n_unique, vblock - grid.parts - grid.shorts, grid.singles);
     clear_primary(wk, vblock - grid.parts - grid.shorts, grid.singles);
