@@ -152,11 +152,10 @@ __device__ __forceinline__ void add_rows(const float* __restrict__ rows, uint32_
 }
 
 // dst[0..dim) = sum of the rows idx[0..n), in that order, by a group of G lanes.  The rows go in
-// batches of eight (four of 32-byte accesses), what is left in one batch of its exact size: no
+// batches of K, what is left in one batch of its exact size: no
 // per-row tests (an ID without a row points at the table's all-zero row), no loads for padding.
-template <int G, int NV, int VW>
+template <int K, int G, int NV, int VW>
 __device__ __forceinline__ void pool_bag(const float* __restrict__ rows, uint32_t dim, const uint32_t* idx, uint32_t n, int gl, float* __restrict__ dst) {
-  constexpr int K = VW == 8 ? 4 : 8;
   Vec<VW> sum[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v)
@@ -165,6 +164,10 @@ __device__ __forceinline__ void pool_bag(const float* __restrict__ rows, uint32_
   uint32_t i = 0;
   for (; i + K <= n; i += K) add_rows<K, G, NV, VW>(rows, dim, idx + i, gl, sum);
   switch (n - i) {
+    case 11: if constexpr (K > 11) add_rows<11, G, NV, VW>(rows, dim, idx + i, gl, sum); break;
+    case 10: if constexpr (K > 10) add_rows<10, G, NV, VW>(rows, dim, idx + i, gl, sum); break;
+    case 9: if constexpr (K > 9) add_rows<9, G, NV, VW>(rows, dim, idx + i, gl, sum); break;
+    case 8: if constexpr (K > 8) add_rows<8, G, NV, VW>(rows, dim, idx + i, gl, sum); break;
     case 7: if constexpr (K > 7) add_rows<7, G, NV, VW>(rows, dim, idx + i, gl, sum); break;
     case 6: if constexpr (K > 6) add_rows<6, G, NV, VW>(rows, dim, idx + i, gl, sum); break;
     case 5: if constexpr (K > 5) add_rows<5, G, NV, VW>(rows, dim, idx + i, gl, sum); break;
@@ -297,7 +300,7 @@ struct PoolTile {
   unsigned int next;
 };
 
-template <int G, int NV, int VW, typename Rows>
+template <int K, int G, int NV, int VW, typename Rows>
 __device__ __forceinline__ void pool_tile_body(const TableView& tv, const Rows& rows, uint32_t* __restrict__ spill, long long n_ids,
                                                const long long* __restrict__ offsets, long long n_bags, float* __restrict__ out,
                                                uint32_t tile_bags, uint32_t vblock, PoolTile& sh) {
@@ -366,7 +369,7 @@ __device__ __forceinline__ void pool_tile_body(const TableView& tv, const Rows& 
     i += grp;
     if (i < n_sums) {
       const uint32_t b = sh.order[i];
-      pool_bag<G, NV, VW>(tv.rows, dim, idx + sh.begin[b], sh.len[b], gl, out + (b0 + b) * (long long)dim);
+      pool_bag<K, G, NV, VW>(tv.rows, dim, idx + sh.begin[b], sh.len[b], gl, out + (b0 + b) * (long long)dim);
     }
     __syncwarp();
   }
@@ -398,7 +401,10 @@ __device__ __forceinline__ void pool_tile_body(const TableView& tv, const Rows& 
 // 512 columns in 32-byte accesses need 80 registers, three blocks: at the 64 of four they spill, and the pull of 2048 bags of
 // up to 64 IDs of 1024 columns took 54 us against 40, of 65 536 bags of up to 8 IDs 106 against 98.  (In 16-byte
 // accesses four stay: three are 50 -> 40 us for the long bags of 516 columns, but 72.7 -> 76.8 for the many short ones.)
-template <int G, int NV, int VW> constexpr int pool_blocks_per_sm() { return NV * VW == 32 && VW == 8 ? 3 : NV > 1 ? 4 : G <= 8 ? 8 : 6; }
+// DEEP, for long bags in batches that are bound by the latency of their rows rather than of their look-ups (pools_deep() on the
+// host has the rule and the figures): half as many rows again in flight per lane group, at four blocks.
+template <int G, int NV, int VW, bool DEEP> constexpr int pool_blocks_per_sm() { return DEEP ? 4 : NV * VW == 32 && VW == 8 ? 3 : NV > 1 ? 4 : G <= 8 ? 8 : 6; }
+template <int VW, bool DEEP> __host__ __device__ constexpr int pool_batch() { return VW == 8 ? (DEEP ? 6 : 4) : (DEEP ? 12 : 8); }
 // (Filing is a chain of two reads, a batch's own record and its ID's slot of the per-call set: four at a time, 8 M IDs of
 // 64 columns 1365 -> 1346 us per step, timed in turn; at the 32 registers of the narrow rows they spill, 4 M IDs 343 -> 359.)
 template <int G> constexpr int kProbesInFlight = G <= 8 ? 1 : 2;
@@ -407,20 +413,20 @@ template <int G> constexpr int kFiledInFlight = G <= 8 ? 1 : 4;
 // TOGETHER (launch_pool): of a look-up that misses the preferred cell, the rest at once.  It needs
 // the registers of six blocks per SM, which narrow rows only have to spare in a batch of one wave of blocks
 // (one request of 208 bags 5.7 -> 4.8 us; 213 000 bags 31.8 -> 32.8, so larger ones look on bucket by bucket).
-template <int G, int NV, int VW, bool TOGETHER>
-__global__ void __launch_bounds__(kPoolThreads, (TOGETHER && G <= 8 ? 6 : pool_blocks_per_sm<G, NV, VW>()))
+template <int G, int NV, int VW, bool TOGETHER, bool DEEP>
+__global__ void __launch_bounds__(kPoolThreads, (TOGETHER && G <= 8 ? 6 : pool_blocks_per_sm<G, NV, VW, DEEP>()))
 probe_pool_kernel(TableView tv, const unsigned long long* __restrict__ ids, uint32_t* __restrict__ spill, long long n_ids,
                   const long long* __restrict__ offsets, long long n_bags, float* __restrict__ out, uint32_t tile_bags) { after_previous_kernel();
   __shared__ PoolTile sh;
-  pool_tile_body<G, NV, VW>(tv, ProbedRows<kProbesInFlight<G>, TOGETHER>{tv, ids, tv.st->stash_hw}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x, sh);
+  pool_tile_body<pool_batch<VW, DEEP>(), G, NV, VW>(tv, ProbedRows<kProbesInFlight<G>, TOGETHER>{tv, ids, tv.st->stash_hw}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x, sh);
 }
 
-template <int G, int NV, int VW>
-__global__ void __launch_bounds__(kPoolThreads, (pool_blocks_per_sm<G, NV, VW>()))
+template <int G, int NV, int VW, bool DEEP>
+__global__ void __launch_bounds__(kPoolThreads, (pool_blocks_per_sm<G, NV, VW, DEEP>()))
 gather_pool_kernel(TableView tv, Work wk, uint32_t* __restrict__ spill, long long n_ids, const long long* __restrict__ offsets,
                  long long n_bags, float* __restrict__ out, uint32_t tile_bags) { after_previous_kernel();
   __shared__ PoolTile sh;
-  pool_tile_body<G, NV, VW>(tv, FiledRows<kFiledInFlight<G>>{wk, n_bags, (uint32_t)tv.capacity}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x, sh);
+  pool_tile_body<pool_batch<VW, DEEP>(), G, NV, VW>(tv, FiledRows<kFiledInFlight<G>>{wk, n_bags, (uint32_t)tv.capacity}, spill, n_ids, offsets, n_bags, out, tile_bags, blockIdx.x, sh);
 }
 
 }  // namespace mono

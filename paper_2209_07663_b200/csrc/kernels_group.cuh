@@ -154,7 +154,7 @@ group_pool_kernel(const GroupItem* __restrict__ items, const uint32_t* __restric
   MONO_GROUP_PROLOGUE;
   __shared__ PoolTile sh;                                // (one for all widths: a block has one)
   const auto pool = [&](auto g, auto nv, auto vw) {
-    pool_tile_body<decltype(g)::value, decltype(nv)::value, decltype(vw)::value>(it.tv, AnyRows{it}, it.occ_row, it.n_ids, it.off, it.n_bags, it.out,
+    pool_tile_body<pool_batch<decltype(vw)::value, false>(), decltype(g)::value, decltype(nv)::value, decltype(vw)::value>(it.tv, AnyRows{it}, it.occ_row, it.n_ids, it.off, it.n_bags, it.out,
                                                                                  it.tile_bags, vblock, sh);
   };
   if (WIDE && it.pool_wide) {

@@ -367,19 +367,39 @@ uint32_t pool_tile(int64_t n_ids, int64_t n_bags, int64_t slots, int groups) {
   return (uint32_t)(tile < 8 ? 8 : tile);
 }
 
+// Whether a pull takes the kernels with more rows in flight and fewer warps.  Bags of six IDs and more, and then: rows that go in
+// 32-byte accesses, whose groups fill a warp (us, announced in brackets: 41 000 bags of up to 64 IDs of 200 columns 87 -> 84 [80 -> 77],
+// 2000 bags 18.9 -> 14.0 [10.8 -> 8.6]; with bags of up to 8 IDs 30.1 -> 31.0, so not those); of an announced batch, whose rows are found
+// in one read, others too while its tiles are one wave (2048 bags of up to 64 IDs of 16 columns 12.6 -> 8.4, of 64 7.6 -> 6.4, 20 000 of up to 24
+// 9.8 -> 8.7 and 10.0 -> 9.5; two waves of 32 columns 17.9 -> 19.9); of one that was not, rows of 33 to 128 columns while its
+// look-ups do not need the warps (2048 bags of up to 64 IDs of 64 columns 11.0 -> 8.8; 20 000 29.2 -> 31.4).
+bool pools_deep(const mono_table* t, int64_t n_ids, int64_t n_bags, int lanes, int floats, bool filed) {
+  if (n_ids < 6 * n_bags) return false;
+  if (floats == 8) return true;
+  const int64_t wave = (int64_t)850 * t->sm_count;                       // IDs of a tile per SM
+  return filed ? n_ids <= 4 * wave : lanes >= 16 && n_ids <= wave;
+}
+
 // The pull: one kernel, which takes the rows from the key store, or, for a batch that was announced
 // (`filed`), from the per-call set, filing the bags for the push on the way.
 int launch_pool(mono_table* t, const unsigned long long* ids, uint32_t* spill, int64_t n_ids, const long long* off, int64_t n_bags,
                 float* out, bool filed) {
   return dispatch_pool(t->tv.dim, out, [&](auto g, auto nv, auto vw) -> int {
     constexpr int G = decltype(g)::value, NV = decltype(nv)::value, VW = decltype(vw)::value;
-    const uint32_t tile = pool_tile(n_ids, n_bags, grid_for(t, pool_blocks_per_sm<G, NV, VW>()), kPoolThreads / G);
-    const unsigned blocks = (unsigned)((n_bags + tile - 1) / tile);
-    if (filed) LAUNCH(t, K_POOL, launch_after(gather_pool_kernel<G, NV, VW>, blocks, kPoolThreads, t->stream, t->tv, t->wk, spill, n_ids, off, n_bags, out, tile));
-    else if (G > 8 || (int64_t)blocks <= grid_for(t, 6)) LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW, true>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
-    else LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW, (G > 8)>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
-    CUDA_TRY(t, cudaGetLastError());
-    return (int)MONO_OK;
+    const auto launch = [&](auto deep) -> int {
+      constexpr bool D = decltype(deep)::value;
+      const uint32_t tile = pool_tile(n_ids, n_bags, grid_for(t, pool_blocks_per_sm<G, NV, VW, D>()), kPoolThreads / G);
+      const unsigned blocks = (unsigned)((n_bags + tile - 1) / tile);
+      if (filed) LAUNCH(t, K_POOL, launch_after(gather_pool_kernel<G, NV, VW, D>, blocks, kPoolThreads, t->stream, t->tv, t->wk, spill, n_ids, off, n_bags, out, tile));
+      else if (G > 8 || (int64_t)blocks <= grid_for(t, 6)) LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW, true, D && (G > 8)>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
+      else LAUNCH(t, K_POOL, launch_after(probe_pool_kernel<G, NV, VW, (G > 8), D && (G > 8)>, blocks, kPoolThreads, t->stream, t->tv, ids, spill, n_ids, off, n_bags, out, tile));
+      CUDA_TRY(t, cudaGetLastError());
+      return (int)MONO_OK;
+    };
+    if constexpr (NV == 1) {
+      if (pools_deep(t, n_ids, n_bags, G, VW, filed)) return launch(std::true_type{});
+    }
+    return launch(std::false_type{});
   });
 }
 

@@ -373,3 +373,14 @@ def test_segments_of_every_length_in_small_and_large_numbers(repeated, dim, grou
         cpu.apply_grads(ids, off, grad, now)
     assert_state_equal(gpu, cpu)
     assert gpu.status()["error_bits"] == 0
+
+
+@pytest.mark.parametrize("dim", [16, 32, 64, 128, 136, 256])
+@pytest.mark.parametrize("bags, mean", [(300, 3), (300, 9), (3000, 40), (16000, 40)])
+def test_pulls_of_short_and_long_bags_in_small_and_large_batches(dim, bags, mean):
+    """Both sides of the rule that takes more rows in flight: by the mean bag length, by the size of the batch (one tile
+    of 850 IDs per SM, four), announced and not; bags of every length up to twice the mean, so every remainder."""
+    t, ids, w = filled(dim)
+    rng = np.random.default_rng(bags + mean)
+    pulls(t, ids, w, rng.integers(0, 2 * mean + 1, bags), rng)
+    assert t.status()["error_bits"] == 0
