@@ -54,12 +54,13 @@ __device__ inline uint32_t find_table(const uint32_t* __restrict__ start, uint32
   return lo;
 }
 
-// A grouped call's descriptors and block maps, from the host's pinned copy.  (A copy by the DMA engine, and the way to it and
-// from there to the next kernel, left the GPU idle for ten microseconds: 64 tables 199.5 -> 180 us per step, three calls.)
+// A grouped call's descriptors and block maps, from the host's pinned copy: n words, of which the smaller of the two
+// buffers holds `room`.  (A copy by the DMA engine, and the way to it and from there to the next kernel, left the GPU
+// idle for ten microseconds: 64 tables 199.5 -> 180 us per step, three calls.)
 __global__ void __launch_bounds__(256)
-group_upload_kernel(uint4* __restrict__ dst, const uint4* src, uint32_t n) { after_previous_kernel();
+group_upload_kernel(uint4* __restrict__ dst, const uint4* src, uint32_t n, uint32_t room, unsigned int* error_bits) { after_previous_kernel();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = __ldcv(src + i);
+  if (i < n && MONO_INDEX_OK(error_bits, i, room)) dst[i] = __ldcv(src + i);
 }
 
 // A block's table: its descriptor, `it`, is copied to shared memory (read where it lies, in global memory, its fields

@@ -678,7 +678,8 @@ int group_upload(GroupPlan& p, mono_table* const* tables) {
   }
   auto& g = p.owner->grp;
   const size_t items_bytes = ((p.items.size() * sizeof(GroupItem) + 255) / 256) * 256;
-  const size_t bytes = items_bytes + p.starts.size() * sizeof(uint32_t);
+  // whole 16-byte words, which is what the upload copies: neither buffer may be kept for a call that it lacks a part of a word for
+  const size_t bytes = (items_bytes + p.starts.size() * sizeof(uint32_t) + 15) / 16 * 16;
   if (bytes > g.dev_bytes) {
     CUDA_TRY(p.owner, cudaStreamSynchronize(p.gs));
     if (g.dev) cudaFree(g.dev);
@@ -698,8 +699,9 @@ int group_upload(GroupPlan& p, mono_table* const* tables) {
   }
   std::memcpy(g.host[slot], p.items.data(), p.items.size() * sizeof(GroupItem));
   std::memcpy(g.host[slot] + items_bytes, p.starts.data(), p.starts.size() * sizeof(uint32_t));
-  const uint32_t words = (uint32_t)((bytes + 15) / 16);                  // (both buffers are larger)
-  launch_after(group_upload_kernel, (words + 255) / 256, 256, p.gs, reinterpret_cast<uint4*>(g.dev), reinterpret_cast<const uint4*>(g.host[slot]), words);
+  const uint32_t words = (uint32_t)(bytes / 16), room = (uint32_t)(std::min(g.dev_bytes, g.host_bytes[slot]) / 16);
+  launch_after(group_upload_kernel, (words + 255) / 256, 256, p.gs, reinterpret_cast<uint4*>(g.dev), reinterpret_cast<const uint4*>(g.host[slot]), words, room,
+               &p.owner->tv.st->error_bits);
   CUDA_TRY(p.owner, cudaGetLastError());
   CUDA_TRY(p.owner, cudaEventRecord(g.used[slot], p.gs));
   p.d_items = reinterpret_cast<const GroupItem*>(g.dev);
