@@ -226,7 +226,11 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
         // every ID of the batch that has a row is trained in this call: mark it for the next sync
         if (resident) { row_word = low & kRowMask; low |= kTouchedBit; }
         else if (rv.row != kNoRow) { low = kResidentBit | kTouchedBit | rv.row; row_word = rv.row | kFreshBit; }
-        if (!settled) cell_address(tv, cell, n_cells)->meta = make_meta(now, low);
+        if (!settled) {
+          cell_address(tv, cell, n_cells)->meta = make_meta(now, low);
+          // (an entry imported at a later time than this push's: its bucket's record may not stay above it.  The stash has none.)
+          if (now < meta_time(meta) && cell < n_cells) atomicMin(tv.oldest + cell / kCellsPerBucket, now);
+        }
         wk.urow[u] = row_word;
         if (row_word != kNoRow) {
           if (MONO_INDEX_OK(&tv.st->error_bits, row_word & ~kFreshBit, tv.capacity)) tv.seen[row_word & ~kFreshBit] = now;
@@ -259,7 +263,8 @@ table_update_kernel(TableView tv, Work wk, uint32_t now) { after_previous_kernel
 // An entry whose metadata is `meta` has just been written into a cell of bucket `bkt`: the
 // bucket's record of its oldest stamp may not stay above that entry's.  (Entries that leave a
 // bucket, and stamps that are renewed, leave the record as it is: it only has to be a lower
-// bound, and the sweep makes it exact again whenever it visits the bucket.)  `rec` is the
+// bound, and the sweep makes it exact again whenever it visits the bucket.  A stamp that a push takes
+// back, of an entry imported at a later time, lowers it: table_update_body.)  `rec` is the
 // record as read before the write; records only fall while entries are being inserted, so a
 // value read earlier is at or above the present one and the test errs on the safe side.
 __device__ inline void note_stamp(const TableView& tv, unsigned long long bkt, unsigned long long meta, uint32_t rec) {
