@@ -431,33 +431,32 @@ struct RowGrid { uint32_t parts, shorts, singles; };
 
 template <int G, int NV, bool FEW>
 __device__ __forceinline__ void update_rows_body(const TableView& tv, const Work& wk, const float* __restrict__ grad, long long n_bags,
-                                                 bool ordered, const RowGrid& grid, uint32_t total_blocks, uint32_t vblock) {
-  __shared__ CheckIn call;
-  check_in(wk, &call);
+                                                 bool ordered, const RowGrid& grid, uint32_t vblock) {
   if (vblock < grid.parts) {
+    const unsigned long long longs = wk.call->longs;
     // Few parts (they are resident all at once): a warp each, because the longest chain of loads is what
     // counts (step of 20 000 IDs 35.8 -> 28.4 us, of 135 000 56 -> 47).  Many: a lane group each, which
     // spends nothing on adding groups up (a warp each: 1 M IDs 154 -> 160 us, 4 M drifting 351 -> 370).
     // (A grouped call, whose tables share the SMs, has no use for it: FEW is false.)
-    if (G < 32 && (!FEW || (uint32_t)call.longs > kFewParts)) reduce_parts<G, G, NV, !FEW>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
-    else reduce_parts<32, G, NV, !FEW && G == 32>(tv, wk, grad, n_bags, ordered, call.longs, vblock, grid.parts);
+    if (G < 32 && (!FEW || (uint32_t)longs > kFewParts)) reduce_parts<G, G, NV, !FEW>(tv, wk, grad, n_bags, ordered, longs, vblock, grid.parts);
+    else reduce_parts<32, G, NV, !FEW && G == 32>(tv, wk, grad, n_bags, ordered, longs, vblock, grid.parts);
   } else if (vblock - grid.parts < grid.shorts) {
     // Likewise: up to 64 bags, eight or four at a time by a small lane group, are the longest chain of a small batch (20 000 IDs of 16
     // columns 10.1 -> 8.6 us, of 32 13.6 -> 13.2; with up to 8192 of them a warp each, 1 M IDs 55.3 -> 58.7).  Where
     // hardly any ID is repeated, adding the groups up is all it adds (160 IDs 6.1 -> 6.7).
-    if (G < 32 && (!FEW || call.n_multi > kFewParts || call.n_multi < kHardlyAny)) reduce_short<G, G, NV, !FEW>(tv, wk, grad, n_bags, call.n_multi, vblock - grid.parts, grid.shorts);
-    else reduce_short<32, G, NV, !FEW && G == 32>(tv, wk, grad, n_bags, call.n_multi, vblock - grid.parts, grid.shorts);
+    const uint32_t n_multi = wk.call->n_multi;
+    if (G < 32 && (!FEW || n_multi > kFewParts || n_multi < kHardlyAny)) reduce_short<G, G, NV, !FEW>(tv, wk, grad, n_bags, n_multi, vblock - grid.parts, grid.shorts);
+    else reduce_short<32, G, NV, !FEW && G == 32>(tv, wk, grad, n_bags, n_multi, vblock - grid.parts, grid.shorts);
   } else {
-    update_singletons<G, NV>(tv, wk, grad, n_bags, call.n_unique, vblock - grid.parts - grid.shorts, grid.singles);
+    update_singletons<G, NV>(tv, wk, grad, n_bags, wk.call->n_unique, vblock - grid.parts - grid.shorts, grid.singles);
     clear_primary(wk, vblock - grid.parts - grid.shorts, grid.singles);
   }
-  check_out(tv.st, wk, &call, total_blocks);
 }
 template <int G, int NV>
 __global__ void __launch_bounds__(kRowThreads, NV == 1 ? 10 : NV == 2 ? 7 : 4)
-update_rows_kernel(TableView tv, Work wk, const float* __restrict__ grad, long long n_bags, int ordered, RowGrid grid, uint32_t total_blocks) {
+update_rows_kernel(TableView tv, Work wk, const float* __restrict__ grad, long long n_bags, int ordered, RowGrid grid) {
   after_previous_kernel();
-  update_rows_body<G, NV, true>(tv, wk, grad, n_bags, ordered != 0, grid, total_blocks, blockIdx.x);
+  update_rows_body<G, NV, true>(tv, wk, grad, n_bags, ordered != 0, grid, blockIdx.x);
 }
 
 }  // namespace mono

@@ -75,7 +75,7 @@ struct Work {
   uint32_t* long_part0;      // [max_long] first part of each
   uint32_t* part_u;          // [max_parts] owner (index into long_u) of each part
   uint32_t* part_order;      // [max_parts] the parts in the order they are reduced in: by window of the batch
-  uint32_t* win_count;       // [2 * kWindows] parts per window, then a cursor per window; zero between calls
+  uint32_t* win_count;       // [2 * kWindows] parts per window, then a cursor per window; zero when expand_parts starts
   double* partials;          // [max_parts][dim]
   uint32_t* part_done;       // [max_parts] partial sums that are there, counted at the first of the kFanIn that belong together; zero between calls
   uint32_t max_long, max_parts;
@@ -92,9 +92,14 @@ __device__ inline bool bag_ok(long long lo, long long hi, long long n_ids) { ret
 // bag -> occurrences: every occurrence learns which bag it belongs to.  A malformed bag
 // writes nothing and marks the call, so that the grouping pass checks every occurrence against the
 // bag it claims (occurrence_covered) and the look-up that follows sets the sticky condition bit.
+// The batch's counters start here.
 __device__ inline void fill_occ_bag_body(const long long* __restrict__ offsets, long long n_bags, long long n_ids,
                                          uint32_t* __restrict__ occ_bag, CallState* call, uint32_t vblock, uint32_t vgrid) {
   const long long stride = (long long)vgrid * blockDim.x;
+  if (vblock == 0 && threadIdx.x == 0) {
+    call->longs = 0ull;
+    call->n_unique = call->n_valid_ids = call->n_insert = call->n_multi = call->seg_cursor = 0u;
+  }
   for (long long b = (long long)vblock * blockDim.x + threadIdx.x; b < n_bags; b += stride) {
     const long long lo = offsets[b], hi = offsets[b + 1];
     if (!bag_ok(lo, hi, n_ids)) { call->bad_offsets = 1u; continue; }

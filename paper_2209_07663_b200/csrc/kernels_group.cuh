@@ -31,7 +31,6 @@ struct GroupItem {
   uint32_t pool_wide;            // lookup: 32-byte accesses (classes 4..6 only)
   uint32_t tile_bags;            // lookup: bags per block
   RowGrid row_grid;              // push: the row updates' blocks
-  uint32_t total_blocks;         // push: of the insertions and the row updates together
   uint32_t active;               // 0: the table takes no part in this call (empty batch)
 };
 
@@ -103,7 +102,7 @@ group_sketch_add_kernel(const GroupItem* __restrict__ items, const uint32_t* __r
 __global__ void __launch_bounds__(256)
 group_table_insert_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
-  table_insert_body(it.tv, it.wk, it.now, it.total_blocks, vblock, vgrid);
+  table_insert_body(it.tv, it.wk, it.now, vblock, vgrid);
 }
 
 // (of a push whose batch was not pulled since it was announced, or not announced)
@@ -177,7 +176,7 @@ __global__ void __launch_bounds__(kRowThreads, WIDE ? 4 : 8)
 group_update_rows_kernel(const GroupItem* __restrict__ items, const uint32_t* __restrict__ start, uint32_t n_tables) {
   MONO_GROUP_PROLOGUE;
   by_lane_class<WIDE>(it.lane_class, [&](auto g, auto nv) {
-    update_rows_body<decltype(g)::value, decltype(nv)::value, false>(it.tv, it.wk, it.grad, it.n_bags, false, it.row_grid, it.total_blocks, vblock);
+    update_rows_body<decltype(g)::value, decltype(nv)::value, false>(it.tv, it.wk, it.grad, it.n_bags, false, it.row_grid, vblock);
   });
 }
 

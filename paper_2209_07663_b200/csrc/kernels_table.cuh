@@ -156,7 +156,10 @@ __device__ inline void table_update_body(const TableView& tv, const Work& wk, ui
   const unsigned long long n_cells = (tv.bucket_mask + 1) * kCellsPerBucket;
   const int lane = threadIdx.x & 31;
   unsigned int n_res = 0;
-  if ((MODE & kLookUp) && vblock == 0 && threadIdx.x == 0 && wk.call->bad_offsets) atomicOr(&tv.st->error_bits, 4u /* MONO_DEV_BAD_OFFSETS */);
+  if ((MODE & kLookUp) && vblock == 0 && threadIdx.x == 0 && wk.call->bad_offsets) {
+    atomicOr(&tv.st->error_bits, 4u /* MONO_DEV_BAD_OFFSETS */);
+    wk.call->bad_offsets = 0u;
+  }
   for (uint32_t base = vblock * blockDim.x; base < n; base += vgrid * blockDim.x) {   // block-uniform
     const uint32_t u = base + threadIdx.x;
     const bool active = u < n;
@@ -340,57 +343,6 @@ __device__ inline void cuckoo_insert(const TableView& tv, Cell item) {
   if (meta_resident(item.meta)) atomicAdd(&tv.st->n_resident, (unsigned long long)(-1LL));
 }
 
-// End of a mono_apply_grads call: fold the per-call counters into the totals and zero them
-// (commit = 0: a grouping that was prepared but never applied is only forgotten).  One warp.
-__device__ inline void close_call(DevState* st, const Work& wk, int commit) {
-  CallState* call = wk.call;
-  const bool had_parts = call->longs != 0ull;
-  __syncwarp();                                      // every lane has read it before it is reset
-  if (had_parts)
-    for (uint32_t i = threadIdx.x & 31; i < 2 * kWindows; i += 32) wk.win_count[i] = 0;
-  if ((threadIdx.x & 31) == 0) {
-    if (commit) {
-      st->sum_ids += call->n_valid_ids;
-      st->sum_unique += call->n_unique;
-      st->sum_new += call->n_insert;
-    }
-    CallState zero = {};
-    *call = zero;
-  }
-}
-__global__ void __launch_bounds__(32)
-forget_call_kernel(DevState* st, Work wk) { after_previous_kernel();
-  if (blockIdx.x == 0) close_call(st, wk, 0);
-}
-
-// A push ends with two kernels that need not follow one another, the insertions and the row updates.  The last of
-// all their `total` blocks closes the call.  What closing takes away are the call's counters, so a block checks in as
-// soon as it has them (one thread reads them, for the block), and the block that is last to check in knows that all others
-// have them too.  (Checking in at the end, behind a barrier and a fence, kept every block's place on the SM for two
-// more microseconds: row updates of 4 M drifting IDs 118 -> 103 us, of 1 M 58.5 -> 56, of 20 000 12.4 -> 10.3; grouped, 64
-// tables, 70 -> 63.  With the ticket in a register to the end, instead of in shared memory, the row updates spill: 8 M
-// IDs 644 -> 662.)
-struct CheckIn {
-  unsigned long long longs;
-  unsigned int n_unique, n_multi, n_insert;
-  unsigned int ticket;
-};
-__device__ inline void check_in(const Work& wk, CheckIn* sh) {
-  if (threadIdx.x == 0) {
-    sh->longs = wk.call->longs;
-    sh->n_unique = wk.call->n_unique;
-    sh->n_multi = wk.call->n_multi;
-    sh->n_insert = wk.call->n_insert;
-  }
-  __syncthreads();                                   // (the counters are here: thread 0 has put them into shared memory)
-  if (threadIdx.x == 0) sh->ticket = atomicAdd(&wk.call->blocks_in, 1u);
-}
-__device__ inline void check_out(DevState* st, const Work& wk, const CheckIn* sh, uint32_t total) {
-  if (threadIdx.x >= 32) return;
-  __syncwarp();
-  if (sh->ticket == total - 1u) close_call(st, wk, 1);
-}
-
 // Probabilistic filter, between phases 2 and 3: every distinct ID that is not in the key
 // store adds its multiplicity to one counter per sketch row.  All additions of a batch are
 // done before any estimate is read (next kernel), so the outcome does not depend on order.
@@ -412,11 +364,16 @@ sketch_add_kernel(TableView tv, Work wk) { after_previous_kernel(); sketch_add_b
 // the threshold) was settled in phase 2, which left the row in urow[], so nothing that
 // updates rows waits for this kernel.  Probabilistic filter: it is inserted, with a row,
 // only if its sketch estimate has reached the threshold; otherwise nothing is stored for it.
-__device__ inline void table_insert_body(const TableView& tv, const Work& wk, uint32_t now, uint32_t total_blocks, uint32_t vblock, uint32_t vgrid) {
+// The batch's counters are added to the table's totals here: nothing adds to them any more, and the row updates beside
+// this kernel only read them.
+__device__ inline void table_insert_body(const TableView& tv, const Work& wk, uint32_t now, uint32_t vblock, uint32_t vgrid) {
   __shared__ BlockAlloc sh;
-  __shared__ CheckIn entry;
-  check_in(wk, &entry);
-  const uint32_t n = entry.n_insert;
+  const uint32_t n = wk.call->n_insert;
+  if (vblock == 0 && threadIdx.x == 0) {
+    tv.st->sum_ids += wk.call->n_valid_ids;
+    tv.st->sum_unique += wk.call->n_unique;
+    tv.st->sum_new += n;
+  }
   const int lane = threadIdx.x & 31;
   const bool sketch = tv.sketch_depth != 0;
   unsigned int n_res = 0, n_done = 0;
@@ -458,11 +415,10 @@ __device__ inline void table_insert_body(const TableView& tv, const Work& wk, ui
       atomicAdd(&tv.st->n_inserted_total, (unsigned long long)n_done);
     }
   }
-  check_out(tv.st, wk, &entry, total_blocks);
 }
 __global__ void __launch_bounds__(256)
-table_insert_kernel(TableView tv, Work wk, uint32_t now, uint32_t total_blocks) { after_previous_kernel();
-  table_insert_body(tv, wk, now, total_blocks, blockIdx.x, gridDim.x);
+table_insert_kernel(TableView tv, Work wk, uint32_t now) { after_previous_kernel();
+  table_insert_body(tv, wk, now, blockIdx.x, gridDim.x);
 }
 
 // Every part of a long segment learns which ID it belongs to (one block per long ID, its threads

@@ -227,13 +227,12 @@ void join_sweep(mono_table* t) {
   t->keys_idle = false;
 }
 
-// Forget a prepared batch: empty the per-call set and the per-call counters.
+// Forget a prepared batch: empty the per-call set.  (The batch's counters start at the next grouping.)
 int discard_prepared(mono_table* t) {
   if (!t->prep.valid) return MONO_OK;
   t->prep.valid = false;
   if (t->prep.ordered) CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_aux, 0));
   init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(t->wk.bset, t->wk.n_slots());
-  forget_call_kernel<<<1, 32, 0, t->stream>>>(t->tv.st, t->wk);
   CUDA_TRY(t, cudaGetLastError());
   return MONO_OK;
 }
@@ -304,7 +303,6 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   w.error_bits = &t->tv.st->error_bits;
   init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(w.bset, slots);
   CUDA_TRY(t, cudaGetLastError());
-  CUDA_TRY(t, cudaMemsetAsync(w.win_count, 0, 2 * kWindows * sizeof(uint32_t), t->stream));
   CUDA_TRY(t, cudaMemsetAsync(w.part_done, 0, w.max_parts * sizeof(uint32_t), t->stream));
   CUDA_TRY(t, cudaMemsetAsync(w.call, 0, sizeof(CallState), t->stream));
   t->max_ids = max_ids;
@@ -465,6 +463,7 @@ int launch_order(mono_table* t) {
     CUDA_TRY(t, cudaEventRecord(t->ev_fork, s));
     CUDA_TRY(t, cudaStreamWaitEvent(a, t->ev_fork, 0));
   }
+  CUDA_TRY(t, cudaMemsetAsync(t->wk.win_count, 0, 2 * kWindows * sizeof(uint32_t), a));
   LAUNCH_ON(t, a, K_EXPAND, launch_after(expand_parts_kernel, grid_for(t, 8) * 4, 128, a, t->wk));
   LAUNCH_ON(t, a, K_ORDER, launch_after(order_parts_kernel, 64, kWindows, a, t->wk));
   CUDA_TRY(t, cudaGetLastError());
@@ -521,11 +520,10 @@ int launch_apply(mono_table* t, const unsigned long long* ids, int64_t n_ids, co
   // rows of new IDs were settled by the commit half, so nothing in the row updates waits for the
   // insertion, which runs beside them on the stream the sweep uses: a sweep that follows this call
   // follows the insertions.  With the probabilistic filter it is the insertion that decides the rows,
-  // and it stays on the table's stream.  Whichever kernel ends last closes the call.
+  // and it stays on the table's stream.
   const bool insert_aside = !t->timing && tv.sketch_depth == 0;
   const unsigned insert_blocks = insert_grid(t, n_ids);
   const RowGrid row_grid = rows_grid(t, n_ids);
-  const unsigned total = insert_blocks + blocks_of(row_grid);
   cudaStream_t k = insert_aside ? t->sweep_stream : s;
   if (insert_aside) {
     CUDA_TRY(t, cudaEventRecord(t->ev_commit, s));
@@ -533,7 +531,7 @@ int launch_apply(mono_table* t, const unsigned long long* ids, int64_t n_ids, co
   } else if (tv.sketch_depth) {
     LAUNCH(t, K_SKETCH, launch_after(sketch_add_kernel, insert_blocks, 256, s, tv, wk));
   }
-  LAUNCH_ON(t, k, K_INSERT, launch_after(table_insert_kernel, insert_blocks, 256, k, tv, wk, now, total));
+  LAUNCH_ON(t, k, K_INSERT, launch_after(table_insert_kernel, insert_blocks, 256, k, tv, wk, now));
   CUDA_TRY(t, cudaGetLastError());
   // the rest of the call touches rows and scratch only: a sweep may run beside it
   CUDA_TRY(t, cudaEventRecord(t->ev_keys, k));
@@ -541,7 +539,7 @@ int launch_apply(mono_table* t, const unsigned long long* ids, int64_t n_ids, co
   if (grad_ready) CUDA_TRY(t, cudaStreamWaitEvent(s, grad_ready, 0));
   rc = dispatch_dim(tv.dim, [&](auto g, auto nv) -> int {
     constexpr int G = decltype(g)::value, NV = decltype(nv)::value;
-    LAUNCH(t, K_ROWS, launch_after(update_rows_kernel<G, NV>, blocks_of(row_grid), kRowThreads, s, tv, wk, grad, n_bags, (int)ordered, row_grid, total));
+    LAUNCH(t, K_ROWS, launch_after(update_rows_kernel<G, NV>, blocks_of(row_grid), kRowThreads, s, tv, wk, grad, n_bags, (int)ordered, row_grid));
     return (int)MONO_OK;
   });
   CUDA_TRY(t, cudaGetLastError());
@@ -1036,10 +1034,8 @@ int mono_group_apply_grads(int32_t n_tables, mono_table* const* tables, const ui
     group_describe(p, i, tables[i], ids[i], n_ids[i], slot_offsets[i], n_bags[i], nullptr, grad_pooled[i], (uint32_t)now, all_prepared);
   for (int32_t i = 0; i < n_tables; ++i) all_ids += n_ids[i];
   // (half a table's share of the resident blocks: a block's preparations cost more here; 64 tables 63.3 -> 60.5 us, a quarter the same)
-  for (int32_t i = 0; i < n_tables; ++i) {
+  for (int32_t i = 0; i < n_tables; ++i)
     p.items[i].row_grid = rows_grid(tables[i], n_ids[i], 0.5 * (double)n_ids[i] / (double)(all_ids ? all_ids : 1));
-    p.items[i].total_blocks = insert_grid(tables[i], n_ids[i]) + blocks_of(p.items[i].row_grid);
-  }
   if ((rc = group_upload(p, tables)) != MONO_OK) return rc;
   if (all_prepared) {
     if (!all_filed) GROUP_LAUNCH(p, K_FILE, GK_FILE, 256, group_file_segments_kernel);

@@ -346,6 +346,75 @@ def test_an_entry_pushed_before_its_imported_time_expires_by_the_push(path, key_
     assert t.status()["error_bits"] == 0
 
 
+@pytest.mark.parametrize("grouped", [False, True])
+@pytest.mark.parametrize("dim, n_bags", [(16, 300), (512, 34000)])
+def test_counters_start_afresh_with_every_batch(dim, n_bags, grouped):
+    """Batches announced, grouped ahead and forgotten again, some with a malformed bag, between batches that are pushed: what
+    was counted for the forgotten ones (IDs, parts and their order, the malformed bag) is in no later one.  34 000
+    bags of 512 columns are beyond 64 MB, so their parts are put in order."""
+    kw = dict(init_scale=0.05, seed=6)
+    gpu, cpu = mb.MonoTable(1 << 12, dim, 2, 0, **kw), mo.OracleTable(1 << 12, dim, 2, 0, **kw)
+    rng = np.random.default_rng(dim)
+    h, known, sums = gpu.handle, set(), np.zeros(3, np.int64)
+
+    def batch(spoilt=False):
+        n = 3 * n_bags
+        hot = np.repeat(rng.permutation(50)[:3], (70, n // 8, n // 4))
+        ids = np.concatenate([hot, rng.integers(50, 3000, n - hot.size)])
+        ids = wl.splitmix64(rng.permutation(ids).astype(np.uint64))
+        off = np.append(np.arange(0, ids.size, 3), ids.size).astype(np.int64)
+        grad = (rng.standard_normal((off.size - 1, dim)) * 0.01).astype(f32)
+        if spoilt:
+            off[7] = off[6] - 2
+        return ids, off, grad, [torch.from_numpy(x).cuda() for x in (ids.view(np.int64), off, grad)]
+
+    def announce(b):
+        if grouped:
+            mb.mono_group_prepare_push([h], [b[3][0]], [b[3][1]])
+        else:
+            mb.mono_prepare_push(h, b[3][0], b[0].size, b[3][1], b[1].size - 1)
+
+    def ahead(b):
+        mb.mono_group_ahead(h, b[3][0], b[0].size, b[3][1], b[1].size - 1)
+
+    def push(b, now):
+        if grouped:
+            mb.mono_group_apply_grads([h], [b[3][0]], [b[3][1]], [b[3][2]], now)
+        else:
+            mb.mono_apply_grads(h, b[3][0], b[0].size, b[3][1], b[1].size - 1, b[3][2], now)
+        cpu.apply_grads(b[0], b[1], b[2], now)
+        distinct = set(b[0].tolist())
+        sums[:] += (b[0].size, len(distinct), len(distinct - known))
+        known.update(distinct)
+        st = gpu.status()
+        assert [st[k] for k in ("sum_ids", "sum_unique", "sum_new")] == sums.tolist(), now
+
+    for now in range(6):
+        good = batch()
+        if now == 1:
+            announce(batch())                                      # given up for another announcement
+            announce(good)
+        elif now == 2:
+            announce(batch())                                      # given up by a push
+        elif now == 3:
+            ahead(batch(spoilt=True))                              # never taken over
+            ahead(good)
+            announce(good)
+        elif now == 4:
+            announce(batch())
+            mb.mono_export_touched(h, None, None, 0)               # forgets it
+        elif now == 5:
+            announce(batch(spoilt=True))
+            assert gpu.status()["error_bits"] == mb.MONO_DEV_BAD_OFFSETS
+            mb.mono_clear_errors(h)
+        push(good, now)
+        assert gpu.status()["error_bits"] == 0, now
+    push(batch(), 6)
+    assert_state_equal(gpu, cpu)
+    assert_audit_ok(gpu)
+    assert gpu.status()["error_bits"] == 0
+
+
 @pytest.mark.parametrize("n_tables", [1, 2, 31, 32, 33, 65, 150])
 def test_grouped_calls_find_every_block_its_table(n_tables):
     """Numbers of tables around those that a warp searches at once; batches of very different size, every fifth empty.
