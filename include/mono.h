@@ -491,7 +491,8 @@ int mono_audit(mono_table* t, mono_audit_t* host_out);
 
 /*
  * Launch accounting for benchmarks (the paper has no counterpart).  Every
- * kernel the hot calls launch is counted per kernel.  With timing enabled,
+ * kernel the hot calls launch is counted per kernel (what prepares scratch that
+ * has just been allocated is not; a grouped call counts for its first table).  With timing enabled,
  * each launch is also bracketed by two CUDA events on the table's stream and
  * mono_timing_read (which synchronises) adds up the elapsed device time per
  * kernel; the events cost a few microseconds per launch, so leave timing off

@@ -31,13 +31,13 @@ using namespace mono;
 static __device__ __align__(256) uint32_t g_noalloc_occ_row[MONO_NOALLOC_MAX_IDS];
 
 enum KernelId {
-  K_POOL, K_FILL_BAG, K_DEDUP, K_LOOKUP, K_UPDATE, K_SKETCH, K_INSERT, K_EXPAND, K_ORDER, K_FILE, K_ROWS, K_EXPIRE, K_STASH_TRIM, K_COUNT
+  K_POOL, K_FILL_BAG, K_DEDUP, K_LOOKUP, K_UPDATE, K_SKETCH, K_INSERT, K_EXPAND, K_ORDER, K_FILE, K_ROWS, K_EXPIRE, K_STASH_TRIM, K_WIPE, K_UPLOAD, K_COUNT
 };
 // (gather_pool: either of the two pooling kernels; table_lookup and table_update are the two halves of table_update_kernel; a push that was not
-// announced runs both in one launch, counted as table_update)
+// announced runs both in one launch, counted as table_update; wipe_call_set: of a batch that was announced or grouped ahead and then forgotten)
 static const char* const kKernelNames[K_COUNT] = {
   "gather_pool", "fill_occ_bag", "dedup_tile", "table_lookup", "table_update", "sketch_add", "table_insert", "expand_parts", "order_parts", "file_segments",
-  "update_rows", "expire", "stash_trim"
+  "update_rows", "expire", "stash_trim", "wipe_call_set", "group_upload"
 };
 static_assert(K_COUNT <= MONO_MAX_KERNELS, "mono_timing_t has room for MONO_MAX_KERNELS kernels");
 
@@ -232,7 +232,7 @@ int discard_prepared(mono_table* t) {
   if (!t->prep.valid) return MONO_OK;
   t->prep.valid = false;
   if (t->prep.ordered) CUDA_TRY(t, cudaStreamWaitEvent(t->stream, t->ev_aux, 0));
-  init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(t->wk.bset, t->wk.n_slots());
+  LAUNCH(t, K_WIPE, init_bset_kernel<<<grid_for(t, 4), 256, 0, t->stream>>>(t->wk.bset, t->wk.n_slots()));
   CUDA_TRY(t, cudaGetLastError());
   return MONO_OK;
 }
@@ -698,6 +698,7 @@ int group_upload(GroupPlan& p, mono_table* const* tables) {
   std::memcpy(g.host[slot], p.items.data(), p.items.size() * sizeof(GroupItem));
   std::memcpy(g.host[slot] + items_bytes, p.starts.data(), p.starts.size() * sizeof(uint32_t));
   const uint32_t words = (uint32_t)(bytes / 16), room = (uint32_t)(std::min(g.dev_bytes, g.host_bytes[slot]) / 16);
+  ++p.owner->launches[K_UPLOAD];
   launch_after(group_upload_kernel, (words + 255) / 256, 256, p.gs, reinterpret_cast<uint4*>(g.dev), reinterpret_cast<const uint4*>(g.host[slot]), words, room,
                &p.owner->tv.st->error_bits);
   CUDA_TRY(p.owner, cudaGetLastError());
@@ -899,7 +900,7 @@ int mono_group_ahead(mono_table* t, const uint64_t* ids, int64_t n_ids, const in
   if (ah.valid) {
     // a batch grouped earlier that was never pushed: forget it
     ah.valid = false;
-    init_bset_kernel<<<grid_for(t, 4), 256, 0, g>>>(ah.bset, slots);
+    LAUNCH_ON(t, g, K_WIPE, init_bset_kernel<<<grid_for(t, 4), 256, 0, g>>>(ah.bset, slots));
     CUDA_TRY(t, cudaGetLastError());
     CUDA_TRY(t, cudaMemsetAsync(ah.call, 0, sizeof(CallState), g));
   }

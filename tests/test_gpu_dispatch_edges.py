@@ -451,6 +451,37 @@ def test_grouped_calls_find_every_block_its_table(n_tables):
         assert g.status()["error_bits"] == 0
 
 
+def test_every_launch_of_a_call_is_counted():
+    """A grouped step's, the uploads of its descriptors among them, for its first table; the wipes of batches that are
+    forgotten."""
+    n = 100
+    pair = [mb.MonoTable(256, dim, 1, 0, key_cells=1024, max_ids=n, max_bags=n) for dim in (8, 64)]
+    h = [t.handle for t in pair]
+    ids = [torch.arange(1 + k, n + 1 + k, device="cuda") for k in range(2)]
+    off = [torch.arange(n + 1, device="cuda")] * 2
+    out = [torch.empty((n, t.dim), device="cuda") for t in pair]
+
+    def counted(table):
+        got = mb.mono_timing_read(table, reset=True)
+        each = {k: v["launches"] for k, v in got["kernels"].items() if v["launches"]}
+        assert got["launches_total"] == sum(each.values())
+        return each
+
+    counted(h[0]), counted(h[1])
+    mb.mono_group_prepare_push(h, ids, off)
+    mb.mono_group_lookup_pool(h, ids, off, out)
+    mb.mono_group_apply_grads(h, ids, off, out, 1)
+    assert counted(h[1]) == {}
+    assert counted(h[0]) == {"group_upload": 3, **dict.fromkeys(("fill_occ_bag", "dedup_tile", "table_lookup", "gather_pool", "table_update", "table_insert", "update_rows"), 1)}
+    mb.mono_prepare_push(h[0], ids[0], n, off[0], n)
+    mb.mono_prepare_push(h[0], ids[1], n, off[1], n)
+    mb.mono_group_ahead(h[0], ids[0], n, off[0], n)
+    mb.mono_group_ahead(h[0], ids[1], n, off[1], n)
+    assert counted(h[0]) == {"wipe_call_set": 2, "fill_occ_bag": 4, "dedup_tile": 4, "table_lookup": 2}
+    for t in pair:
+        t.close()
+
+
 @pytest.mark.parametrize("repeated", [1, 255, 256, 4096, 4097])
 @pytest.mark.parametrize("dim", [4, 20, 64, 100, 132])
 @pytest.mark.parametrize("grouped", [False, True])
