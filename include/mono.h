@@ -163,8 +163,9 @@ typedef struct {
   uint64_t free_rows;
   uint64_t unaccounted_rows;    /* rows neither owned nor free */
   uint32_t ok;                  /* 1 iff all of the above are consistent with the counters */
-  uint32_t behind_records;      /* entries last seen before the time their bucket's sweep record holds
-                                   (saturating); the expiry sweep would not find them */
+  uint32_t behind_records;      /* entries last seen before the time their bucket's sweep record holds, which
+                                   the expiry sweep would not find, and entries whose row's time is before
+                                   the one in their cell, which is a lower bound of it (saturating) */
 } mono_audit_t;
 
 /*

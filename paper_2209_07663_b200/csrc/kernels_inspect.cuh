@@ -121,7 +121,7 @@ export_touched_kernel(TableView tv, unsigned long long n_cells, unsigned long lo
 
 struct AuditCounters {
   unsigned long long occupied, misplaced, duplicate_keys, resident_cells, bad_rows, shared_rows, free_rows,
-      unaccounted_rows, behind_records;
+      unaccounted_rows, behind_records;     // behind_records: entries behind their bucket's record, and rows behind their cell's time
 };
 
 // row_marks: one bit per row, zeroed by the caller.
@@ -155,6 +155,8 @@ audit_cells_kernel(TableView tv, unsigned long long n_cells, unsigned int* row_m
       ++n_res;
       const uint32_t row = meta_row(c.meta);
       if (row >= tv.capacity) { atomicAdd(&out->bad_rows, 1ull); continue; }
+      // (its time was not written when the ID got the row, or is another ID's: the export shows it, and the sweep will go by it)
+      if (meta_time(c.meta) > tv.seen[row]) atomicAdd(&out->behind_records, 1ull);
       const unsigned int bit = 1u << (row & 31);
       if (atomicOr(row_marks + (row >> 5), bit) & bit) atomicAdd(&out->shared_rows, 1ull);
     }
