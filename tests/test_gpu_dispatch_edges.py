@@ -451,6 +451,40 @@ def test_grouped_calls_find_every_block_its_table(n_tables):
         assert g.status()["error_bits"] == 0
 
 
+@pytest.mark.parametrize("dim", [260, 512, 516, 1024])
+@pytest.mark.parametrize("announced", [False, True])
+def test_grouped_calls_of_the_widest_rows(dim, announced):
+    """Rows of more than 256 columns beside narrow ones in one group: segments of 1 to 66 occurrences and long ones, whose
+    parts go up one level of the tree and two; long bags and empty ones; pooled to an output aligned to 32 bytes and to 16."""
+    pair, batch = [], []
+    for k, d in enumerate((dim, 16, dim)):
+        kw = dict(init_scale=0.05, seed=k)
+        pair.append((mb.MonoTable(512, d, 2, 0, key_cells=2048, **kw), mo.OracleTable(512, d, 2, 0, **kw)))
+        rng = np.random.default_rng(dim + k)
+        times = np.concatenate([np.arange(1, 67), [200, 1500], np.ones(60, np.int64)])
+        ids = rng.permutation(np.repeat(wl.splitmix64(np.arange(1, times.size + 1, dtype=np.uint64)), times))
+        off = np.sort(np.concatenate([[0, ids.size], rng.integers(0, ids.size, 400)])).astype(np.int64)
+        grad = (rng.standard_normal((off.size - 1, d)) * 0.01).astype(f32)
+        batch.append((ids, off, grad))
+    h = [g.handle for g, _ in pair]
+    ids, off, grad = ([torch.from_numpy(b[k].view(np.int64) if k == 0 else b[k]).cuda() for b in batch] for k in range(3))
+    for now in range(3):
+        stores = [torch.full((b[2].size + 8,), float("nan"), device="cuda") for b in batch]
+        out = [s[4 * (now % 2):][:b[2].size].view(b[2].shape) for s, b in zip(stores, batch)]
+        if announced:
+            mb.mono_group_prepare_push(h, ids, off)
+        mb.mono_group_lookup_pool(h, ids, off, out)
+        for (_, cpu), b, o in zip(pair, batch, out):
+            assert_vectors_close(o.cpu().numpy(), cpu.lookup_pool(b[0], b[1]), f"step {now}")
+        mb.mono_group_apply_grads(h, ids, off, grad, now)
+        for (_, cpu), b in zip(pair, batch):
+            cpu.apply_grads(*b, now)
+    for gpu, cpu in pair:
+        assert_state_equal(gpu, cpu)
+        assert_audit_ok(gpu)
+        assert gpu.status()["error_bits"] == 0
+
+
 def test_every_launch_of_a_call_is_counted():
     """A grouped step's, the uploads of its descriptors among them, for its first table; the wipes of batches that are
     forgotten."""
