@@ -181,7 +181,8 @@ typedef struct {
  *  cuda_stream       a cudaStream_t (NULL = the default stream) on the current device
  * Allocates capacity * dim * 8 bytes of rows+accumulators, key_cells * 16 bytes
  * of keys, key_cells bytes of sweep records (below, mono_expire), capacity * 4
- * bytes of free-row bookkeeping and the scratch.
+ * bytes of free-row bookkeeping, capacity * 4 bytes of the rows' last-access
+ * times and the scratch.
  */
 int mono_table_create(mono_table** out, uint64_t capacity, uint32_t dim,
                       uint32_t filter_threshold, uint32_t ttl, const mono_opt* opt,
@@ -401,7 +402,7 @@ int mono_fence(mono_table* t);
  * Device-resident snapshot (Section 2.3: the parameter servers snapshot their state so that
  * training can go back to it; here the copy stays in device memory, for callers that want to
  * return to a state quickly -- benchmarks that repeat a timed region from the same state,
- * what-if runs).  mono_snapshot_save copies the key store, the rows and accumulators, the
+ * what-if runs).  mono_snapshot_save copies the key store, the rows, accumulators and rows' times, the
  * free-row list, the counters and the sketch into a second set of buffers owned by the table
  * (allocated on the first save: as much memory again as the table itself; MONO_ERR_NOMEM if
  * that does not fit) and remembers the table's clock.  mono_snapshot_restore copies them back

@@ -266,7 +266,8 @@ table_update_kernel(TableView tv, Work wk, uint32_t now) { after_previous_kernel
 // An entry whose metadata is `meta` has just been written into a cell of bucket `bkt`: the
 // bucket's record of its oldest stamp may not stay above that entry's.  (Entries that leave a
 // bucket, and stamps that are renewed, leave the record as it is: it only has to be a lower
-// bound, and the sweep makes it exact again whenever it visits the bucket.  A stamp that a push takes
+// bound, and the sweep sets it to the oldest of its cells' times, bounds themselves for IDs that own rows, whenever
+// it visits the bucket.  A stamp that a push takes
 // back, of an entry imported at a later time, lowers it: table_update_body.)  `rec` is the
 // record as read before the write; records only fall while entries are being inserted, so a
 // value read earlier is at or above the present one and the test errs on the safe side.
@@ -483,8 +484,9 @@ order_parts_kernel(Work wk) { after_previous_kernel(); order_parts_body(wk, bloc
 // The sweep reads, per bucket, the record of its oldest stamp (4 bytes, in order) and opens only
 // the buckets in which that stamp is past the expire time: an entry that has to go has a stamp at
 // or above its bucket's record, so its bucket is always opened, and the outcome is that of a sweep
-// over every cell.  A bucket that is opened gets an exact record again.  Nothing else touches the
-// key store while this runs.
+// over every cell.  A bucket that is opened gets a tighter record: the oldest time in the cells that stay, which of an ID
+// that owns a row is the row's if the cell's was past the ttl and else a bound of it.  Nothing else touches the key store
+// or the rows' times while this runs.
 // A block lists the buckets to open in shared memory, round by round until there are enough to fill it, then takes them one
 // cell per thread, so that all their loads are in flight together and the four lanes of a bucket read its 64 bytes as one.
 // The rows it frees are listed too and go on the free stack together: the top of the stack is one word that all blocks
