@@ -307,6 +307,7 @@ int reserve(mono_table* t, int64_t max_ids, int64_t max_bags) {
   CUDA_TRY(t, cudaGetLastError());
   CUDA_TRY(t, cudaMemsetAsync(w.part_done, 0, w.max_parts * sizeof(uint32_t), t->stream));
   CUDA_TRY(t, cudaMemsetAsync(w.call, 0, sizeof(CallState), t->stream));
+  CUDA_TRY(t, cudaMemsetAsync(w.win_count, 0, 2 * kWindows * sizeof(uint32_t), t->stream));
   t->max_ids = max_ids;
   t->max_bags = max_bags;
   return MONO_OK;
@@ -465,10 +466,11 @@ int launch_order(mono_table* t) {
     CUDA_TRY(t, cudaEventRecord(t->ev_fork, s));
     CUDA_TRY(t, cudaStreamWaitEvent(a, t->ev_fork, 0));
   }
-  CUDA_TRY(t, cudaMemsetAsync(t->wk.win_count, 0, 2 * kWindows * sizeof(uint32_t), a));
   LAUNCH_ON(t, a, K_EXPAND, launch_after(expand_parts_kernel, grid_for(t, 8) * 4, 128, a, t->wk));
   LAUNCH_ON(t, a, K_ORDER, launch_after(order_parts_kernel, 64, kWindows, a, t->wk));
   CUDA_TRY(t, cudaGetLastError());
+  // (for the next batch: in front of the two it let the pull's blocks be queued before theirs, 4 M drifting IDs at key load 0.9 407 -> 413 us)
+  CUDA_TRY(t, cudaMemsetAsync(t->wk.win_count, 0, 2 * kWindows * sizeof(uint32_t), a));
   CUDA_TRY(t, cudaEventRecord(t->ev_aux, a));
   return MONO_OK;
 }
